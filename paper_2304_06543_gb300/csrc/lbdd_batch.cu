@@ -467,6 +467,13 @@ int batch_wait(lbdd_batch* b, int* first_rc) {
   return LBDD_OK;
 }
 
+// Lets go of the pass's solvers: their owner may destroy them from now on.
+// The pass's results (batch_rounds, batch_status) stay readable by index.
+void batch_detach(lbdd_batch* b) {
+  for (lbdd_solver* x : b->solvers) x->in_batches--;
+  b->solvers.clear();
+}
+
 int batch_launches(const lbdd_batch* b) { return 2 + (int)b->groups.size(); }
 int64_t batch_rounds(const lbdd_batch* b, int i) { return b->h_out[2 * b->slot_of[i] + 1]; }
 int64_t batch_status(const lbdd_batch* b, int i) { return b->h_out[2 * b->slot_of[i]]; }

@@ -46,6 +46,7 @@ int batch_set(lbdd_batch* b, lbdd_solver* const* solvers, const int64_t* rem, in
               int cluster_size, int max_clusters, bool shortest_first, const uint8_t* first);
 int batch_launch(lbdd_batch* b, int64_t max_rounds);
 int batch_wait(lbdd_batch* b, int* first_rc);
+void batch_detach(lbdd_batch* b);
 int batch_launches(const lbdd_batch* b);
 int64_t batch_rounds(const lbdd_batch* b, int i);
 int64_t batch_status(const lbdd_batch* b, int i);
@@ -244,6 +245,9 @@ static void engine_loop(lbdd_server* S) {
     if (!rc) rc = batch_launch(S->batch, -1);
     int first = LBDD_OK;
     if (!rc) rc = batch_wait(S->batch, &first);
+    // finished solvers are destroyed by the retirement thread: the batch must
+    // not reach for them in the next pass
+    batch_detach(S->batch);
     const int64_t t_b = now_ns(S->t0);
     lk.lock();
     S->passes++;
