@@ -1,0 +1,1001 @@
+// One-CTA ASRAL solver with price-guided searches (included by
+// asral_solver.cu, which holds the shared prologue).
+//
+// Same rounds, same results as Solver<T> (Alg. 2 with Alg. 1 and Alg. 4 per
+// round); what differs is how much of the Bellman-Ford of Alg. 3 is run.
+//
+// Prices.  Every center v keeps a price P(v), a lower bound on the cost of
+// getting one unit out of v: over every path v -> ... -> u of Gamma, the
+// transfer costs plus q_n(u), the penalty one more unit would pay at u (0
+// with a vacancy).  The bounds are the feasible potentials of the successive
+// shortest path method for min-cost flow (Edmonds and Karp 1972; Tomizawa
+// 1971): for every table entry P(u) <= T[u][v] + P(v), and P(v) <= q_n(v).
+// All prices start at 0 with an empty table.  When unit d joins center j:
+//
+//  * Only d's own edges can break the first inequality, so the merge of d's
+//    row into T[j] also tests P(j) <= t_d(v) + P(v).  If it holds, no
+//    negative cycle passes through j (Alg. 1 applies nothing); if also
+//    P(j) >= q_j(last), the penalty j's last unit pays, no negative path
+//    starts at j (Alg. 4 applies nothing), and the round ends there.
+//  * Otherwise one synchronous Bellman-Ford from j answers both: a label
+//    l(v) is expanded only while l(v) + P(v) does not exceed the best value
+//    found so far (P(j) + cycle cost for Alg. 1; min l(u) + q_n(u) for
+//    Alg. 4).  Every node of every shortest path to the sink passes that
+//    test, because l(v) + P(v) bounds the value of any completion from v, so
+//    the sink's label, hop counts and lowest-index parents are those of the
+//    full Bellman-Ford, and the path applied is the same.
+//  * After a cycle was applied, Alg. 4 searches again; the bound uses the
+//    prices raised by the first search's labels, max(P(v), P(j) + L - l1(v))
+//    (L the cycle's cost), less `off`, the most by which those exceed q_n.
+//  * The round ends by raising prices: P(v) = max(P(v), D - l1(v), D2 -
+//    l2(v)), D the shortest way from d to a paid slot (L + D2 after a
+//    cycle, D2 from j).  For a row of T that did not change this keeps both
+//    inequalities by l(v) <= l(u) + T[u][v]; the rows that did change are
+//    tested entry by entry (verify).  Should one ever fail, the prices are
+//    rebuilt from the table by reverse Bellman-Ford sweeps before the next
+//    round, so the pruning never rests on an untested bound.
+//
+// What this buys (counted on instances of the city shape, 8,000 x 500, and of
+// the batched mix, 6,007 x 126): 48 sweeps of 180 labels and 19 sweeps of 52
+// per round become 22 sweeps of 12 labels and 8 of 12; half of the mix's
+// rounds run no sweep at all.
+//
+// Layout.  A frontier of a dozen labels is too little work to spread over a
+// cluster: one CTA runs the whole round.  Thread t owns columns t, t + 512,
+// ...; every thread reads the whole frontier list (broadcast loads) and keeps
+// its own column's minimum, so a sweep needs one barrier of the ceil(k / 32)
+// warps that own a column and no cross-warp reduction.  Labels that improved
+// are appended to the next list by one shared-memory atomic per warp (order
+// inside a list does not matter: equal labels take the lower node).  The
+// costs of T sit in shared memory as T (int16 or int32) when they fit beside
+// the rest, otherwise they are read from the global table through L1.
+#pragma once
+
+namespace lbdd {
+
+// Bits of a node in a packed (hop, node) key (k <= 8191).
+constexpr int kGNodeBits = 13;
+constexpr int kGOrd = 64;                       // prefetched (unit, center) pairs
+constexpr int kGAff = 1024;                     // affected entries per rescan chunk, at least
+
+struct GLayout {
+  uint32_t pot, lab1, lab2, hop, list, slack, pen, qn, seg, tailp, path, pathu, mid, raff, cpath, aff,
+      ord, misc, ring, base_total, tsm, total;
+  int nring;
+};
+
+// Rows of CM in flight: 8 where they are short, 4 otherwise (they cover the
+// DRAM latency of about four rounds that run no search).
+__host__ __device__ inline int guided_ring(int32_t k, int32_t elem) {
+  return (int64_t)k * elem <= 3072 ? 8 : 4;
+}
+
+// Row stride of the cost table in entries (an odd number of words with int16
+// costs, so that the rows of one column spread over the banks).
+__host__ __device__ inline int32_t guided_stride(int32_t k, int32_t elem) {
+  return slice_stride((k + 1) & ~1, elem);
+}
+
+__host__ __device__ inline GLayout make_guided_layout(int32_t k, int32_t elem) {
+  GLayout L;
+  uint32_t o = 0;
+  const uint32_t ku = (uint32_t)k, lt = elem == 2 ? 4u : 8u;
+  auto take = [&](uint32_t bytes) { const uint32_t at = o; o = align16(o + bytes); return at; };
+  L.pot = take(4u * ku);
+  L.lab1 = take(lt * ku);
+  L.lab2 = take(lt * ku);
+  L.hop = take(2u * ku);
+  const uint32_t aff = ku > (uint32_t)kGAff ? ku : (uint32_t)kGAff;
+  const uint32_t lists = 2u * 2u * lt * (ku + 2);
+  L.list = take(lists > 8u * aff ? lists : 8u * aff);   // also the minima of a rescan
+  L.slack = take(4u * ku);
+  L.pen = take(4u * ku);
+  L.qn = take(4u * ku);
+  L.seg = take(4u * ku);
+  L.tailp = take(4u * ku);
+  L.path = take(4u * (ku + 2));
+  L.pathu = take(4u * (ku + 2));
+  L.mid = take(4u * (ku + 2));
+  L.raff = take(4u * (ku + 2));
+  L.cpath = take(4u * (ku + 2));
+  L.aff = take(4u * aff);
+  L.ord = take(8u * kGOrd);
+  L.misc = take(128u);
+  L.nring = guided_ring(k, elem);
+  // the prologue's radix sort uses the ring and what follows (17 KB)
+  const uint32_t row = align16((uint32_t)elem * ku);
+  const uint32_t ringb = (uint32_t)L.nring * row;
+  L.ring = take(ringb > 18432u ? ringb : 18432u);
+  L.base_total = o;
+  L.tsm = take((uint32_t)elem * ku * (uint32_t)guided_stride(k, elem));
+  L.total = o;
+  return L;
+}
+
+// Frontier entry: label and byte offset of the node's row of costs.
+template <typename LT> struct GEnt;
+template <> struct __align__(8) GEnt<int32_t> { int32_t l; uint32_t off; };
+template <> struct __align__(16) GEnt<int64_t> { int64_t l; uint32_t off, pad; };
+
+// Penalties and prices stay below this in a guided solve (the host checks the
+// penalties), so that a label plus either fits 32 bits with int16 costs.
+constexpr int32_t kGPenLimit = 1 << 30;
+constexpr int32_t kGNever = kGPenLimit + (1 << 29);   // a price or slot out of every bound
+
+struct GMisc {
+  int32_t paid;       // best value of a path to a paid slot in the last search
+  uint32_t sink;      // its hop count << kGNodeBits | node, if paid < ql
+  uint32_t next[3];   // parents on the way back, by hop count modulo 3
+  int32_t cnt[3];     // list lengths, by sweep modulo 3
+  int32_t naff, len, bad, stop;
+};
+
+template <typename T, bool TSM>
+struct Guided {
+  using LT = typename Solver<T>::LT;
+  using Ent = GEnt<LT>;
+  static constexpr int VPL = 16 / (int)sizeof(T);
+  static constexpr int32_t kInf = Solver<T>::kTsInf;
+  static constexpr LT kNoLab = Solver<T>::kNoLab;
+
+  const DevInst& I;
+  const T* cm;
+  int64_t ld;
+  int32_t *tc, *td, *pool, *page_tab, *pos;
+  int32_t max_pages;
+  int32_t n, k, ws;
+  int tid, flags;
+  int32_t *s_pot, *s_slack, *s_pen, *s_seg, *s_tail, *s_path, *s_pathu, *s_raff, *s_cpath,
+      *s_aff, *s_ord;
+  int32_t* s_qn;      // q_n of every center: what one more unit would pay there
+  int32_t* s_mid;     // prices of a second search; positions while units move
+  LT *s_lab1, *s_lab2;
+  uint16_t* s_hop;    // sweep of every label's last change in the last search
+  Ent* s_list;        // [2][k + 2]
+  GMisc* M;
+  unsigned char* s_ring;
+  uint32_t ring_row;
+  int nring;
+  T* tt;              // [k][ws] costs of T: shared memory, or the global mirror
+  Book* B;
+
+  __device__ Guided(const DevInst& inst, unsigned char* base, const GLayout& L, Book* book, int fl)
+      : I(inst) {
+    cm = static_cast<const T*>(inst.cm);
+    ld = inst.ld;
+    tc = inst.tc;
+    td = inst.td;
+    pool = inst.pool;
+    page_tab = inst.page_tab;
+    pos = inst.pos;
+    max_pages = inst.max_pages;
+    n = inst.n;
+    k = inst.k;
+    ws = guided_stride(k, (int32_t)sizeof(T));
+    tid = threadIdx.x;
+    flags = fl;
+    auto i32 = [&](uint32_t at) { return reinterpret_cast<int32_t*>(base + at); };
+    s_pot = i32(L.pot);
+    s_lab1 = reinterpret_cast<LT*>(base + L.lab1);
+    s_lab2 = reinterpret_cast<LT*>(base + L.lab2);
+    s_hop = reinterpret_cast<uint16_t*>(base + L.hop);
+    s_list = reinterpret_cast<Ent*>(base + L.list);
+    s_slack = i32(L.slack);
+    s_pen = i32(L.pen);
+    s_seg = i32(L.seg);
+    s_tail = i32(L.tailp);
+    s_path = i32(L.path);
+    s_pathu = i32(L.pathu);
+    s_mid = i32(L.mid);
+    s_qn = i32(L.qn);
+    s_raff = i32(L.raff);
+    s_cpath = i32(L.cpath);
+    s_aff = i32(L.aff);
+    s_ord = i32(L.ord);
+    M = reinterpret_cast<GMisc*>(base + L.misc);
+    s_ring = base + L.ring;
+    ring_row = align16((uint32_t)sizeof(T) * (uint32_t)k);
+    nring = L.nring;
+    tt = TSM ? reinterpret_cast<T*>(base + L.tsm) : static_cast<T*>(inst.mirror);
+    B = book;
+  }
+
+  __device__ __forceinline__ bool timer() const { return (flags & OPT_PHASE_TIMERS) && tid == 0; }
+  __device__ __forceinline__ const T* row(int32_t d) const { return cm + (int64_t)d * ld; }
+  __device__ __forceinline__ int32_t edge(int32_t u, int cl) const {
+    return (int32_t)tt[(int64_t)u * ws + cl];
+  }
+  __device__ __forceinline__ void set_entry(int32_t u, int cl, int32_t t, int32_t d) {
+    tc[(int64_t)u * k + cl] = t;
+    td[(int64_t)u * k + cl] = d;
+    tt[(int64_t)u * ws + cl] = (T)(t == kTInf ? kInf : t);
+  }
+  // q_c(x), x >= 1: penalty of the x-th allotment beyond capacity (Def. 4).
+  __device__ __forceinline__ int32_t qval(int32_t c, int32_t x) const {
+    return __ldg(I.pen + (int64_t)c * I.Q + min(max(x, 1), I.Q) - 1);
+  }
+  // One unit more (+1) or less (-1) at c.
+  __device__ __forceinline__ void shift_load(int32_t c, int32_t by) {
+    const int32_t x = s_slack[c] + by;
+    s_slack[c] = x;
+    if (I.Q > 1) s_pen[c] = qval(c, x + 1);
+    s_qn[c] = x >= 0 ? s_pen[c] : 0;
+  }
+
+  // ------------------------------------------------------- member lists --
+  // Page of entry idx of c's list; the last page's id is kept in shared memory.
+  __device__ __forceinline__ int32_t page_of(int32_t c, int32_t idx, int32_t len) const {
+    const int32_t p = idx >> kPageShift;
+    return p == (len - 1) >> kPageShift ? s_tail[c] : page_tab[(int64_t)c * max_pages + p];
+  }
+  __device__ __forceinline__ int32_t* mslot(int32_t c, int32_t idx, int32_t len) const {
+    return pool + (int64_t)page_of(c, idx, len) * kPageWords + (idx & (kPage - 1));
+  }
+  // One thread at a time calls these two.  `own` is CM(d, c).
+  __device__ void list_append(int32_t c, int32_t d, int32_t own) {
+    const int32_t idx = s_seg[c];
+    if (idx < 0 || idx >= n) { B->err0 = ST_ERR_INVARIANT; return; }
+    if ((idx & (kPage - 1)) == 0) {
+      if (B->free_top <= 0) { B->err0 = ST_ERR_INVARIANT; return; }
+      const int32_t page = I.free_stack[--B->free_top];
+      page_tab[(int64_t)c * max_pages + (idx >> kPageShift)] = page;
+      s_tail[c] = page;
+    }
+    int32_t* slot = pool + (int64_t)s_tail[c] * kPageWords + (idx & (kPage - 1));
+    slot[0] = d;
+    slot[kPage] = own;
+    pos[d] = idx;
+    s_seg[c] = idx + 1;
+  }
+  __device__ void list_remove_at(int32_t c, int32_t idx) {
+    const int32_t len = s_seg[c], last = len - 1;
+    if (idx < 0 || idx > last || B->free_top >= I.npages) { B->err0 = ST_ERR_INVARIANT; return; }
+    if (idx != last) {
+      const int32_t* from = mslot(c, last, len);
+      int32_t* to = mslot(c, idx, len);
+      const int32_t moved = from[0], own = from[kPage];
+      to[0] = moved;
+      to[kPage] = own;
+      pos[moved] = idx;
+    }
+    if ((last & (kPage - 1)) == 0) {
+      I.free_stack[B->free_top++] = s_tail[c];
+      if (last > 0) s_tail[c] = page_tab[(int64_t)c * max_pages + ((last - 1) >> kPageShift)];
+    }
+    s_seg[c] = last;
+  }
+
+  // ------------------------------------------------------------- search --
+  __device__ __forceinline__ void group_sync(int nthr) const {
+    if (nthr == 32) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+  }
+  static __device__ __forceinline__ int32_t clamp32(int64_t x) {
+    return (int32_t)max((int64_t)INT32_MIN, min((int64_t)INT32_MAX, x));
+  }
+  static __device__ __forceinline__ LT relax(LT l, int32_t t, LT b) {
+    if constexpr (sizeof(LT) == 4) return __viaddmin_s32(l, t, b);
+    else return min(b, l + (LT)t);
+  }
+  // The cost at byte offset `at` of the table, in shared memory or in the mirror.
+  __device__ __forceinline__ int32_t cost_at(uint32_t at) const {
+    int32_t t;
+    if constexpr (TSM) {
+      if constexpr (sizeof(T) == 2)
+        asm volatile("ld.shared.s16 %0, [%1];" : "=r"(t) : "r"(at) : "memory");
+      else
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(t) : "r"(at) : "memory");
+    } else {
+      t = (int32_t)*reinterpret_cast<const T*>(reinterpret_cast<const unsigned char*>(tt) + at);
+    }
+    return t;
+  }
+  static __device__ __forceinline__ Ent entry(uint32_t at) {
+    Ent e;
+    if constexpr (sizeof(LT) == 4) {
+      asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(e.l), "=r"(e.off) : "r"(at) : "memory");
+    } else {
+      uint32_t lo, hi;
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(lo), "=r"(hi), "=r"(e.off), "=r"(e.pad) : "r"(at) : "memory");
+      e.l = (int64_t)(((uint64_t)hi << 32) | lo);
+    }
+    return e;
+  }
+  // Pruned synchronous Bellman-Ford from j into `lab` and s_hop.  cyc: look
+  // for a cycle through j (lab[j] holds its value); np: for a path to a paid
+  // slot cheaper than ql (M->paid its value, M->sink its last node).  `price`
+  // holds the bounds.  Every thread calls it.
+  //
+  // A sweep is a dependent chain of a few warps, so its cost is the number of
+  // instructions on that chain (about five cycles each for a lone warp), not
+  // its bytes.  It keeps only the least label per column: which predecessor
+  // gave it is looked up for the few nodes of the path that is applied
+  // (follow), by label and hop count; an edge costs one load and one
+  // add-and-minimum.  A lane owns one column, in registers up to 512 centers.
+  // The infinite entry of a frontier node's row (its own column) never beats
+  // the node's own label; nodes without members are never on the list.
+  __device__ void search(int32_t j, bool cyc, bool np, LT* lab, const int32_t* price, int32_t ql) {
+    constexpr LT kFixed = std::numeric_limits<LT>::min();   // a label nothing improves
+    const int32_t pj = s_pot[j];
+    const uint32_t tbase = TSM ? smem_u32(tt) : 0u;
+    const uint32_t rowb = (uint32_t)ws * (uint32_t)sizeof(T);
+    const uint32_t lbase = smem_u32(s_list), lsize = (uint32_t)(k + 2) * (uint32_t)sizeof(Ent);
+    for (int cl = tid; cl < k; cl += kThreads) lab[cl] = cyc || cl != j ? kNoLab : kFixed;
+    if (tid == 0) {
+      M->paid = INT32_MAX;
+      M->sink = ~0u;
+      M->next[0] = M->next[1] = M->next[2] = ~0u;
+      M->cnt[1] = 0;
+      Ent e;
+      e.l = 0;
+      e.off = tbase + (uint32_t)j * rowb;
+      s_list[0] = e;
+    }
+    __syncthreads();
+    const int nthr = min(kThreads, (k + 31) & ~31);
+    if (tid < nthr) {
+      // frontier nodes in flight: shared memory or L2 latency
+      constexpr int U = TSM ? 8 : 16;
+      const int lane = tid & 31;
+      const bool single = k <= nthr;
+      int sweep = 1, m = 1, par = 0, c3 = 1;   // par: list read; c3: counter of the next list
+      LT b = kFixed;
+      int32_t qv = kGNever, pv = kGNever;
+      for (;; ++sweep) {
+        const uint32_t in = lbase + (uint32_t)par * lsize;
+        Ent* out = s_list + (par ^ 1) * (k + 2);
+        const int c3n = c3 == 2 ? 0 : c3 + 1;
+        if (tid == 0) {
+          M->cnt[c3n] = 0;
+          if (timer()) front_stat(m);
+        }
+        const LT bc = cyc ? (LT)pj + min((LT)-1, lab[j]) : kFixed;
+        const int32_t paid = M->paid;
+        const int32_t bp = np ? min(ql - 1, paid) : INT32_MIN;
+        unsigned bits = 0;
+        for (int cl = tid, c0 = 0; c0 < k; c0 += nthr, cl += nthr) {
+          if (!single || sweep == 1) {
+            const bool real = cl < k && cl != j;
+            b = cl < k ? lab[cl] : kFixed;
+            qv = real ? s_qn[cl] : kGNever;
+            // a center without members has no edges (its row is infinite)
+            pv = real && s_seg[cl] > 0 ? price[cl] : kGNever;
+          }
+          const LT old = b;
+          const uint32_t colb = (uint32_t)min(cl, k - 1) * (uint32_t)sizeof(T);
+          LT b2 = b;
+          for (int f = 0; f < m; f += U) {
+            Ent e[U];
+            int32_t t[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q)   // past the end: the last node again
+              e[q] = entry(in + (uint32_t)min(f + q, m - 1) * (uint32_t)sizeof(Ent));
+#pragma unroll
+            for (int q = 0; q < U; ++q) t[q] = cost_at(e[q].off + colb);
+#pragma unroll
+            for (int q = 0; q < U; q += 2) {
+              b = relax(e[q].l, t[q], b);
+              b2 = relax(e[q + 1].l, t[q + 1], b2);
+            }
+          }
+          b = min(b, b2);
+          const bool up = b < old;
+          if (up) {
+            lab[cl] = b;
+            s_hop[cl] = (uint16_t)sweep;
+          }
+          int32_t now = bp;
+          if (np) {
+            const int32_t vm = __reduce_min_sync(0xffffffffu, up ? clamp_sum(b, qv) : INT32_MAX);
+            if (vm < paid && lane == 0) atomicMin(&M->paid, vm);
+            now = min(bp, vm);
+          }
+          const LT key = b + (LT)pv;
+          const bool push = up && (key <= (LT)now || key <= bc);
+          if (nthr == 32) bits = __ballot_sync(0xffffffffu, push);
+          if (push) {
+            const int at = nthr == 32 ? __popc(bits & ((1u << lane) - 1u)) : atomicAdd(&M->cnt[c3], 1);
+            Ent ne;
+            ne.l = b;
+            ne.off = tbase + (uint32_t)cl * rowb;
+            out[at] = ne;
+          }
+        }
+        group_sync(nthr);
+        m = nthr == 32 ? __popc(bits) : M->cnt[c3];
+        c3 = c3n;
+        par ^= 1;
+        if (m == 0) break;
+        if (sweep > k + 1) {   // labels settle within k + 1 sweeps
+          if (tid == 0) M->bad = 1;
+          break;
+        }
+      }
+      if (np && M->paid < ql) {   // fewest hops, then lowest node, among the best slots
+        const int32_t best = M->paid;
+        uint32_t hu = ~0u;
+        for (int cl = tid; cl < k; cl += nthr)
+          if (cl != j && lab[cl] != kNoLab && (int64_t)lab[cl] + s_qn[cl] == best)
+            hu = min(hu, ((uint32_t)s_hop[cl] << kGNodeBits) | (uint32_t)cl);
+        hu = __reduce_min_sync(0xffffffffu, hu);
+        if (lane == 0 && hu != ~0u) atomicMin(&M->sink, hu);
+      }
+      if (tid == 0) {
+        B->bf_calls++;
+        B->bf_sweeps += sweep;
+        B->bf_max = max(B->bf_max, (int64_t)sweep);
+      }
+    }
+    __syncthreads();
+  }
+  static __device__ __forceinline__ int32_t clamp_sum(LT a, int32_t b) {
+    if constexpr (sizeof(LT) == 4) return a + b;
+    else return clamp32(a + b);
+  }
+
+  __device__ __forceinline__ void front_stat(int m) {
+    B->front_sum += m;
+    B->front_hist[m <= 1 ? 0 : m <= 4 ? 1 : m <= 16 ? 2 : m <= 64 ? 3 : m <= 256 ? 4 : 5]++;
+  }
+
+  // -------------------------------------------------------------- apply --
+  // The canonical shortest path that ends at node `last` (the cycle through
+  // j if last < 0), backwards into s_pathu: the parent of a node v with label
+  // l and hop count h is the lowest-index u with l(u) + T[u][v] = l and
+  // hop(u) = h - 1.  Thread = node, one barrier per hop.  Returns its length,
+  // -1 if there is none.
+  __device__ int follow(int32_t j, int32_t last, const LT* lab) {
+    int32_t v = last < 0 ? j : last;
+    int h = s_hop[v], m = 0;
+    LT l = lab[v];
+    if (last >= 0) {
+      if (tid == 0) s_pathu[0] = v;
+      m = 1;
+    }
+    for (; h > 1; --h) {
+      uint32_t* slot = &M->next[h % 3];
+      for (int u = tid; u < k; u += kThreads)
+        if (s_hop[u] == h - 1 && u != j && u != v && lab[u] != kNoLab &&
+            lab[u] + (LT)edge(u, v) == l) {
+          atomicMin(slot, (uint32_t)u);
+          break;
+        }
+      __syncthreads();
+      const uint32_t best = *slot;
+      if (tid == 0) M->next[(h + 1) % 3] = ~0u;   // read before the last barrier
+      if (best == ~0u) return -1;
+      v = (int32_t)best;
+      l = lab[v];
+      if (tid == 0) s_pathu[m] = v;
+      ++m;
+    }
+    if (l != (LT)edge(j, v)) return -1;
+    if (tid == 0) s_pathu[m] = j;
+    return m + 1 < 2 ? -1 : m + 1;
+  }
+
+  // Follows the parents from `last` to j and applies the transfers of that
+  // path (Alg. 1 and Alg. 4, "if cost < 0" branch): every center on it hands
+  // its best unit for the next center on; for a cycle the last one hands to
+  // j, for a path the last center only gains and j only loses a unit.  Then
+  // the rows of T of those centers.  Warp 0 moves the units while the other
+  // warps already take the arriving units into the rows (that needs no member
+  // list); what is left per call is a chain of four global latencies: the
+  // moved units, their rows, member ids, member costs.  Returns the length of
+  // the path (s_path), -1 if the walk is bad.
+  __device__ int apply(int32_t j, bool npath, int32_t last, const LT* lab, int64_t cost) {
+    const uint64_t t0 = timer() ? clock_cycles() : 0;
+    const int lane = tid & 31;
+    const int m = follow(j, last, lab);
+    if (m < 0) return m;
+    if (tid < 32) {
+      __syncwarp();
+      if (lane == 0) M->naff = 0;
+      for (int i = lane; i < m; i += 32) s_path[i] = s_pathu[m - 1 - i];
+      __syncwarp();
+      for (int i = lane; i < m; i += 32) {
+        const int32_t to = (i + 1 < m) ? s_path[i + 1] : (npath ? -1 : j);
+        int32_t x = to >= 0 ? __ldcg(td + (int64_t)s_path[i] * k + to) : -1;
+        if (to >= 0 && (uint32_t)x >= (uint32_t)n) { x = -1; B->err0 = ST_ERR_INVARIANT; }
+        s_pathu[i] = x;
+        s_raff[i] = 0;
+      }
+    }
+    __syncthreads();
+    const int chunk = min(32, max(k, kGAff) / k);   // rows whose affected entries fit s_aff
+    for (int i0 = 0; i0 < m; i0 += chunk) {
+      if (tid >= 32) merge_rows(npath, m, i0, min(m, i0 + chunk));
+      else if (i0 == 0) move_units(j, npath, m, cost);
+      __syncthreads();
+      const uint64_t t1 = timer() ? clock_cycles() : 0;
+      if (timer() && i0 == 0) B->t_apply += t1 - t0;
+      if (M->naff) rescan_affected(i0, min(m, i0 + chunk));
+      __syncthreads();
+      if (timer()) B->t_rescan += clock_cycles() - t1;
+      if (i0 + chunk < m) {
+        if (tid == 0) M->naff = 0;
+        __syncthreads();
+      }
+    }
+    return m;
+  }
+
+  __device__ __forceinline__ int32_t arriving(bool npath, int m, int i) const {
+    return i > 0 ? s_pathu[i - 1] : (npath ? -1 : s_pathu[m - 1]);
+  }
+
+  // Warp 0: member lists, allotment, loads and objective.
+  __device__ void move_units(int32_t j, bool npath, int m, int64_t cost) {
+    const int lane = tid & 31;
+    int32_t pos0 = -1, ownl = 0;   // of j's leaving unit and the last arriving unit (paths)
+    for (int b = 0; b < m; b += 32) {
+      const int i = b + lane;
+      int32_t c = 0, x_out = -1, x_in = -1, at = -1, own = 0;
+      if (i < m) {
+        c = s_path[i];
+        x_out = s_pathu[i];
+        x_in = arriving(npath, m, i);
+        if (x_out >= 0) at = pos[x_out];
+        if (x_in >= 0) own = (int32_t)row(x_in)[c];   // CM(x_in, its new center)
+        if (x_out >= 0) I.assign[x_out] = (i + 1 < m) ? s_path[i + 1] : j;
+      }
+      if (b == 0) pos0 = __shfl_sync(0xffffffffu, at, 0);
+      if (m - 1 >= b && m - 1 < b + 32) ownl = __shfl_sync(0xffffffffu, own, m - 1 - b);
+      __syncwarp();   // every position of this batch is read before any is replaced
+      if (x_out >= 0 && x_in >= 0) {
+        if (at >= 0 && at < s_seg[c]) {
+          int32_t* slot = mslot(c, at, s_seg[c]);
+          slot[0] = x_in;
+          slot[kPage] = own;
+          s_mid[i] = at;      // x_in's new position, stored below
+        } else {
+          s_mid[i] = -1;
+          B->err0 = ST_ERR_INVARIANT;
+        }
+      }
+    }
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) {   // positions, once all old ones were read
+      const int32_t x_in = arriving(npath, m, i);
+      if (s_pathu[i] >= 0 && x_in >= 0 && s_mid[i] >= 0) pos[x_in] = s_mid[i];
+    }
+    __syncwarp();
+    if (lane == 0) {
+      if (npath) {
+        const int32_t term = s_path[m - 1];
+        list_remove_at(j, pos0);
+        if (s_pathu[m - 2] >= 0) list_append(term, s_pathu[m - 2], ownl);
+        else B->err0 = ST_ERR_INVARIANT;
+        shift_load(j, -1);
+        shift_load(term, 1);
+        B->paths++;
+        B->moves += m - 1;
+      } else {
+        B->cycles++;
+        B->moves += m;
+      }
+      B->delta += cost;
+    }
+  }
+
+  // Warps 1..15: rows i0..i1 of the path.  Center s_path[i] lost unit
+  // s_pathu[i] and gained the one before it (either may be absent): an entry
+  // whose best unit was not the leaving one keeps its minimum over the
+  // remaining members and only takes the arriving unit in; the others are
+  // listed in s_aff.  All rows go through together, so that their loads
+  // overlap.
+  __device__ void merge_rows(bool npath, int m, int i0, int i1) {
+    constexpr int U = 4, W = kWarps - 1;
+    const int nblk = (k + 31) >> 5, lane = tid & 31;   // a warp takes 32 columns of one row
+    int r = 0, blk = (tid >> 5) - 1;
+    while (blk >= nblk) { blk -= nblk; ++r; }
+    while (i0 + r < i1) {
+      int32_t bd[U], ct[U], ow[U], rr[U], vv[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int i = i0 + r, v = blk * 32 + lane;
+        rr[q] = r;
+        vv[q] = v;
+        bd[q] = -2;   // no item
+        ct[q] = ow[q] = 0;
+        if (i < i1) {
+          const int32_t c = s_path[i], x_in = arriving(npath, m, i);
+          if (v < k && v != c) {
+            bd[q] = __ldcg(td + (int64_t)c * k + v);
+            if (x_in >= 0) {
+              const T* rx = row(x_in);
+              ct[q] = (int32_t)rx[v];
+              ow[q] = (int32_t)rx[c];
+            }
+          }
+          blk += W;
+          while (blk >= nblk) { blk -= nblk; ++r; }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int i = i0 + rr[q], v = vv[q];
+        if (i >= i1) break;
+        const int32_t c = s_path[i], x_out = s_pathu[i], x_in = arriving(npath, m, i);
+        const bool hit = bd[q] >= 0 && bd[q] == x_out;
+        if (!hit && bd[q] != -2 && x_in >= 0) {
+          const int32_t t = ct[q] - ow[q];
+          const int32_t e = edge(c, v);
+          const int32_t bt = e == kInf ? kTInf : e;
+          if (lex_less(t, x_in, bt, bd[q])) set_entry(c, v, t, x_in);
+        }
+        const unsigned bits = __ballot_sync(0xffffffffu, hit);
+        if (bits) {
+          int at = 0;
+          const int leader = __ffs(bits) - 1;
+          if (lane == leader) {
+            at = atomicAdd(&s_raff[i], __popc(bits));
+            M->naff = 1;
+          }
+          at = __shfl_sync(0xffffffffu, at, leader);
+          if (hit) s_aff[rr[q] * k + at + __popc(bits & ((1u << lane) - 1u))] = v;
+        }
+      }
+    }
+  }
+
+  // The listed entries of rows i0..i1, each the minimum over its center's
+  // members.  A warp takes a block of at most 32 entries of one row and a
+  // part of the member list: lane = (entry, member of eight in flight), with
+  // as many lanes per entry as the block leaves, so that few entries of a
+  // long list (a large center) still fill the warps and many entries of a
+  // short one read neighbouring columns of the same rows.  Lists of more
+  // than one part meet in a 64-bit shared minimum per entry.
+  __device__ void rescan_affected(int i0, int i1) {
+    constexpr int U = 8;
+    const int lane = tid & 31, warp = tid >> 5;
+    unsigned long long* s_best = reinterpret_cast<unsigned long long*>(s_list);   // [rows][k]
+    // lane = row: entries, list length, log2 of the entries per warp, tasks
+    const int i = i0 + lane;
+    const int na = i < i1 ? s_raff[i] : 0;
+    const int len = na > 0 ? s_seg[s_path[i]] : 0;
+    const int le = na > 16 ? 5 : na > 8 ? 4 : na > 4 ? 3 : na > 2 ? 2 : na > 1 ? 1 : 0;
+    const int parts = na > 0 ? max(1, (len + (U << (5 - le)) - 1) / (U << (5 - le))) : 0;
+    int incl = ((na + 31) >> 5) * parts;
+    const int mine = incl;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += o;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const bool split = __any_sync(0xffffffffu, parts > 1);
+    if (warp == 0) {
+      const int rows = __reduce_add_sync(0xffffffffu, len);
+      if (lane == 0) B->col_rows += rows;
+    }
+    if (split) {
+      for (int r = warp; r < i1 - i0; r += kWarps) {
+        const int na_r = __shfl_sync(0xffffffffu, na, r);
+        for (int e = lane; e < na_r; e += 32) s_best[r * k + e] = ~0ull;
+      }
+      __syncthreads();
+    }
+    for (int t = warp; t < total; t += kWarps) {
+      const int r = __popc(__ballot_sync(0xffffffffu, incl <= t));
+      const int na_r = __shfl_sync(0xffffffffu, na, r), len_r = __shfl_sync(0xffffffffu, len, r);
+      const int le_r = __shfl_sync(0xffffffffu, le, r), parts_r = __shfl_sync(0xffffffffu, parts, r);
+      const int t0 = t - __shfl_sync(0xffffffffu, incl - mine, r);
+      const int blk = t0 / parts_r, part = t0 - blk * parts_r;
+      const int e = (blk << 5) + (lane & ((1 << le_r) - 1)), sub = lane >> le_r;
+      const int step = 32 >> le_r;
+      const int32_t c = s_path[i0 + r];
+      const int32_t v = e < na_r ? s_aff[r * k + e] : 0;
+      const int32_t base = part * U * step + sub;
+      unsigned long long best = ~0ull;
+      if (e < na_r && base < len_r) {
+        // a part is a power of two of at most a page's entries: one page
+        const int32_t* sl = mslot(c, base, len_r);
+        const int left = (len_r - base + step - 1) >> (5 - le_r);
+        const T* cv = cm + v;
+        int32_t id[U], ow[U], x[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          const int32_t at = (q < left ? q : 0) << (5 - le_r);   // past the end: the first again
+          id[q] = sl[at];
+          ow[q] = sl[at + kPage];
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          if ((uint32_t)id[q] >= (uint32_t)n) id[q] = 0;   // guard: corrupt entry
+          x[q] = (int32_t)cv[(int64_t)id[q] * ld];
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+          best = min(best, ((unsigned long long)((uint32_t)(x[q] - ow[q]) ^ 0x80000000u) << 32) |
+                               (uint32_t)id[q]);
+      }
+      for (int s = 1 << le_r; s < 32; s <<= 1)
+        best = min(best, (unsigned long long)__shfl_xor_sync(0xffffffffu, best, s));
+      if (e < na_r && sub == 0) {
+        if (parts_r > 1) atomicMin(&s_best[r * k + e], best);
+        else put_entry(c, v, best);
+      }
+    }
+    if (split) {
+      __syncthreads();
+      for (int r = warp; r < i1 - i0; r += kWarps) {
+        const int na_r = __shfl_sync(0xffffffffu, na, r);
+        if (__shfl_sync(0xffffffffu, parts, r) > 1)
+          for (int e = lane; e < na_r; e += 32)
+            put_entry(s_path[i0 + r], s_aff[r * k + e], s_best[r * k + e]);
+      }
+    }
+  }
+  __device__ __forceinline__ void put_entry(int32_t c, int32_t v, unsigned long long best) {
+    if (best == ~0ull) set_entry(c, v, kTInf, -1);
+    else set_entry(c, v, (int32_t)((int64_t)(best >> 32) - 2147483648LL),
+                   (int32_t)(best & 0xffffffffu));
+  }
+
+  // Rows list[0..m) of T against the prices: sets M->bad if an entry breaks
+  // P(u) <= T[u][v] + P(v), or a price exceeds q_n.
+  __device__ bool broken_rows(const int32_t* list, int m) {
+    const int kp = (k + 31) & ~31;
+    const int total = m * kp;
+    bool bad = false;
+    for (int it = tid; it < total; it += kThreads) {
+      const int i = it / kp, v = it % kp;
+      const int32_t c = list[i];
+      if (v < k && v != c) {
+        const int32_t t = edge(c, v);
+        if (t != kInf && (int64_t)s_pot[c] > (int64_t)t + s_pot[v]) bad = true;
+      } else if (v == c && s_pot[c] > s_qn[c]) {
+        bad = true;
+      }
+    }
+    return bad;
+  }
+
+  // Prices from the table: P = q_n lowered by whole sweeps until every entry
+  // holds (reverse Bellman-Ford; exact distances to a paid slot).
+  __device__ bool rebuild_prices() {
+    const int lane = tid & 31, warp = tid >> 5;
+    for (int v = tid; v < k; v += kThreads) s_pot[v] = s_qn[v];
+    __syncthreads();
+    for (int sweep = 0; sweep <= k + 1; ++sweep) {
+      bool any = false;
+      for (int u = warp; u < k; u += kWarps) {
+        int64_t best = INT64_MAX;
+        for (int v = lane; v < k; v += 32) {
+          const int32_t t = v != u ? edge(u, v) : kInf;
+          if (t != kInf) best = min(best, (int64_t)t + s_pot[v]);
+        }
+        for (int off = 16; off > 0; off >>= 1)
+          best = min(best, (int64_t)__shfl_xor_sync(0xffffffffu, best, off));
+        if (best < s_pot[u]) {
+          any = true;
+          __syncwarp();
+          if (lane == 0) s_pot[u] = clamp32(best);
+        }
+        __syncwarp();
+      }
+      if (__syncthreads_or(any) == 0) return true;
+    }
+    return false;   // a negative cycle in Gamma: Lemmas 1/2 broken
+  }
+
+  // ----------------------------------------------------------- the loop --
+  __device__ __forceinline__ void load_order(int64_t r, int64_t r_end, int slot) {
+    const int32_t d = r < r_end ? I.order[r] : -1;
+    const int32_t j = (uint32_t)d < (uint32_t)n ? I.smin[d] : -1;
+    s_ord[2 * slot] = d;
+    s_ord[2 * slot + 1] = (uint32_t)j < (uint32_t)k ? j : -1;
+  }
+  __device__ __forceinline__ void fetch_row(int32_t q, int32_t count) {
+    if (q < count) {
+      const int32_t d = s_ord[2 * (q & (kGOrd - 1))];
+      if ((uint32_t)d < (uint32_t)n) {
+        unsigned char* dst = s_ring + (uint32_t)(q & (nring - 1)) * ring_row;
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(row(d));
+        for (uint32_t b = 16u * (uint32_t)tid; b < ring_row; b += 16u * kThreads)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + b)),
+                       "l"(src + b) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+
+  __device__ void run_rounds(uint64_t deadline) {
+    const uint64_t tstart = tid == 0 ? gtimer_ns() : 0;
+    const uint64_t cstart = tid == 0 ? clock_cycles() : 0;
+    const int64_t r_begin = I.ctl[CTL_ROUNDS];
+    const int64_t r_end = min((int64_t)n, I.ctl[CTL_TARGET]);
+    const int32_t count = (int32_t)max((int64_t)0, r_end - r_begin);
+    for (int v = tid; v < k; v += kThreads) {
+      const int32_t ld = I.load[v], sg = I.seg_size[v];
+      s_slack[v] = ld - __ldg(I.cap + v);
+      s_pen[v] = qval(v, s_slack[v] + 1);
+      s_qn[v] = s_slack[v] >= 0 ? s_pen[v] : 0;
+      s_seg[v] = sg;
+      s_tail[v] = sg > 0 ? page_tab[(int64_t)v * max_pages + ((sg - 1) >> kPageShift)] : 0;
+      s_pot[v] = I.pot[v];
+    }
+    if (tid == 0) {
+      B->delta = I.ctl[CTL_DELTA];
+      B->free_top = I.ctl[CTL_FREE_TOP];
+      B->cycles = B->paths = B->bf_calls = B->bf_sweeps = B->bf_max = B->moves = B->skipped = B->rows = 0;
+      B->t_merge = B->t_relax = B->t_sync = B->t_gather = B->t_apply = B->t_rescan = 0;
+      B->t_rloop = B->t_rred = 0;
+      B->err0 = 0;
+      B->npath_reused = 0;
+      B->col_rows = 0;
+      B->front_sum = 0;
+      for (int h = 0; h < 6; ++h) B->front_hist[h] = 0;
+      M->bad = 0;
+      M->stop = 0;
+      M->naff = 0;
+    }
+    if (TSM || I.ctl[CTL_MIRROR] == 0)
+      for (int64_t u = 0; u < k; ++u)
+        for (int cl = tid; cl < ws; cl += kThreads) {
+          const int32_t t = cl < k ? tc[u * k + cl] : kTInf;
+          tt[u * ws + cl] = (T)(t == kTInf ? kInf : t);
+        }
+    if (tid < kGOrd) load_order(r_begin + tid, r_end, tid);
+    __syncthreads();
+    bool prices_ok = I.ctl[CTL_POT] != 0;
+    int64_t status = ST_OK;
+    int32_t q = 0;
+    for (int i = 0; i + 1 < nring; ++i) fetch_row(i, count);
+    for (; q < count; ++q) {
+      if (deadline && q > 0 && q % kQuantumCheck == 0) {
+        if (tid == 0) M->stop = gtimer_ns() >= deadline ? 1 : 0;
+        __syncthreads();
+        if (M->stop) break;
+      }
+      if (!prices_ok) {
+        if (!rebuild_prices()) { status = ST_ERR_INVARIANT; break; }
+        prices_ok = true;
+      }
+      const uint64_t tm0 = timer() ? clock_cycles() : 0;
+      fetch_row(q + nring - 1, count);
+      if (q > 0 && q % 32 == 0 && tid >= kThreads - 32) {
+        const int32_t at = q + 32 + (tid & 31);
+        load_order(r_begin + at, r_end, at & (kGOrd - 1));
+      }
+      const int32_t d = s_ord[2 * (q & (kGOrd - 1))], j = s_ord[2 * (q & (kGOrd - 1)) + 1];
+      if (d < 0 || j < 0) { status = ST_ERR_INVARIANT; break; }   // uniform guard
+      if (nring == 8) asm volatile("cp.async.wait_group 7;" ::: "memory");
+      else asm volatile("cp.async.wait_group 3;" ::: "memory");
+      __syncthreads();
+      // Alg. 2, allotment: d joins j; its edges enter row j of T
+      const T* r = reinterpret_cast<const T*>(s_ring + (uint32_t)(q & (nring - 1)) * ring_row);
+      const int32_t own = (int32_t)r[j];
+      const bool over = s_slack[j] >= 0;
+      const int32_t ql = over ? s_pen[j] : 0;   // q_j(load - cap + 1), paid by d
+      const int32_t pj = s_pot[j];
+      bool viol = false;
+      for (int cl = tid; cl < k; cl += kThreads) {
+        if (cl == j) continue;
+        const int32_t t = (int32_t)r[cl] - own;
+        const int32_t e = edge(j, cl);
+        const int32_t bt = e == kInf ? kTInf : e;
+        // equal costs take the lower unit: a reduction nobody waits for (so
+        // td is read past L1 everywhere)
+        if (t < bt) set_entry(j, cl, t, d);
+        else if (t == bt)
+          atomicMin(reinterpret_cast<unsigned*>(td + (int64_t)j * k + cl), (unsigned)d);
+        viol |= (int64_t)t + s_pot[cl] < (int64_t)pj;
+      }
+      viol = __syncthreads_or(viol) != 0;
+      if (tid == kThreads - 32) {
+        I.assign[d] = j;
+        list_append(j, d, own);
+        shift_load(j, 1);
+        B->delta += own + ql;
+      }
+      if (timer()) B->t_merge += clock_cycles() - tm0;
+      if (!viol) {
+        if (tid == 0) B->skipped++;
+        if (!over || pj >= ql) continue;
+      }
+      // Alg. 1 and Alg. 4 at j
+      const uint64_t ts0 = timer() ? clock_cycles() : 0;
+      search(j, viol, over, s_lab1, s_pot, ql);
+      if (timer()) B->t_relax += clock_cycles() - ts0;
+      if (M->bad) { status = ST_ERR_INVARIANT; break; }
+      const int64_t cycv = viol ? (int64_t)s_lab1[j] : 0;
+      const uint32_t sink1 = M->sink;
+      const int64_t D1 = over ? (int64_t)M->paid : INT32_MAX;   // exact below ql
+      bool bad = false;
+      if (cycv >= 0) {
+        const int64_t dd = min(D1, (int64_t)ql);
+        for (int v = tid; v < k; v += kThreads) {
+          if (v == j) s_pot[v] = (int32_t)max((int64_t)pj, dd);
+          else if (s_lab1[v] != kNoLab) s_pot[v] = (int32_t)max((int64_t)s_pot[v], dd - (int64_t)s_lab1[v]);
+        }
+        if (over && tid == 0) B->npath_reused++;
+        if (over && D1 < ql) {
+          const int m = apply(j, true, (int32_t)(sink1 & ((1u << kGNodeBits) - 1)), s_lab1, D1 - ql);
+          if (m < 0) { status = ST_ERR_INVARIANT; break; }
+          bad = broken_rows(s_path, m);
+        }
+      } else {
+        const int mc = apply(j, false, -1, s_lab1, cycv);
+        if (mc < 0) { status = ST_ERR_INVARIANT; break; }
+        for (int i = tid; i < mc; i += kThreads) s_cpath[i] = s_path[i];
+        int64_t d2 = 0, D2 = 0;
+        int m2 = 0;
+        if (over) {
+          const int64_t dt = pj + cycv;
+          const uint64_t ts1 = timer() ? clock_cycles() : 0;
+          const int64_t off = max((int64_t)0, dt - D1);
+          for (int v = tid; v < k; v += kThreads) {
+            int64_t p = s_pot[v];
+            if (v != j && s_lab1[v] != kNoLab) p = max(p, dt - (int64_t)s_lab1[v]);
+            s_mid[v] = (int32_t)max(p - off, (int64_t)-kGPenLimit);
+          }
+          search(j, false, true, s_lab2, s_mid, ql);
+          if (timer()) B->t_relax += clock_cycles() - ts1;
+          if (M->bad) { status = ST_ERR_INVARIANT; break; }
+          D2 = M->paid;
+          d2 = min((int64_t)ql, D2);
+        }
+        const uint32_t sink2 = M->sink;
+        const int64_t dd = over ? cycv + d2 : min(D1, cycv);
+        if (!over) d2 = dd - cycv;
+        for (int v = tid; v < k; v += kThreads) {
+          int64_t p = s_pot[v];
+          if (v == j) {
+            p = max((int64_t)pj, d2);
+          } else {
+            if (s_lab1[v] != kNoLab) p = max(p, dd - (int64_t)s_lab1[v]);
+            if (over && s_lab2[v] != kNoLab) p = max(p, d2 - (int64_t)s_lab2[v]);
+          }
+          s_pot[v] = clamp32(p);
+        }
+        if (over && D2 < ql) {
+          m2 = apply(j, true, (int32_t)(sink2 & ((1u << kGNodeBits) - 1)), s_lab2, D2 - ql);
+          if (m2 < 0) { status = ST_ERR_INVARIANT; break; }
+        }
+        __syncthreads();   // prices and rows are final
+        bad = broken_rows(s_cpath, mc) | broken_rows(s_path, m2);
+      }
+      if (__syncthreads_or(bad)) prices_ok = false;   // rebuilt before the next round
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    for (int v = tid; v < k; v += kThreads) {
+      I.pot[v] = s_pot[v];
+      I.load[v] = s_slack[v] + __ldg(I.cap + v);
+      I.seg_size[v] = s_seg[v];
+    }
+    if (tid == 0) {
+      I.ctl[CTL_POT] = prices_ok && status == ST_OK ? 1 : 0;
+      if (count > 0) I.ctl[CTL_MIRROR] = TSM ? 0 : 1;
+      I.ctl[CTL_ROUNDS] = r_begin + q;
+      I.ctl[CTL_DELTA] = B->delta;
+      I.ctl[CTL_FREE_TOP] = B->free_top;
+      I.ctl[CTL_STATUS] = status != ST_OK ? status : B->err0;
+      I.ctl[CTL_CYCLES] += B->cycles;
+      I.ctl[CTL_PATHS] += B->paths;
+      I.ctl[CTL_BF_CALLS] += B->bf_calls;
+      I.ctl[CTL_BF_SWEEPS] += B->bf_sweeps;
+      I.ctl[CTL_BF_MAX] = max(I.ctl[CTL_BF_MAX], B->bf_max);
+      I.ctl[CTL_MOVES] += B->moves;
+      I.ctl[CTL_NCYC_SKIPPED] += B->skipped;
+      I.ctl[CTL_ROWS_SCANNED] += B->rows;
+      I.ctl[CTL_T_TOTAL] += gtimer_ns() - tstart;
+      I.ctl[CTL_T_CYCLES] += clock_cycles() - cstart;
+      I.ctl[CTL_T_MERGE] += B->t_merge;
+      I.ctl[CTL_T_RELAX] += B->t_relax;
+      I.ctl[CTL_T_APPLY] += B->t_apply;
+      I.ctl[CTL_T_RESCAN] += B->t_rescan;
+      I.ctl[CTL_TSM_ON] = TSM ? 1 : 0;
+      I.ctl[CTL_NPATH_REUSED] += B->npath_reused;
+      I.ctl[CTL_COL_ROWS] += B->col_rows;
+      I.ctl[CTL_FRONT_SUM] += B->front_sum;
+      for (int h = 0; h < 6; ++h) I.ctl[CTL_FRONT_HIST + h] += B->front_hist[h];
+    }
+    __syncthreads();
+  }
+};
+
+}  // namespace lbdd

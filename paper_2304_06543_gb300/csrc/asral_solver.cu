@@ -1418,6 +1418,7 @@ struct Solver {
     __syncthreads();
     cluster_sync_all();
     if (rank == 0 && tid == 0) {
+      if (r > r_begin) I.ctl[CTL_POT] = I.ctl[CTL_MIRROR] = 0;   // rounds that keep neither
       I.ctl[CTL_ROUNDS] = r;
       I.ctl[CTL_DELTA] = B->delta;
       I.ctl[CTL_FREE_TOP] = B->free_top;
@@ -1556,6 +1557,97 @@ asral_cluster_kernel(const DevInst* __restrict__ insts, int ninst, int* work_cou
   }
 }
 
+}  // namespace lbdd
+
+#include "asral_guided.cuh"
+
+namespace lbdd {
+
+// Instances of a launch solved one per CTA with the guided rounds.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1)
+asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_counter, int flags,
+                    uint64_t quantum_ns) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ DevInst s_inst;
+  __shared__ Book s_book;
+  __shared__ int s_item;
+  __shared__ uint64_t s_deadline;
+  const int tid = threadIdx.x;
+  if (tid == 0) s_deadline = quantum_ns ? gtimer_ns() + quantum_ns : 0;
+  const uint32_t avail = dyn_smem_bytes();
+  for (;;) {
+    if (tid == 0) {   // next instance with rounds left and no error
+      int it = ninst;
+      if (!s_deadline || gtimer_ns() < s_deadline) {
+        for (;;) {
+          it = atomicAdd(work_counter, 1);
+          if (it >= ninst) break;
+          const int64_t* c = insts[it].ctl;
+          const int64_t target = min((int64_t)insts[it].n, __ldcg(c + CTL_TARGET));
+          if (__ldcg(c + CTL_STATUS) == 0 &&
+              (__ldcg(c + CTL_PROLOGUE) == 0 || __ldcg(c + CTL_ROUNDS) < target))
+            break;
+        }
+      }
+      s_item = it;
+      if (it < ninst) s_inst = insts[it];
+    }
+    __syncthreads();
+    if (s_item >= ninst) break;
+    const GLayout L = make_guided_layout(s_inst.k, (int)sizeof(T));
+    if (s_inst.ctl[CTL_PROLOGUE] == 0) {
+      const uint64_t t0 = gtimer_ns();
+      Solver<T> S(s_inst);
+      S.B = &s_book;
+      S.tid = tid;
+      S.rank = 0;
+      S.C = 1;
+      S.flags = flags;
+      S.cm = static_cast<const T*>(s_inst.cm);
+      S.n = s_inst.n;
+      S.k = s_inst.k;
+      S.w = own_width(S.k, 1, Solver<T>::VPL);
+      S.c0 = 0;
+      S.c1 = S.wr = S.k;
+      S.s_red = smem + L.ring;
+      S.prologue();
+      for (int v = tid; v < s_inst.k; v += kThreads) s_inst.pot[v] = 0;
+      if (tid == 0) {
+        s_inst.ctl[CTL_FREE_TOP] = s_inst.npages;
+        s_inst.ctl[CTL_ROUNDS] = 0;
+        s_inst.ctl[CTL_DELTA] = 0;
+        s_inst.ctl[CTL_POT] = 1;
+        s_inst.ctl[CTL_PROLOGUE] = 1;
+        s_inst.ctl[CTL_T_PROLOGUE] += gtimer_ns() - t0;
+      }
+      __syncthreads();
+    }
+    if (L.total <= avail && !(flags & OPT_NO_TC_SMEM)) {
+      Guided<T, true> G(s_inst, smem, L, &s_book, flags);
+      G.run_rounds(s_deadline);
+    } else {
+      Guided<T, false> G(s_inst, smem, L, &s_book, flags);
+      G.run_rounds(s_deadline);
+    }
+  }
+}
+
+// Shared memory of a guided CTA for k centers (with the cost slice of T
+// when that fits `limit`), 0 if it does not fit.
+size_t guided_smem_bytes(int32_t k, int elem_bytes, size_t limit) {
+  if (k >= 1 << kGNodeBits) return 0;
+  const GLayout L = make_guided_layout(k, elem_bytes);
+  return L.total <= limit ? L.total : L.base_total <= limit ? L.base_total : 0;
+}
+
+int32_t guided_pen_limit() { return kGPenLimit; }
+
+// Bytes of the global mirror of T's costs.
+size_t guided_mirror_bytes(int32_t k, int elem_bytes) {
+  return (size_t)k * guided_stride(k, elem_bytes) * elem_bytes;
+}
+
 // Shared-memory bytes of one CTA for an instance with k centers on C-CTA
 // clusters (includes the 16-byte work-item slot).  with_slice: also the
 // owned cost slice.
@@ -1570,15 +1662,14 @@ int solver_max_k(int C, int elem_bytes) {
 }
 
 template <typename T>
-cudaError_t prepare_solver_t(int C, size_t smem);
+cudaError_t prepare_solver_t(int C, size_t smem, int flags);
 
 template <typename T>
 cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, int C,
                             int nclusters, size_t smem, int flags, cudaStream_t st,
                             uint64_t quantum_ns, bool set_attrs) {
-  auto kern = asral_cluster_kernel<T>;
   if (set_attrs) {
-    const cudaError_t e = prepare_solver_t<T>(C, smem);
+    const cudaError_t e = prepare_solver_t<T>(C, smem, flags);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
@@ -1586,6 +1677,9 @@ cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, i
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
+  if (flags & OPT_GUIDED)   // no cluster: every CTA takes instances of its own
+    return cudaLaunchKernelEx(&cfg, asral_guided_kernel<T>, d_insts, ninst, d_counter, flags,
+                              quantum_ns);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)C;
@@ -1593,7 +1687,7 @@ cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, i
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, d_insts, ninst, d_counter, flags, quantum_ns);
+  return cudaLaunchKernelEx(&cfg, asral_cluster_kernel<T>, d_insts, ninst, d_counter, flags, quantum_ns);
 }
 
 // Kernel attributes only ever grow (a launch needs at least its own dynamic
@@ -1601,16 +1695,25 @@ cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, i
 // Attributes belong to the current device, so the high-water marks are kept
 // per device.
 template <typename T>
-cudaError_t prepare_solver_t(int C, size_t smem) {
+cudaError_t prepare_solver_t(int C, size_t smem, int flags) {
   constexpr int kDevs = 64;
   static std::mutex mu;
-  static size_t cur_smem[kDevs] = {};
+  static size_t cur_smem[kDevs] = {}, cur_guided[kDevs] = {};
   static bool non_portable[kDevs] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kDevs) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(mu);
+  if (flags & OPT_GUIDED) {
+    if (smem > cur_guided[dev]) {
+      e = cudaFuncSetAttribute(asral_guided_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)smem);
+      if (e != cudaSuccess) return e;
+      cur_guided[dev] = smem;
+    }
+    return cudaSuccess;
+  }
   auto kern = asral_cluster_kernel<T>;
   if (smem > cur_smem[dev]) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1625,8 +1728,9 @@ cudaError_t prepare_solver_t(int C, size_t smem) {
   return cudaSuccess;
 }
 
-cudaError_t prepare_solver(int C, int elem_bytes, size_t smem) {
-  return elem_bytes == 2 ? prepare_solver_t<int16_t>(C, smem) : prepare_solver_t<int32_t>(C, smem);
+cudaError_t prepare_solver(int C, int elem_bytes, size_t smem, int flags) {
+  return elem_bytes == 2 ? prepare_solver_t<int16_t>(C, smem, flags)
+                         : prepare_solver_t<int32_t>(C, smem, flags);
 }
 
 cudaError_t launch_solver(const DevInst* d_insts, int ninst, int* d_counter, int C,
@@ -1641,7 +1745,17 @@ cudaError_t launch_solver(const DevInst* d_insts, int ninst, int* d_counter, int
 
 // Largest number of co-resident clusters of size C for this kernel.
 template <typename T>
-static int max_clusters_t(int C, size_t smem) {
+static int max_clusters_t(int C, size_t smem, int flags) {
+  if (prepare_solver_t<T>(C, smem, flags) != cudaSuccess) return -1;
+  if (flags & OPT_GUIDED) {
+    int per_sm = 0, dev = 0, sms = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, asral_guided_kernel<T>, kThreads,
+                                                      smem) != cudaSuccess ||
+        cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return -1;
+    return per_sm * sms;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)C, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -1654,13 +1768,13 @@ static int max_clusters_t(int C, size_t smem) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   auto kern = asral_cluster_kernel<T>;
-  if (prepare_solver_t<T>(C, smem) != cudaSuccess) return -1;
   int num = 0;
   return cudaOccupancyMaxActiveClusters(&num, kern, &cfg) == cudaSuccess ? num : -1;
 }
 
-int solver_max_clusters(int C, int elem_bytes, size_t smem) {
-  return elem_bytes == 2 ? max_clusters_t<int16_t>(C, smem) : max_clusters_t<int32_t>(C, smem);
+int solver_max_clusters(int C, int elem_bytes, size_t smem, int flags) {
+  return elem_bytes == 2 ? max_clusters_t<int16_t>(C, smem, flags)
+                         : max_clusters_t<int32_t>(C, smem, flags);
 }
 
 }  // namespace lbdd

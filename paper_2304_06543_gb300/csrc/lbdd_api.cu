@@ -213,6 +213,9 @@ extern "C" int32_t lbdd_max_centers(void) {
   return best;
 }
 
+// Centers up to which a lone solve runs guided on one CTA by default.
+constexpr int32_t kGuidedMaxK = 1024;
+
 static int fits(const lbdd_solver* s, int C) { return fits_k(s->k, s->elem, C) ? 1 : 0; }
 
 size_t lbdd::solver_footprint(int32_t n, int32_t k, int in_elem, int elem) {
@@ -227,9 +230,10 @@ size_t lbdd::solver_footprint(int32_t n, int32_t k, int in_elem, int elem) {
   b += 2 * a(4ull * k);                       // cap, pen
   b += 2 * a(4ull * n) + a(12ull * n);        // smin, order, sort_tmp
   b += 2 * a(4ull * n);                       // assign, pos
-  b += 2 * a(4ull * k);                       // load, seg_size
+  b += 3 * a(4ull * k);                       // load, seg_size, pot
   b += a(4ull * k * max_pages) + a(4ull * npages * kPageWords) + a(4ull * npages);
   b += 2 * a(4ull * k * k);                   // tc, td
+  if (guided_smem_bytes(k, elem, kMaxSmem) > 0) b += a(guided_mirror_bytes(k, elem));
   b += a(8ull * CTL_COUNT) + a(16) + a(sizeof(DevInst));
   return b;
 }
@@ -249,6 +253,7 @@ static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, 
   if (!s) return LBDD_ERR_OOM;
   s->n = n;
   s->n_cap = n;
+  s->max_pen = *std::max_element(pen, pen + k);
   s->k = k;
   s->st = static_cast<cudaStream_t>(cuda_stream);
   int rc = check_device(&s->device, &s->num_sms);
@@ -272,6 +277,9 @@ static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, 
   if (!rc) rc = dalloc(s, &s->free_stack, npages);
   if (!rc) rc = dalloc(s, &s->tc, (size_t)k * k);
   if (!rc) rc = dalloc(s, &s->td, (size_t)k * k);
+  if (!rc) rc = dalloc(s, &s->pot, k);
+  if (!rc && guided_smem_bytes(k, s->elem, kMaxSmem) > 0)
+    rc = dev_alloc(s, &s->mirror, guided_mirror_bytes(k, s->elem));
   if (!rc) rc = dalloc(s, &s->ctl, CTL_COUNT);
   if (!rc) rc = dalloc(s, &s->counter, 4);
   if (!rc) rc = dalloc(s, &s->d_inst, 1);
@@ -280,7 +288,8 @@ static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, 
   I.cm = s->cm; I.ld = s->ld; I.n = n; I.k = k; I.cap = s->cap; I.pen = s->pen; I.Q = 1;
   I.smin = s->smin; I.order = s->order; I.sort_tmp = s->sort_tmp; I.assign = s->assign;
   I.pos = s->pos; I.load = s->load; I.seg_size = s->seg_size; I.page_tab = s->page_tab;
-  I.pool = s->pool; I.free_stack = s->free_stack; I.tc = s->tc; I.td = s->td; I.ctl = s->ctl;
+  I.pool = s->pool; I.free_stack = s->free_stack; I.tc = s->tc; I.td = s->td; I.pot = s->pot; I.mirror = s->mirror;
+  I.ctl = s->ctl;
   I.max_pages = max_pages; I.npages = npages;
   auto fail = [&](cudaError_t e, const char* w) { int r = cuda_fail(e, w); free_all(s); delete s; return r; };
   cudaError_t e;
@@ -289,6 +298,7 @@ static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, 
   if ((e = cudaMemsetAsync(s->ctl, 0, sizeof(int64_t) * CTL_COUNT, s->st))) return fail(e, "ctl");
   if ((e = cudaMemsetAsync(s->assign, 0xff, 4ull * n, s->st))) return fail(e, "assign");
   if ((e = cudaMemsetAsync(s->load, 0, 4ull * k, s->st))) return fail(e, "load");
+  if ((e = cudaMemsetAsync(s->pot, 0, 4ull * k, s->st))) return fail(e, "pot");
   // defined contents everywhere, so that a corrupt index can never leave the pool
   if ((e = cudaMemsetAsync(s->page_tab, 0, 4ull * k * max_pages, s->st))) return fail(e, "pages");
   if ((e = cudaMemsetAsync(s->pool, 0, 4ull * npages * kPageWords, s->st))) return fail(e, "pool");
@@ -431,6 +441,7 @@ extern "C" int lbdd_set_penalty_table(lbdd_solver* s, const int32_t* qtab, int32
   int rc = dalloc(s, &table, (size_t)s->k * Q);
   if (rc) return rc;
   CK(cudaMemcpyAsync(table, qtab, 4ull * s->k * Q, cudaMemcpyHostToDevice, s->st));
+  s->max_pen = *std::max_element(qtab, qtab + (size_t)s->k * Q);
   s->h_inst.pen = table;
   s->h_inst.Q = Q;
   CK(cudaMemcpyAsync(s->d_inst, &s->h_inst, sizeof(DevInst), cudaMemcpyHostToDevice, s->st));
@@ -495,10 +506,30 @@ int lbdd::solver_flags(const lbdd_solver* s) {
          (s->strict ? OPT_STRICT : 0);
 }
 
+bool lbdd::solver_guided(const lbdd_solver* s, int C) {
+  return C == 1 && s->ncyc_skip && s->npath_reuse && !s->strict && s->mirror &&
+         s->max_pen < guided_pen_limit() &&
+         guided_smem_bytes(s->k, s->elem, kMaxSmem) > 0;
+}
+
+bool lbdd::solver_fits(const lbdd_solver* s, int C) {
+  return solver_guided(s, C) || fits_k(s->k, s->elem, C);
+}
+
+int lbdd::launch_flags(const lbdd_solver* s, int C) {
+  return solver_flags(s) | (solver_guided(s, C) ? OPT_GUIDED : 0);
+}
+
+size_t lbdd::launch_smem_of(const lbdd_solver* s, int C) {
+  return solver_guided(s, C) ? guided_smem_bytes(s->k, s->elem, kMaxSmem)
+                             : launch_smem(s->k, C, s->elem);
+}
+
 int lbdd::choose_cluster(lbdd_solver* s) {
+  if (s->cluster == 0 && s->k <= kGuidedMaxK && solver_guided(s, 1)) return 1;
   int C = pick_cluster(s);
-  while (C > 1 && !fits(s, C)) C >>= 1;
-  return fits(s, C) ? C : 0;
+  while (C > 1 && !solver_fits(s, C)) C >>= 1;
+  return solver_fits(s, C) ? C : 0;
 }
 
 extern "C" int lbdd_solve(lbdd_solver* s, int64_t max_rounds) {
@@ -507,9 +538,9 @@ extern "C" int lbdd_solve(lbdd_solver* s, int64_t max_rounds) {
   if (rc) return rc;
   const int C = choose_cluster(s);
   if (C < 1) return LBDD_ERR_ARG;
-  const size_t smem = launch_smem(s->k, C, s->elem);
+  const size_t smem = launch_smem_of(s, C);
   CK(cudaMemsetAsync(s->counter, 0, sizeof(int32_t), s->st));
-  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, solver_flags(s), s->st));
+  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, launch_flags(s, C), s->st));
   int64_t st = 0;
   CK(cudaMemcpyAsync(&st, s->ctl + CTL_STATUS, sizeof(int64_t), cudaMemcpyDeviceToHost, s->st));
   CK(cudaStreamSynchronize(s->st));
@@ -519,8 +550,8 @@ extern "C" int lbdd_solve(lbdd_solver* s, int64_t max_rounds) {
 int lbdd::solve_timed(lbdd_solver* s, int64_t max_rounds, int C, float* ms) {
   int rc = set_target(s, max_rounds, s->st);
   if (rc) return rc;
-  if (C < 1 || !fits(s, C)) return LBDD_ERR_ARG;
-  const size_t smem = launch_smem(s->k, C, s->elem);
+  if (C < 1 || !solver_fits(s, C)) return LBDD_ERR_ARG;
+  const size_t smem = launch_smem_of(s, C);
   struct Events {   // destroyed on every return path
     cudaEvent_t a = nullptr, b = nullptr;
     ~Events() {
@@ -531,9 +562,9 @@ int lbdd::solve_timed(lbdd_solver* s, int64_t max_rounds, int C, float* ms) {
   CK(cudaEventCreate(&ev.a));
   CK(cudaEventCreate(&ev.b));
   CK(cudaMemsetAsync(s->counter, 0, sizeof(int32_t), s->st));
-  CK(prepare_solver(C, s->elem, smem));
+  CK(prepare_solver(C, s->elem, smem, launch_flags(s, C)));
   CK(cudaEventRecord(ev.a, s->st));
-  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, solver_flags(s), s->st, 0,
+  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, launch_flags(s, C), s->st, 0,
                    false));
   CK(cudaEventRecord(ev.b, s->st));
   int64_t st = 0;

@@ -82,7 +82,10 @@ static int wid(int elem) { return elem == 2 ? 0 : 1; }
 
 // Default cluster size when nothing is measured: about 128 owned columns
 // per CTA (fewer SMs per instance than a lone solve, which favours latency).
-static int default_cluster(int32_t k, int elem) {
+static int default_cluster(const lbdd_solver* s) {
+  if (solver_guided(s, 1)) return 1;   // one CTA runs the guided rounds
+  const int32_t k = s->k;
+  const int elem = s->elem;
   int C = 1;
   while (C < 16 && (int64_t)C * 128 < k) C <<= 1;
   while (C < 16 && !fits_k(k, elem, C)) C <<= 1;
@@ -128,10 +131,10 @@ static int choose_sizes(lbdd_solver* const* v, int m, int forced_C, int dev,
     }
     const double* row = tab.ns[wid(s->elem)][bucket_of(s->k)];
     for (int C = 1; C <= 16; C <<= 1)
-      if (row[cidx(C)] > 0 && fits_k(s->k, s->elem, C)) (*cands)[i].push_back({C, row[cidx(C)]});
+      if (row[cidx(C)] > 0 && solver_fits(s, C)) (*cands)[i].push_back({C, row[cidx(C)]});
     if ((*cands)[i].empty()) {
-      const int C = default_cluster(s->k, s->elem);
-      if (!fits_k(s->k, s->elem, C)) return LBDD_ERR_ARG;
+      const int C = default_cluster(s);
+      if (!solver_fits(s, C)) return LBDD_ERR_ARG;
       (*est)[i] = Est{C, (double)s->k / C + 1.0};
       continue;
     }
@@ -154,7 +157,7 @@ static int build_groups(lbdd_solver* const* v, const int64_t* rem, int m,
   groups->clear();
   for (int i = 0; i < m; ++i) {
     Group* g = nullptr;
-    const int fl = solver_flags(v[i]);
+    const int fl = launch_flags(v[i], est[i].C);
     for (auto& x : *groups)
       if (x.elem == v[i]->elem && x.C == est[i].C && x.flags == fl) g = &x;
     if (!g) {
@@ -180,9 +183,8 @@ static int build_groups(lbdd_solver* const* v, const int64_t* rem, int m,
       const double la = (double)rem[a] * est[a].t, lb = (double)rem[b] * est[b].t;
       return order == LONGEST_FIRST ? la > lb : la < lb;
     });
-    int32_t kmax = 0;
-    for (int i : g.idx) kmax = std::max(kmax, v[i]->k);
-    g.smem = launch_smem(kmax, g.C, g.elem);
+    g.smem = 0;
+    for (int i : g.idx) g.smem = std::max(g.smem, launch_smem_of(v[i], g.C));
     if (g.smem > kMaxSmem) return LBDD_ERR_ARG;
   }
   return LBDD_OK;
@@ -190,7 +192,7 @@ static int build_groups(lbdd_solver* const* v, const int64_t* rem, int m,
 
 // Upper bound on a group's clusters: its instances, co-residency, the SMs.
 static int group_cap(const Group& g, int max_clusters, int sms, int* cap) {
-  const int fit = solver_max_clusters(g.C, g.elem, g.smem);
+  const int fit = solver_max_clusters(g.C, g.elem, g.smem, g.flags);
   if (fit < 1) {
     (void)cudaGetLastError();   // the refused query's error is reported as LBDD_ERR_ARG
     return LBDD_ERR_ARG;
@@ -418,7 +420,7 @@ int batch_set(lbdd_batch* b, lbdd_solver* const* solvers, const int64_t* rem, in
     }
   }
   CK(cudaMemcpyAsync(b->d_insts, b->h_insts, sizeof(DevInst) * m, cudaMemcpyHostToDevice, b->st));
-  for (auto& g : b->groups) CK(prepare_solver(g.C, g.elem, g.smem));
+  for (auto& g : b->groups) CK(prepare_solver(g.C, g.elem, g.smem, g.flags));
   return LBDD_OK;
 }
 
@@ -447,7 +449,7 @@ int batch_capture(lbdd_batch* b) {
 // Starts one pass (max_rounds more rounds for every instance) on b->st.
 int batch_launch(lbdd_batch* b, int64_t max_rounds) {
   b->h_params[0] = max_rounds;
-  for (auto& g : b->groups) CK(prepare_solver(g.C, g.elem, g.smem));
+  for (auto& g : b->groups) CK(prepare_solver(g.C, g.elem, g.smem, g.flags));
   if (b->exec) {
     CK(cudaGraphLaunch(b->exec, b->st));
     return LBDD_OK;
@@ -566,7 +568,7 @@ extern "C" int lbdd_autotune(lbdd_solver* const* solvers, int m, int probe_round
     double row[kNC] = {0, 0, 0, 0, 0};
     const int64_t rounds = tmp->n;
     for (int C = 1; C <= 16 && rc == LBDD_OK; C <<= 1) {
-      if (!fits_k(tmp->k, tmp->elem, C)) continue;
+      if (!solver_fits(tmp, C)) continue;
       float ms = 0;
       rc = lbdd_reset(tmp);
       if (!rc) rc = solve_timed(tmp, 0, C, &ms);          // prologue only

@@ -53,7 +53,9 @@ enum CtlIndex {
   CTL_COL_ROWS,        // member rows read by column-subset rescans
   CTL_FRONT_SUM,       // sum of Bellman-Ford frontier sizes over sweeps
   CTL_FRONT_HIST,      // 6 bins of frontier sizes: 1, 2-4, 5-16, 17-64, 65-256, >256
-  CTL_COUNT = CTL_FRONT_HIST + 6
+  CTL_POT = CTL_FRONT_HIST + 6,  // 1: the prices hold for the current table (guided rounds)
+  CTL_MIRROR,          // 1: the global mirror of T's costs is current (guided rounds)
+  CTL_COUNT
 };
 
 // Status codes shared with include/lbdd.h.
@@ -70,6 +72,7 @@ enum : int {
   OPT_NO_TC_SMEM = 4,     // keep the owned cost slice in global memory only
   OPT_PHASE_TIMERS = 8,   // time the phases of every round (CTA 0, thread 0)
   OPT_STRICT = 32,        // strict-LBDD (Alg. 5): vacancies as zero-cost dummy units
+  OPT_GUIDED = 64,        // one-CTA launch of the price-guided rounds (set by the host)
 };
 
 // Device view of one instance.  Pointers are device memory owned by the
@@ -93,6 +96,8 @@ struct DevInst {
   int32_t* free_stack;  // pages
   int32_t* tc;          // k x k best-transfer cost (row u = from u)
   int32_t* td;          // k x k best-transfer unit
+  int32_t* pot;         // k: prices of the centers (guided rounds)
+  void* mirror;         // k x guided_stride: T's costs in the CM's type (guided rounds), or null
   int64_t* ctl;         // CTL_COUNT
   int32_t max_pages;    // per center
   int32_t npages;       // in the pool

@@ -14,8 +14,12 @@ namespace lbdd {
 // asral_solver.cu
 size_t solver_smem_bytes(int32_t k, int C, int elem_bytes, bool with_slice);
 int solver_max_k(int C, int elem_bytes);
-int solver_max_clusters(int C, int elem_bytes, size_t smem);
-cudaError_t prepare_solver(int C, int elem_bytes, size_t smem);
+size_t guided_smem_bytes(int32_t k, int elem_bytes, size_t limit);
+size_t guided_mirror_bytes(int32_t k, int elem_bytes);
+int32_t guided_pen_limit();
+// flags: OPT_GUIDED selects the one-CTA guided kernel (C is then 1).
+int solver_max_clusters(int C, int elem_bytes, size_t smem, int flags = 0);
+cudaError_t prepare_solver(int C, int elem_bytes, size_t smem, int flags = 0);
 cudaError_t launch_solver(const DevInst* d_insts, int ninst, int* d_counter, int C,
                           int nclusters, int elem_bytes, size_t smem, int flags,
                           cudaStream_t st, uint64_t quantum_ns = 0, bool set_attrs = true);
@@ -40,7 +44,8 @@ struct lbdd_solver {
   int32_t *cap = nullptr, *pen = nullptr, *smin = nullptr, *order = nullptr,
           *sort_tmp = nullptr, *assign = nullptr, *pos = nullptr, *load = nullptr,
           *seg_size = nullptr, *page_tab = nullptr, *pool = nullptr, *free_stack = nullptr,
-          *tc = nullptr, *td = nullptr, *counter = nullptr;
+          *tc = nullptr, *td = nullptr, *pot = nullptr, *counter = nullptr;
+  void* mirror = nullptr;
   int64_t* ctl = nullptr;
   lbdd::DevInst* d_inst = nullptr;
   lbdd::DevInst h_inst;
@@ -54,6 +59,7 @@ struct lbdd_solver {
   int device = 0;
   int num_sms = 0;
   int32_t n_cap = 0;       // units the unit-indexed arrays and the page pool hold (>= n)
+  int32_t max_pen = 0;     // largest penalty (guided rounds need it below guided_pen_limit())
   int in_batches = 0;      // batches that hold a copy of this solver's device view
   int32_t* ins_row = nullptr;  // k costs of a unit being inserted (device staging)
   size_t bytes = 0;        // device bytes held now
@@ -73,6 +79,14 @@ bool fits_k(int32_t k, int elem, int C);
 // Latency-oriented default cluster size of one solver (largest that fits).
 int choose_cluster(lbdd_solver* s);
 int solver_flags(const lbdd_solver* s);
+// Whether s's next rounds on C-CTA clusters run guided (one CTA, both
+// shortcuts on, not strict, the guided layout fits).
+bool solver_guided(const lbdd_solver* s, int C);
+// Whether s runs on C-CTA clusters, guided or not.
+bool solver_fits(const lbdd_solver* s, int C);
+// Launch flags and dynamic shared memory of s's rounds on C-CTA clusters.
+int launch_flags(const lbdd_solver* s, int C);
+size_t launch_smem_of(const lbdd_solver* s, int C);
 int status_to_rc(int64_t st);
 // Device bytes lbdd_create allocates for an n x k instance whose costs are
 // stored with elem-byte entries (in_elem: entry size of the caller's CM,
