@@ -112,7 +112,9 @@ __host__ __device__ inline GLayout make_guided_layout(int32_t k, int32_t elem) {
   return L;
 }
 
-// Frontier entry: label and byte offset of the node's row of costs.
+// Frontier entry: label and byte offset of the node's row of costs (top bit:
+// a strict instance's center with a vacancy).
+constexpr uint32_t kGVacant = 0x80000000u;
 template <typename LT> struct GEnt;
 template <> struct __align__(8) GEnt<int32_t> { int32_t l; uint32_t off; };
 template <> struct __align__(16) GEnt<int64_t> { int64_t l; uint32_t off, pad; };
@@ -130,7 +132,7 @@ struct GMisc {
   int32_t naff, len, bad, stop;
 };
 
-template <typename T, bool TSM>
+template <typename T, bool TSM, bool STRICT>
 struct Guided {
   using LT = typename Solver<T>::LT;
   using Ent = GEnt<LT>;
@@ -204,6 +206,14 @@ struct Guided {
   __device__ __forceinline__ const T* row(int32_t d) const { return cm + (int64_t)d * ld; }
   __device__ __forceinline__ int32_t edge(int32_t u, int cl) const {
     return (int32_t)tt[(int64_t)u * ws + cl];
+  }
+  // Cost of the edge u -> column cl in the graph of Alg. 1; in a strict
+  // instance a center with a vacancy passes a dummy unit on for nothing
+  // (Alg. 5), members or not.
+  __device__ __forceinline__ bool vacant(int32_t u) const { return STRICT && s_slack[u] < 0; }
+  __device__ __forceinline__ int32_t arc(int32_t u, int cl) const {
+    const int32_t t = edge(u, cl);
+    return vacant(u) ? min(t, 0) : t;
   }
   __device__ __forceinline__ void set_entry(int32_t u, int cl, int32_t t, int32_t d) {
     tc[(int64_t)u * k + cl] = t;
@@ -329,7 +339,7 @@ struct Guided {
       M->cnt[1] = 0;
       Ent e;
       e.l = 0;
-      e.off = tbase + (uint32_t)j * rowb;
+      e.off = (tbase + (uint32_t)j * rowb) | (vacant(j) ? kGVacant : 0u);
       s_list[0] = e;
     }
     __syncthreads();
@@ -360,7 +370,7 @@ struct Guided {
             b = cl < k ? lab[cl] : kFixed;
             qv = real ? s_qn[cl] : kGNever;
             // a center without members has no edges (its row is infinite)
-            pv = real && s_seg[cl] > 0 ? price[cl] : kGNever;
+            pv = real && (s_seg[cl] > 0 || vacant(cl)) ? price[cl] : kGNever;
           }
           const LT old = b;
           const uint32_t colb = (uint32_t)min(cl, k - 1) * (uint32_t)sizeof(T);
@@ -372,7 +382,10 @@ struct Guided {
             for (int q = 0; q < U; ++q)   // past the end: the last node again
               e[q] = entry(in + (uint32_t)min(f + q, m - 1) * (uint32_t)sizeof(Ent));
 #pragma unroll
-            for (int q = 0; q < U; ++q) t[q] = cost_at(e[q].off + colb);
+            for (int q = 0; q < U; ++q) {
+              t[q] = cost_at((STRICT ? e[q].off & ~kGVacant : e[q].off) + colb);
+              if (STRICT && (e[q].off & kGVacant)) t[q] = min(t[q], 0);
+            }
 #pragma unroll
             for (int q = 0; q < U; q += 2) {
               b = relax(e[q].l, t[q], b);
@@ -398,7 +411,7 @@ struct Guided {
             const int at = nthr == 32 ? __popc(bits & ((1u << lane) - 1u)) : atomicAdd(&M->cnt[c3], 1);
             Ent ne;
             ne.l = b;
-            ne.off = tbase + (uint32_t)cl * rowb;
+            ne.off = (tbase + (uint32_t)cl * rowb) | (vacant(cl) ? kGVacant : 0u);
             out[at] = ne;
           }
         }
@@ -457,7 +470,7 @@ struct Guided {
       uint32_t* slot = &M->next[h % 3];
       for (int u = tid; u < k; u += kThreads)
         if (s_hop[u] == h - 1 && u != j && u != v && lab[u] != kNoLab &&
-            lab[u] + (LT)edge(u, v) == l) {
+            lab[u] + (LT)arc(u, v) == l) {
           atomicMin(slot, (uint32_t)u);
           break;
         }
@@ -470,7 +483,7 @@ struct Guided {
       if (tid == 0) s_pathu[m] = v;
       ++m;
     }
-    if (l != (LT)edge(j, v)) return -1;
+    if (l != (LT)arc(j, v)) return -1;
     if (tid == 0) s_pathu[m] = j;
     return m + 1 < 2 ? -1 : m + 1;
   }
@@ -496,8 +509,10 @@ struct Guided {
       __syncwarp();
       for (int i = lane; i < m; i += 32) {
         const int32_t to = (i + 1 < m) ? s_path[i + 1] : (npath ? -1 : j);
-        int32_t x = to >= 0 ? __ldcg(td + (int64_t)s_path[i] * k + to) : -1;
-        if (to >= 0 && (uint32_t)x >= (uint32_t)n) { x = -1; B->err0 = ST_ERR_INVARIANT; }
+        // a dummy unit moves where the edge's cost came from a vacancy
+        const bool dummy = STRICT && vacant(s_path[i]) && edge(s_path[i], to) > 0;
+        int32_t x = to >= 0 && !dummy ? __ldcg(td + (int64_t)s_path[i] * k + to) : -1;
+        if (to >= 0 && !dummy && (uint32_t)x >= (uint32_t)n) { x = -1; B->err0 = ST_ERR_INVARIANT; }
         s_pathu[i] = x;
         s_raff[i] = 0;
       }
@@ -542,13 +557,13 @@ struct Guided {
       }
       if (b == 0) pos0 = __shfl_sync(0xffffffffu, at, 0);
       if (m - 1 >= b && m - 1 < b + 32) ownl = __shfl_sync(0xffffffffu, own, m - 1 - b);
+      if (i < m) s_mid[i] = at;
       __syncwarp();   // every position of this batch is read before any is replaced
       if (x_out >= 0 && x_in >= 0) {
         if (at >= 0 && at < s_seg[c]) {
           int32_t* slot = mslot(c, at, s_seg[c]);
           slot[0] = x_in;
           slot[kPage] = own;
-          s_mid[i] = at;      // x_in's new position, stored below
         } else {
           s_mid[i] = -1;
           B->err0 = ST_ERR_INVARIANT;
@@ -561,6 +576,20 @@ struct Guided {
       if (s_pathu[i] >= 0 && x_in >= 0 && s_mid[i] >= 0) pos[x_in] = s_mid[i];
     }
     __syncwarp();
+    if (STRICT && lane == 0) {
+      // centers that only lose or only gain a real unit: a dummy is on the
+      // other side of their pair of edges
+      for (int i = 0; i < m; ++i) {
+        const int32_t c = s_path[i], x_out = s_pathu[i], x_in = arriving(npath, m, i);
+        if (x_out >= 0 && x_in < 0) {
+          list_remove_at(c, s_mid[i]);
+          shift_load(c, -1);
+        } else if (x_out < 0 && x_in >= 0) {
+          list_append(c, x_in, (int32_t)row(x_in)[c]);
+          shift_load(c, 1);
+        }
+      }
+    }
     if (lane == 0) {
       if (npath) {
         const int32_t term = s_path[m - 1];
@@ -744,9 +773,9 @@ struct Guided {
       const int i = it / kp, v = it % kp;
       const int32_t c = list[i];
       if (v < k && v != c) {
-        const int32_t t = edge(c, v);
+        const int32_t t = arc(c, v);
         if (t != kInf && (int64_t)s_pot[c] > (int64_t)t + s_pot[v]) bad = true;
-      } else if (v == c && s_pot[c] > s_qn[c]) {
+      } else if (v == c && !STRICT && s_pot[c] > s_qn[c]) {
         bad = true;
       }
     }
@@ -757,14 +786,18 @@ struct Guided {
   // holds (reverse Bellman-Ford; exact distances to a paid slot).
   __device__ bool rebuild_prices() {
     const int lane = tid & 31, warp = tid >> 5;
-    for (int v = tid; v < k; v += kThreads) s_pot[v] = s_qn[v];
+    bool room = false;
+    for (int v = tid; v < k; v += kThreads) room |= vacant(v);
+    room = __syncthreads_or(room) != 0;
+    for (int v = tid; v < k; v += kThreads)
+      s_pot[v] = !STRICT ? s_qn[v] : room && !vacant(v) ? kGPenLimit - 1 : 0;
     __syncthreads();
     for (int sweep = 0; sweep <= k + 1; ++sweep) {
       bool any = false;
       for (int u = warp; u < k; u += kWarps) {
         int64_t best = INT64_MAX;
         for (int v = lane; v < k; v += 32) {
-          const int32_t t = v != u ? edge(u, v) : kInf;
+          const int32_t t = v != u ? arc(u, v) : kInf;
           if (t != kInf) best = min(best, (int64_t)t + s_pot[v]);
         }
         for (int off = 16; off > 0; off >>= 1)
@@ -784,7 +817,7 @@ struct Guided {
   // ----------------------------------------------------------- the loop --
   __device__ __forceinline__ void load_order(int64_t r, int64_t r_end, int slot) {
     const int32_t d = r < r_end ? I.order[r] : -1;
-    const int32_t j = (uint32_t)d < (uint32_t)n ? I.smin[d] : -1;
+    const int32_t j = !STRICT && (uint32_t)d < (uint32_t)n ? I.smin[d] : -1;
     s_ord[2 * slot] = d;
     s_ord[2 * slot + 1] = (uint32_t)j < (uint32_t)k ? j : -1;
   }
@@ -800,6 +833,26 @@ struct Guided {
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+
+  // Alg. 5: the cheapest center with a vacancy, lowest index on equal cost
+  // (-1: none).  Every thread calls it; the row is in shared memory.
+  __device__ int32_t strict_target(const T* r) {
+    int32_t bv = INT32_MAX, bj = INT32_MAX;
+    for (int v = tid; v < k; v += kThreads)
+      if (vacant(v) && (int32_t)r[v] < bv) { bv = (int32_t)r[v]; bj = v; }
+    const int32_t wv = __reduce_min_sync(0xffffffffu, bv);
+    const int32_t wj = __reduce_min_sync(0xffffffffu, bv == wv ? bj : INT32_MAX);
+    if ((tid & 31) == 0) {
+      s_aff[2 * (tid >> 5)] = wv;
+      s_aff[2 * (tid >> 5) + 1] = wj;
+    }
+    __syncthreads();
+    bv = (tid & 31) < kWarps ? s_aff[2 * (tid & 31)] : INT32_MAX;
+    bj = (tid & 31) < kWarps ? s_aff[2 * (tid & 31) + 1] : INT32_MAX;
+    const int32_t mv = __reduce_min_sync(0xffffffffu, bv);
+    const int32_t mj = __reduce_min_sync(0xffffffffu, bv == mv ? bj : INT32_MAX);
+    return mj == INT32_MAX ? -1 : mj;
   }
 
   __device__ void run_rounds(uint64_t deadline) {
@@ -860,15 +913,20 @@ struct Guided {
         const int32_t at = q + 32 + (tid & 31);
         load_order(r_begin + at, r_end, at & (kGOrd - 1));
       }
-      const int32_t d = s_ord[2 * (q & (kGOrd - 1))], j = s_ord[2 * (q & (kGOrd - 1)) + 1];
-      if (d < 0 || j < 0) { status = ST_ERR_INVARIANT; break; }   // uniform guard
+      const int32_t d = s_ord[2 * (q & (kGOrd - 1))];
+      int32_t j = s_ord[2 * (q & (kGOrd - 1)) + 1];
+      if (d < 0 || (!STRICT && j < 0)) { status = ST_ERR_INVARIANT; break; }   // uniform guard
       if (nring == 8) asm volatile("cp.async.wait_group 7;" ::: "memory");
       else asm volatile("cp.async.wait_group 3;" ::: "memory");
       __syncthreads();
       // Alg. 2, allotment: d joins j; its edges enter row j of T
       const T* r = reinterpret_cast<const T*>(s_ring + (uint32_t)(q & (nring - 1)) * ring_row);
+      if (STRICT) {
+        j = strict_target(r);
+        if (j < 0) { status = ST_ERR_INVARIANT; break; }
+      }
       const int32_t own = (int32_t)r[j];
-      const bool over = s_slack[j] >= 0;
+      const bool over = !STRICT && s_slack[j] >= 0;
       const int32_t ql = over ? s_pen[j] : 0;   // q_j(load - cap + 1), paid by d
       const int32_t pj = s_pot[j];
       bool viol = false;
@@ -897,6 +955,7 @@ struct Guided {
         if (!over || pj >= ql) continue;
       }
       // Alg. 1 and Alg. 4 at j
+      if (STRICT) __syncthreads();   // j's vacancy counts the allotment
       const uint64_t ts0 = timer() ? clock_cycles() : 0;
       search(j, viol, over, s_lab1, s_pot, ql);
       if (timer()) B->t_relax += clock_cycles() - ts0;
@@ -906,7 +965,7 @@ struct Guided {
       const int64_t D1 = over ? (int64_t)M->paid : INT32_MAX;   // exact below ql
       bool bad = false;
       if (cycv >= 0) {
-        const int64_t dd = min(D1, (int64_t)ql);
+        const int64_t dd = over ? min(D1, (int64_t)ql) : (int64_t)pj;
         for (int v = tid; v < k; v += kThreads) {
           if (v == j) s_pot[v] = (int32_t)max((int64_t)pj, dd);
           else if (s_lab1[v] != kNoLab) s_pot[v] = (int32_t)max((int64_t)s_pot[v], dd - (int64_t)s_lab1[v]);
@@ -939,8 +998,8 @@ struct Guided {
           d2 = min((int64_t)ql, D2);
         }
         const uint32_t sink2 = M->sink;
-        const int64_t dd = over ? cycv + d2 : min(D1, cycv);
-        if (!over) d2 = dd - cycv;
+        if (!over) d2 = pj;
+        const int64_t dd = cycv + d2;
         for (int v = tid; v < k; v += kThreads) {
           int64_t p = s_pot[v];
           if (v == j) {

@@ -1563,7 +1563,9 @@ asral_cluster_kernel(const DevInst* __restrict__ insts, int ninst, int* work_cou
 
 namespace lbdd {
 
-// Instances of a launch solved one per CTA with the guided rounds.
+// The guided rounds.  CTA 0 of every cluster runs them; the others share the
+// prologue (a scan of every row of CM), which is all there is to share: a
+// round's frontier is a dozen labels.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 1)
 asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_counter, int flags,
@@ -1571,13 +1573,14 @@ asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_coun
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ DevInst s_inst;
   __shared__ Book s_book;
-  __shared__ int s_item;
+  __shared__ int32_t s_item;
   __shared__ uint64_t s_deadline;
   const int tid = threadIdx.x;
+  const int rank = (int)cluster_rank(), C = (int)cluster_nrank();
   if (tid == 0) s_deadline = quantum_ns ? gtimer_ns() + quantum_ns : 0;
   const uint32_t avail = dyn_smem_bytes();
   for (;;) {
-    if (tid == 0) {   // next instance with rounds left and no error
+    if (rank == 0 && tid == 0) {   // next instance with rounds left and no error
       int it = ninst;
       if (!s_deadline || gtimer_ns() < s_deadline) {
         for (;;) {
@@ -1591,44 +1594,53 @@ asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_coun
         }
       }
       s_item = it;
-      if (it < ninst) s_inst = insts[it];
     }
     __syncthreads();
-    if (s_item >= ninst) break;
+    cluster_sync_all();
+    const int item = C == 1 ? s_item : dsmem_ld32(dsmem_addr(&s_item, 0));
+    if (C > 1) cluster_sync_all();   // read before CTA 0 takes the next one
+    if (item >= ninst) break;
+    if (tid == 0) s_inst = insts[item];
+    __syncthreads();
     const GLayout L = make_guided_layout(s_inst.k, (int)sizeof(T));
-    if (s_inst.ctl[CTL_PROLOGUE] == 0) {
+    if (__ldcg(s_inst.ctl + CTL_PROLOGUE) == 0) {
       const uint64_t t0 = gtimer_ns();
       Solver<T> S(s_inst);
       S.B = &s_book;
       S.tid = tid;
-      S.rank = 0;
-      S.C = 1;
+      S.rank = rank;
+      S.C = C;
       S.flags = flags;
       S.cm = static_cast<const T*>(s_inst.cm);
       S.n = s_inst.n;
       S.k = s_inst.k;
-      S.w = own_width(S.k, 1, Solver<T>::VPL);
-      S.c0 = 0;
-      S.c1 = S.wr = S.k;
+      S.w = own_width(S.k, C, Solver<T>::VPL);
+      S.c0 = rank * S.w;
+      S.c1 = min(S.k, S.c0 + S.w);
+      S.wr = max(0, S.c1 - S.c0);
       S.s_red = smem + L.ring;
-      S.prologue();
-      for (int v = tid; v < s_inst.k; v += kThreads) s_inst.pot[v] = 0;
-      if (tid == 0) {
+      S.prologue();   // every CTA has read CTL_PROLOGUE by its cluster barriers
+      for (int v = tid; v < s_inst.k && rank == 0; v += kThreads) s_inst.pot[v] = 0;
+      if (rank == 0 && tid == 0) {
         s_inst.ctl[CTL_FREE_TOP] = s_inst.npages;
         s_inst.ctl[CTL_ROUNDS] = 0;
         s_inst.ctl[CTL_DELTA] = 0;
         s_inst.ctl[CTL_POT] = 1;
+        s_inst.ctl[CTL_MIRROR] = 0;
         s_inst.ctl[CTL_PROLOGUE] = 1;
         s_inst.ctl[CTL_T_PROLOGUE] += gtimer_ns() - t0;
       }
       __syncthreads();
     }
-    if (L.total <= avail && !(flags & OPT_NO_TC_SMEM)) {
-      Guided<T, true> G(s_inst, smem, L, &s_book, flags);
-      G.run_rounds(s_deadline);
+    if (rank != 0) continue;   // waits at the next instance's barrier
+    const bool tsm = L.total <= avail && !(flags & OPT_NO_TC_SMEM);
+    auto rounds = [&](auto G) { G.run_rounds(s_deadline); };
+    if (flags & OPT_STRICT) {
+      if (tsm) rounds(Guided<T, true, true>(s_inst, smem, L, &s_book, flags));
+      else rounds(Guided<T, false, true>(s_inst, smem, L, &s_book, flags));
     } else {
-      Guided<T, false> G(s_inst, smem, L, &s_book, flags);
-      G.run_rounds(s_deadline);
+      if (tsm) rounds(Guided<T, true, false>(s_inst, smem, L, &s_book, flags));
+      else rounds(Guided<T, false, false>(s_inst, smem, L, &s_book, flags));
     }
   }
 }
@@ -1665,6 +1677,11 @@ template <typename T>
 cudaError_t prepare_solver_t(int C, size_t smem, int flags);
 
 template <typename T>
+static auto solver_kernel(int flags) {
+  return flags & OPT_GUIDED ? asral_guided_kernel<T> : asral_cluster_kernel<T>;
+}
+
+template <typename T>
 cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, int C,
                             int nclusters, size_t smem, int flags, cudaStream_t st,
                             uint64_t quantum_ns, bool set_attrs) {
@@ -1677,9 +1694,6 @@ cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, i
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  if (flags & OPT_GUIDED)   // no cluster: every CTA takes instances of its own
-    return cudaLaunchKernelEx(&cfg, asral_guided_kernel<T>, d_insts, ninst, d_counter, flags,
-                              quantum_ns);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)C;
@@ -1687,7 +1701,8 @@ cudaError_t launch_solver_t(const DevInst* d_insts, int ninst, int* d_counter, i
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, asral_cluster_kernel<T>, d_insts, ninst, d_counter, flags, quantum_ns);
+  return cudaLaunchKernelEx(&cfg, solver_kernel<T>(flags), d_insts, ninst, d_counter, flags,
+                            quantum_ns);
 }
 
 // Kernel attributes only ever grow (a launch needs at least its own dynamic
@@ -1698,32 +1713,24 @@ template <typename T>
 cudaError_t prepare_solver_t(int C, size_t smem, int flags) {
   constexpr int kDevs = 64;
   static std::mutex mu;
-  static size_t cur_smem[kDevs] = {}, cur_guided[kDevs] = {};
-  static bool non_portable[kDevs] = {};
+  static size_t cur_smem[2][kDevs] = {};      // [guided][device]
+  static bool non_portable[2][kDevs] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kDevs) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(mu);
-  if (flags & OPT_GUIDED) {
-    if (smem > cur_guided[dev]) {
-      e = cudaFuncSetAttribute(asral_guided_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
-      if (e != cudaSuccess) return e;
-      cur_guided[dev] = smem;
-    }
-    return cudaSuccess;
-  }
-  auto kern = asral_cluster_kernel<T>;
-  if (smem > cur_smem[dev]) {
+  auto kern = solver_kernel<T>(flags);
+  const int g = flags & OPT_GUIDED ? 1 : 0;
+  if (smem > cur_smem[g][dev]) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    cur_smem[dev] = smem;
+    cur_smem[g][dev] = smem;
   }
-  if (C > 8 && !non_portable[dev]) {
+  if (C > 8 && !non_portable[g][dev]) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    non_portable[dev] = true;
+    non_portable[g][dev] = true;
   }
   return cudaSuccess;
 }
@@ -1747,15 +1754,6 @@ cudaError_t launch_solver(const DevInst* d_insts, int ninst, int* d_counter, int
 template <typename T>
 static int max_clusters_t(int C, size_t smem, int flags) {
   if (prepare_solver_t<T>(C, smem, flags) != cudaSuccess) return -1;
-  if (flags & OPT_GUIDED) {
-    int per_sm = 0, dev = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, asral_guided_kernel<T>, kThreads,
-                                                      smem) != cudaSuccess ||
-        cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return -1;
-    return per_sm * sms;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)C, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -1767,9 +1765,8 @@ static int max_clusters_t(int C, size_t smem, int flags) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  auto kern = asral_cluster_kernel<T>;
   int num = 0;
-  return cudaOccupancyMaxActiveClusters(&num, kern, &cfg) == cudaSuccess ? num : -1;
+  return cudaOccupancyMaxActiveClusters(&num, solver_kernel<T>(flags), &cfg) == cudaSuccess ? num : -1;
 }
 
 int solver_max_clusters(int C, int elem_bytes, size_t smem, int flags) {

@@ -145,6 +145,7 @@ static int ingest_cm(lbdd_solver* s, const void* cm, int dtype, int is_device, i
   s->cm = store;
   s->ld = ld;
   s->elem = in_elem;
+  s->max_cost = res[1];
   if (in_elem == 4 && res[1] <= INT16_MAX) {
     const int64_t ld16 = lbdd_cm_pitch(k, LBDD_CM_I16);
     void* narrow = nullptr;
@@ -507,9 +508,12 @@ int lbdd::solver_flags(const lbdd_solver* s) {
 }
 
 bool lbdd::solver_guided(const lbdd_solver* s, int C) {
-  return C == 1 && s->ncyc_skip && s->npath_reuse && !s->strict && s->mirror &&
-         s->max_pen < guided_pen_limit() &&
-         guided_smem_bytes(s->k, s->elem, kMaxSmem) > 0;
+  if (!s->ncyc_skip || !s->npath_reuse || !s->mirror || s->max_pen >= guided_pen_limit() ||
+      guided_smem_bytes(s->k, s->elem, kMaxSmem) == 0)
+    return false;
+  // strict prices are bounded by the costs
+  if (s->strict && s->elem == 4 && s->max_cost >= guided_pen_limit()) return false;
+  return C == 1 || fits_k(s->k, s->elem, C);
 }
 
 bool lbdd::solver_fits(const lbdd_solver* s, int C) {

@@ -17,7 +17,7 @@ int solver_max_k(int C, int elem_bytes);
 size_t guided_smem_bytes(int32_t k, int elem_bytes, size_t limit);
 size_t guided_mirror_bytes(int32_t k, int elem_bytes);
 int32_t guided_pen_limit();
-// flags: OPT_GUIDED selects the one-CTA guided kernel (C is then 1).
+// flags: OPT_GUIDED selects the guided kernel.
 int solver_max_clusters(int C, int elem_bytes, size_t smem, int flags = 0);
 cudaError_t prepare_solver(int C, int elem_bytes, size_t smem, int flags = 0);
 cudaError_t launch_solver(const DevInst* d_insts, int ninst, int* d_counter, int C,
@@ -59,6 +59,7 @@ struct lbdd_solver {
   int device = 0;
   int num_sms = 0;
   int32_t n_cap = 0;       // units the unit-indexed arrays and the page pool hold (>= n)
+  int32_t max_cost = 0;    // largest cost at creation
   int32_t max_pen = 0;     // largest penalty (guided rounds need it below guided_pen_limit())
   int in_batches = 0;      // batches that hold a copy of this solver's device view
   int32_t* ins_row = nullptr;  // k costs of a unit being inserted (device staging)
@@ -79,8 +80,8 @@ bool fits_k(int32_t k, int elem, int C);
 // Latency-oriented default cluster size of one solver (largest that fits).
 int choose_cluster(lbdd_solver* s);
 int solver_flags(const lbdd_solver* s);
-// Whether s's next rounds on C-CTA clusters run guided (one CTA, both
-// shortcuts on, not strict, the guided layout fits).
+// Whether s's next rounds on C-CTA clusters run guided (both shortcuts on,
+// penalties and the layout within the guided limits).
 bool solver_guided(const lbdd_solver* s, int C);
 // Whether s runs on C-CTA clusters, guided or not.
 bool solver_fits(const lbdd_solver* s, int C);
