@@ -22,19 +22,20 @@
 //   5. the scan: CM rows are streamed and every 16-byte column group keeps a
 //      running lexicographic minimum; at the end of an item (or of a CTA's
 //      share of one) the partial minima are folded in shared memory and
-//      merged into a packed (cost, d) 64-bit table with atomicMin.  Rows of
-//      512 bytes and more: bt_scan_bulk, every CTA an equal contiguous share
-//      of the grouped rows, staged whole by bulk copies; shorter rows:
-//      bt_scan_rows, items from a queue, 16 bytes per thread and load;
+//      merged into a packed (cost, d) 64-bit table with atomicMin
+//      (bt_scan_bulk: every CTA an equal contiguous share of the grouped
+//      rows, staged whole by bulk copies);
 //   6. bt_unpack: the (tc, td) int32 pair.
 // Step 5 reads every CM byte of the allotted rows once and is the HBM-bound
 // kernel; the other steps move O(n + k*k) bytes.
 //
 // Tables of 256 to 512 centers take a shorter path with no grouping (rows of
 // 512 bytes to 2 KB gather poorly): bt_own, then bt_scan_stream reads the CM
-// in row order, one 128-byte column slice and one row range per CTA, keeping
+// in row order, one narrow column slice and one row range per CTA, keeping
 // the minima in shared memory, and bt_merge_ranges combines the ranges into
-// (tc, td).
+// (tc, td).  Fewer than 256 centers: the whole table of a row range fits
+// shared memory, one kernel in row order and at most one merge
+// (bt_scan_table).
 #include <atomic>
 #include <algorithm>
 
@@ -45,13 +46,12 @@ namespace lbdd {
 constexpr int kChunkMax = 512;          // rows per work item, at most (16-bit row index)
 constexpr int kChunkMin = 64;           // rows per work item, at least (bounds the item count)
 constexpr int kItemsPerSm = 8;          // work items per SM the plan aims for
-constexpr int kScanUnroll = 6;          // bt_scan_rows: rows in flight per thread
 constexpr int kTiles = 64;              // unit ranges of bt_count / bt_place
 constexpr int kTileThreads = 1024;
 constexpr int kTileUnroll = 8;          // assign loads in flight per thread
 
-// ctl words (int32): error flag, scan queue, item count, chunk, allotted rows
-enum { BT_ERR = 0, BT_QUEUE, BT_ITEMS, BT_CHUNK, BT_ROWS, BT_CTL_WORDS = 8 };
+// ctl words (int32): error flag, item count, chunk, allotted rows
+enum { BT_ERR = 0, BT_ITEMS, BT_CHUNK, BT_ROWS, BT_CTL_WORDS = 8 };
 
 struct BtWorkspace {
   int* ctl;                     // BT_CTL_WORDS control words
@@ -99,9 +99,12 @@ static BtWorkspace carve(void* base, int32_t n, int32_t k) {
   return W;
 }
 
+static size_t table_part_bytes(int32_t n, int32_t k);
+
 size_t bt_workspace_bytes(int32_t n, int32_t k) {
   if (n < 1 || k < 1) return 0;
-  return carve(nullptr, n, k).bytes + 256;
+  // the packed tables of short rows take the place of everything else
+  return std::max(carve(nullptr, n, k).bytes, table_part_bytes(n, k)) + 256;
 }
 
 // ------------------------------------------------------------- grouping ---
@@ -170,7 +173,7 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t* s_wa
 
 // One CTA of kThreads: segment starts (exclusive prefix of the counts,
 // centers in index order) into cnt[0..k), the allotted total into cnt[k],
-// and the work items.  Clears the scan queue; records the item count, the
+// and the work items.  Records the item count, the
 // chunk and the allotted rows in ctl.
 __global__ void __launch_bounds__(kThreads) bt_plan(int32_t* cnt, int32_t k, int num_sms,
                                                     int4* items, int* ctl) {
@@ -198,7 +201,6 @@ __global__ void __launch_bounds__(kThreads) bt_plan(int32_t* cnt, int32_t k, int
   }
   if (tid == 0) {
     cnt[k] = total;
-    ctl[BT_QUEUE] = 0;
     ctl[BT_ITEMS] = nitems;
     ctl[BT_CHUNK] = chunk;
     ctl[BT_ROWS] = total;
@@ -282,125 +284,9 @@ __global__ void __launch_bounds__(kThreads) bt_sort_items(const int4* __restrict
 // positive int16).  The int32 scan keeps (t, row) pairs with a strict '<':
 // a thread sees the rows of an item in increasing order.
 
-// Rows shorter than 512 bytes: every thread loads its 16-byte column group
-// of kScanUnroll rows at once, and the unit ids of the next kScanUnroll rows
-// while those are reduced.
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 1)
-bt_scan_rows(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
-             const int32_t* __restrict__ perm, const int4* __restrict__ items,
-             unsigned long long* t64, int* ctl) {
-  constexpr int VPL = 16 / (int)sizeof(T);
-  constexpr int U = kScanUnroll;
-  __shared__ int2 red[kThreads * VPL];
-  __shared__ int s_item[2];
-  const int S = (k + VPL - 1) / VPL;       // 16-byte column groups per row
-  const int R = kThreads / S;              // row groups
-  const int tid = threadIdx.x, slot = tid % S, g = tid / S;
-  const int32_t total = ctl[BT_ITEMS];
-  int* work = ctl + BT_QUEUE;
-  // items come from a global queue: CTAs that finish early take more
-  if (tid == 0) s_item[0] = atomicAdd(work, 1);
-  __syncthreads();
-  for (int32_t item = s_item[0];;) {
-    if (item >= total) break;
-    const int4 desc = items[item];
-    // fetch the next item now; it is read after the reduction's barrier
-    if (tid == 0) s_item[1] = atomicAdd(work, 1);
-    const int32_t c = desc.x, r0 = desc.y, r1 = desc.y + desc.z;
-    int32_t bt[VPL], bd[VPL];
-#pragma unroll
-    for (int q = 0; q < VPL; ++q) { bt[q] = kTInf; bd[q] = -1; }
-    uint32_t key[VPL];
-#pragma unroll
-    for (int q = 0; q < VPL; ++q) key[q] = 0xffffffffu;
-    if (g < R) {
-      int32_t dn[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int32_t pu = r0 + g + u * R;
-        dn[u] = pu < r1 ? (int32_t)min((uint32_t)__ldg(perm + pu), (uint32_t)(n - 1)) : -1;
-      }
-      for (int32_t p = r0 + g; p < r1; p += U * R) {
-        int32_t d[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) d[u] = dn[u];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int32_t pu = p + (U + u) * R;
-          dn[u] = pu < r1 ? (int32_t)min((uint32_t)__ldg(perm + pu), (uint32_t)(n - 1)) : -1;
-        }
-        int32_t own[U];
-        Vec16<T> x[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          if (d[u] >= 0) {
-            const T* rp = cm + (int64_t)d[u] * ld;
-            own[u] = (int32_t)rp[c];
-            x[u] = load16(rp + slot * VPL);
-          }
-        }
-        if constexpr (sizeof(T) == 2) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            if (d[u] < 0) continue;
-            const uint32_t crow = ((uint32_t)(32768 - own[u]) << 16) | (uint32_t)(p + u * R - r0);
-            const uint4 wv = *reinterpret_cast<const uint4*>(&x[u]);
-            const uint32_t w4[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              key[2 * q] = min(key[2 * q], (w4[q] << 16) + crow);
-              key[2 * q + 1] = min(key[2 * q + 1], (w4[q] & 0xffff0000u) + crow);
-            }
-          }
-        } else {
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            if (d[u] < 0) continue;
-#pragma unroll
-            for (int q = 0; q < VPL; ++q) {
-              const int32_t t = (int32_t)x[u].v[q] - own[u];
-              if (t < bt[q]) { bt[q] = t; bd[q] = d[u]; }
-            }
-          }
-        }
-      }
-      if constexpr (sizeof(T) == 2) {
-#pragma unroll
-        for (int q = 0; q < VPL; ++q) {
-          if (key[q] != 0xffffffffu) {
-            bt[q] = (int32_t)(key[q] >> 16) - 32768;
-            bd[q] = (int32_t)min((uint32_t)__ldg(perm + r0 + (int32_t)(key[q] & 0xffffu)),
-                                 (uint32_t)(n - 1));
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < VPL; ++q) red[g * S * VPL + slot * VPL + q] = make_int2(bt[q], bd[q]);
-    }
-    __syncthreads();
-    for (int col = tid; col < k; col += kThreads) {
-      int32_t t = kTInf, dd = -1;
-      for (int gg = 0; gg < R; ++gg) {
-        const int2 e = red[gg * S * VPL + col];
-        if (lex_less(e.x, e.y, t, dd)) { t = e.x; dd = e.y; }
-      }
-      if (dd >= 0 && col != c) {
-        const unsigned long long pk =
-            ((unsigned long long)(uint32_t)(t + (int64_t)2147483648LL) << 32) | (uint32_t)dd;
-        atomicMin(&t64[(int64_t)c * k + col], pk);
-      }
-    }
-    item = s_item[1];
-    __syncthreads();
-    if (tid == 0) s_item[0] = item;   // keep s_item[1] free for the next fetch
-  }
-}
-
-
 // ---------------------------------------------------- bulk-copy row scan ---
 //
-// Rows of kBulkMinRowBytes and more.  CTA b scans the grouped rows
+// CTA b scans the grouped rows
 // [b * rows / G, (b + 1) * rows / G) of perm: equal bytes per CTA, no work
 // queue.  Warp kWarps (the producer) walks that range: the segment starts
 // (all k + 1 of them, copied into shared memory at start) give the center
@@ -417,7 +303,6 @@ bt_scan_rows(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
 // bounded: past kScanWaitLimitNs the waiter sets ctl[BT_ERR] and leaves (the
 // producer first waits, bounded, for its copies in flight), and bt_unpack
 // then marks the whole table.
-constexpr int kBulkMinRowBytes = 512;
 constexpr int kStageBytes = 32768;       // target bytes per stage (the producer's cost is per stage)
 constexpr int kSmemLimit = 232448;       // dynamic shared memory of one CTA (227 KB)
 constexpr int kMaxStages = 16;
@@ -733,24 +618,30 @@ __global__ void __launch_bounds__(kThreads) bt_unpack(const unsigned long long* 
 //
 // Rows of kStreamMinK..kStreamMaxK centers (512 bytes to 2 KB) are short for
 // row gathers, so this path reads the CM in row order instead and needs no
-// grouping.  CTA (j, r) owns the 128-byte column slice j (64 int16 or 32 int32
-// columns) and the row range r, and keeps in shared memory one key per
+// grouping.  CTA (j, r) owns the column slice j (32 columns: 64 bytes of int16,
+// 128 of int32 costs) and the row range r, and keeps in shared memory one key per
 // (center, column of the slice): ((t + 32768) << 16) | (d - first row of the
 // range) in 32 bits for int16, ((t + 2^31) << 32) | (d - first row) in 64
 // bits for int32, so the smaller key is the lexicographically smaller (t, d)
 // inside the range.  A thread
-// owns 16 bytes (8 columns) of every 128th row; each is copied into the
+// owns 16 bytes of every 256th (128th) row; each is copied into the
 // thread's own shared slot by cp.async kStreamStages rows ahead (the bytes in
 // flight are bounded by shared memory, not registers), then the thread
 // compares its keys with the table and lowers an entry with a shared atomicMin only where its
 // key is smaller (entries only decrease, so a stale read never hides a
-// smaller key).  A table row (256 bytes) is laid out as two halves: the
-// first half of every thread's keys in the first 128 bytes, the other half in
-// the second, so each 128-bit shared load of 8 threads covers 32 banks.  bt_own gathers
-// CM(d, assign[d]) first; bt_merge_ranges takes, for every (u, v), the
+// smaller key).  A table row is laid out as two halves: the first half of
+// every thread's keys, then the other half, so that the 128-bit shared loads
+// of 8 threads cover 32 banks.  bt_own gathers CM(d, assign[d]) first (int16:
+// together with the center, in one word); bt_merge_ranges takes, for every (u, v), the
 // smallest t over the ranges in range order (ranges ascend in d, so the first
 // range that attains it holds the smallest d) and writes tc/td.
-constexpr int kStreamThreads = 1024;    // 8 threads per 128-byte row slice, 128 rows at a time
+//
+// What bounds it is shared memory (staging, table reads and minima take about
+// 40 cycles of its pipe per 512 bytes), then the partial tables.  Slices of
+// 64 bytes instead of 128 with int16 costs halve the ranges, their tables and
+// the share of keys that lower an entry: 200,000 x 500 int16 64.0 -> 62.1 us
+// per call.
+constexpr int kStreamThreads = 1024;    // 4 or 8 threads per row slice, 256 or 128 rows at a time
 constexpr int kStreamStages = 5;        // rows in flight per thread (cp.async stages)
 
 __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
@@ -761,18 +652,36 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Per cost type: columns per slice (128 bytes of a row), the key, and the
-// key's split into cost and row offset.  A key row is 256 bytes either way.
+// Shared minimum at address `at`, where `key` is smaller than `cur`: one
+// predicated reduction instead of a branch around an atomic.
+__device__ __forceinline__ void red_min_if_less(uint32_t at, uint32_t key, uint32_t cur) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p red.shared.min.u32 [%0], %1;\n\t}"
+               ::"r"(at), "r"(key), "r"(cur) : "memory");
+}
+// The same for a signed minimum; also voids the word at `unit`.
+__device__ __forceinline__ void red_min_void_if_less(uint32_t at, int32_t t, int32_t cur,
+                                                     uint32_t unit) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %1, %2;\n\t@p red.shared.min.s32 [%0], %1;\n\t"
+      "@p st.shared.u32 [%3], %4;\n\t}" ::"r"(at), "r"(t), "r"(cur), "r"(unit), "r"(~0u) : "memory");
+}
+__device__ __forceinline__ void red_min_if_equal(uint32_t at, uint32_t d, int32_t t, int32_t cur) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %2, %3;\n\t@p red.shared.min.u32 [%0], %1;\n\t}"
+               ::"r"(at), "r"(d), "r"(t), "r"(cur) : "memory");
+}
+
+// Per cost type: columns per slice, the key, and the key's split into cost
+// and row offset.
 template <typename T> struct StreamKey;
 template <> struct StreamKey<int16_t> {
   using K = uint32_t;                    // ((t + 32768) << 16) | row offset
-  static constexpr int kCols = 64;
+  static constexpr int kCols = 32;       // 64 bytes of a row
   static __device__ __forceinline__ int32_t cost(K key) { return (int32_t)(key >> 16) - 32768; }
   static __device__ __forceinline__ uint32_t offset(K key) { return key & 0xffffu; }
 };
 template <> struct StreamKey<int32_t> {
   using K = unsigned long long;          // ((t + 2^31) << 32) | row offset
-  static constexpr int kCols = 32;
+  static constexpr int kCols = 32;       // 128 bytes of a row
   static __device__ __forceinline__ int32_t cost(K key) {
     return (int32_t)((int64_t)(key >> 32) - 2147483648LL);
   }
@@ -787,8 +696,10 @@ __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontro
 __device__ __forceinline__ void release_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Dynamic shared memory of bt_scan_stream: the key table, then the stages.
+template <typename T>
 static size_t stream_smem_bytes(int32_t k) {
-  return 256 * (size_t)k + (size_t)kStreamStages * kStreamThreads * 16;
+  return (size_t)StreamKey<T>::kCols * sizeof(typename StreamKey<T>::K) * (size_t)k +
+         (size_t)kStreamStages * kStreamThreads * 16;
 }
 
 // Row ranges of the row-order path on `num_sms` SMs, 0 if it does not apply.
@@ -814,7 +725,10 @@ __global__ void __launch_bounds__(kThreads) bt_own(const int32_t* __restrict__ a
   for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * kThreads) {
     const int32_t a = assign[i];
-    own[i] = (a >= 0 && a < k) ? (int32_t)cm[i * ld + a] : 0;
+    if constexpr (sizeof(T) == 2)   // center + 1 and own cost in one word, 0 = no center
+      own[i] = (a >= 0 && a < k) ? ((a + 1) << 16) | (uint16_t)cm[i * ld + a] : 0;
+    else
+      own[i] = (a >= 0 && a < k) ? (int32_t)cm[i * ld + a] : 0;
   }
 }
 
@@ -830,46 +744,61 @@ bt_scan_stream(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
   constexpr int P = kStreamStages;
   extern __shared__ __align__(16) unsigned char stream_smem[];
   K* acc = reinterpret_cast<K*>(stream_smem);   // k rows of COLS keys, then the stages
-  const int tid = threadIdx.x, cg = tid & 7, rl = tid >> 3;
+  constexpr int TPR = COLS / VPL;              // threads per row slice
+  constexpr int RPS = kStreamThreads / TPR;    // rows at a time
+  constexpr int KB = COLS * (int)sizeof(K);    // bytes of a key row
+  const int tid = threadIdx.x, cg = tid % TPR, rl = tid / TPR;
   const int j = blockIdx.x % nslice, r = blockIdx.x / nslice;
   const int64_t R0 = (int64_t)r * n / nranges, R1 = (int64_t)(r + 1) * n / nranges;
   const int c0 = j * COLS;
   const int w = min(COLS, k - c0);
   const bool act = cg * VPL < w;
   const uint4 none = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
-  for (int i = tid; i < k * 16; i += kStreamThreads) reinterpret_cast<uint4*>(acc)[i] = none;
+  for (int i = tid; i < k * (KB / 16); i += kStreamThreads) reinterpret_cast<uint4*>(acc)[i] = none;
   __syncthreads();
   wait_predecessor();   // own[] comes from bt_own
   const T* colp = cm + c0 + cg * VPL;
-  // rows of this thread: R0 + rl + 128 i, i < M; row i's 16 bytes go to
+  // rows of this thread: R0 + rl + RPS i, i < M; row i's 16 bytes go to
   // stage i % P of the thread's own shared slots P rows ahead (cp.async: a
   // thread waits only for its own copies, no barrier), its center and own
   // cost to a register ring P rows ahead
   const int64_t span = R1 - R0;
-  const int32_t M = act && rl < span ? (int32_t)((span - rl + 127) / 128) : 0;
-  uint4* stage = reinterpret_cast<uint4*>(stream_smem + 256 * (size_t)k);   // [P][kStreamThreads]
+  const int32_t M = act && rl < span ? (int32_t)((span - rl + RPS - 1) / RPS) : 0;
+  uint4* stage = reinterpret_cast<uint4*>(stream_smem + KB * (size_t)k);   // [P][kStreamThreads]
+  // int16: one word per row holds both (bt_own)
+  constexpr bool kPacked = sizeof(T) == 2;
   int32_t ra[P], ro[P];
 #pragma unroll
   for (int q = 0; q < P; ++q) {
-    const int64_t d = R0 + rl + 128 * q;
-    ra[q] = -1;
+    const int64_t d = R0 + rl + RPS * q;
+    ra[q] = kPacked ? 0 : -1;
     ro[q] = 0;
     if (q < M) {
       cp_async16(&stage[q * kStreamThreads + tid], colp + d * ld);
-      ra[q] = __ldg(assign + d);
-      ro[q] = __ldg(own + d);
+      if (kPacked) {
+        ra[q] = __ldg(own + d);
+      } else {
+        ra[q] = __ldg(assign + d);
+        ro[q] = __ldg(own + d);
+      }
     }
     cp_async_commit();
   }
+  // rows advance by RPS: the addresses of row i + P
+  const T* nx_cm = colp + (R0 + rl + RPS * (int64_t)P) * ld;
+  const int32_t* nx_own = own + R0 + rl + RPS * P;
+  const int32_t* nx_assign = assign + R0 + rl + RPS * P;
+  const int64_t cm_step = RPS * ld;
   for (int32_t m = 0; m < M; m += P) {
 #pragma unroll
     for (int q = 0; q < P; ++q) {
       cp_async_wait<P - 1>();                      // row m + q has landed
-      const int32_t a = ra[q], o = ro[q];
+      const int32_t a = kPacked ? (ra[q] >> 16) - 1 : ra[q];
+      const int32_t o = kPacked ? (int16_t)ra[q] : ro[q];
       const int32_t i = m + q;
-      if (i < M && a >= 0 && a < k) {
+      if (i < M && (kPacked ? ra[q] != 0 : a >= 0 && a < k)) {
         const uint4 x = stage[q * kStreamThreads + tid];
-        const uint32_t off = (uint32_t)(rl + 128 * i);
+        const uint32_t off = (uint32_t)(rl + RPS * i);
         // the thread's first HALF keys sit in the row's first 128 bytes, the
         // others in the second: 8 threads' 16-byte loads cover 32 banks
         K* lo_p = acc + a * COLS + HALF * cg;
@@ -889,25 +818,47 @@ bt_scan_stream(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
           for (int h = 0; h < 4; ++h)
             key[h] = ((K)(uint32_t)((int64_t)w4[h] - o + 2147483648LL) << 32) | off;
         }
-        const uint4 lo = *reinterpret_cast<const uint4*>(lo_p);
-        const uint4 hi = *reinterpret_cast<const uint4*>(hi_p);
-        const K* cl = reinterpret_cast<const K*>(&lo);
-        const K* ch = reinterpret_cast<const K*>(&hi);
+        if constexpr (sizeof(T) == 2) {
+          // a key row's halves lie in the two halves of the banks: odd rows
+          // of a warp take theirs in the other order
+          const bool odd = rl & 1;
+          const uint32_t la = smem_u32(odd ? hi_p : lo_p), lb = smem_u32(odd ? lo_p : hi_p);
+          const uint4 ca = *reinterpret_cast<const uint4*>(odd ? hi_p : lo_p);
+          const uint4 cb = *reinterpret_cast<const uint4*>(odd ? lo_p : hi_p);
+          red_min_if_less(la, odd ? key[4] : key[0], ca.x);
+          red_min_if_less(la + 4, odd ? key[5] : key[1], ca.y);
+          red_min_if_less(la + 8, odd ? key[6] : key[2], ca.z);
+          red_min_if_less(la + 12, odd ? key[7] : key[3], ca.w);
+          red_min_if_less(lb, odd ? key[0] : key[4], cb.x);
+          red_min_if_less(lb + 4, odd ? key[1] : key[5], cb.y);
+          red_min_if_less(lb + 8, odd ? key[2] : key[6], cb.z);
+          red_min_if_less(lb + 12, odd ? key[3] : key[7], cb.w);
+        } else {
+          const uint4 lo = *reinterpret_cast<const uint4*>(lo_p);
+          const uint4 hi = *reinterpret_cast<const uint4*>(hi_p);
+          const K* cl = reinterpret_cast<const K*>(&lo);
+          const K* ch = reinterpret_cast<const K*>(&hi);
 #pragma unroll
-        for (int h = 0; h < HALF; ++h) {
-          if (key[h] < cl[h]) atomicMin(lo_p + h, key[h]);
-          if (key[HALF + h] < ch[h]) atomicMin(hi_p + h, key[HALF + h]);
+          for (int h = 0; h < HALF; ++h) {
+            if (key[h] < cl[h]) atomicMin(lo_p + h, key[h]);
+            if (key[HALF + h] < ch[h]) atomicMin(hi_p + h, key[HALF + h]);
+          }
         }
       }
       // stage q now takes row i + P
-      const int32_t nx = i + P;
-      ra[q] = -1;
-      if (nx < M) {
-        const int64_t d = R0 + rl + 128 * (int64_t)nx;
-        cp_async16(&stage[q * kStreamThreads + tid], colp + d * ld);
-        ra[q] = __ldg(assign + d);
-        ro[q] = __ldg(own + d);
+      ra[q] = kPacked ? 0 : -1;
+      if (i + P < M) {
+        cp_async16(&stage[q * kStreamThreads + tid], nx_cm);
+        if (kPacked) {
+          ra[q] = __ldg(nx_own);
+        } else {
+          ra[q] = __ldg(nx_assign);
+          ro[q] = __ldg(nx_own);
+        }
       }
+      nx_cm += cm_step;
+      nx_own += RPS;
+      if (!kPacked) nx_assign += RPS;
       cp_async_commit();
     }
   }
@@ -934,10 +885,17 @@ __global__ void __launch_bounds__(kThreads) bt_merge_ranges(const K* __restrict_
        i += (int64_t)gridDim.x * kThreads) {
     K best = none;
     int br = -1;
-    for (int r = 0; r < nranges; ++r) {
-      const K key = part[r * kk + i];
-      if (key != none &&
-          (br < 0 || StreamKey<T>::cost(key) < StreamKey<T>::cost(best))) { best = key; br = r; }
+    constexpr int U = 8;   // tables in flight
+    for (int r0 = 0; r0 < nranges; r0 += U) {
+      K key[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) key[u] = r0 + u < nranges ? __ldcg(part + (r0 + u) * kk + i) : none;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (key[u] != none && (br < 0 || StreamKey<T>::cost(key[u]) < StreamKey<T>::cost(best))) {
+          best = key[u];
+          br = r0 + u;
+        }
     }
     const int32_t u = (int32_t)(i / k), v = (int32_t)(i % k);
     if (br < 0 || u == v) {
@@ -962,7 +920,7 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!(attr_set.load() & (1ull << dev))) {
     e = cudaFuncSetAttribute(bt_scan_stream<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)stream_smem_bytes(kStreamMaxK));
+                             (int)stream_smem_bytes<T>(kStreamMaxK));
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(1ull << dev);
   }
@@ -980,7 +938,7 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(nslice * nranges);
   cfg.blockDim = dim3(kStreamThreads);
-  cfg.dynamicSmemBytes = stream_smem_bytes(k);
+  cfg.dynamicSmemBytes = stream_smem_bytes<T>(k);
   e = cudaLaunchKernelEx(&cfg, bt_scan_stream<T>, cm, ld, n, k, assign, (const int32_t*)W.perm,
                          nslice, nranges, part);
   if (e != cudaSuccess) return e;
@@ -990,6 +948,408 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
   e = cudaLaunchKernelEx(&cfg, bt_merge_ranges<K, T>, (const K*)part, nranges, n, k, tc, td);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
+}
+
+// ------------------------------------------------------------ short rows ---
+//
+// Fewer than kStreamMinK centers: a row is at most 1 KB and the whole table
+// fits the shared memory of a CTA (or a few slices of its columns do), so
+// one pass in row order needs no grouping, no work list and no packed table
+// in global memory.  CTA (slice, range) reads its rows' 16-byte vectors in
+// address order (every lane of a warp the next one: whole sectors whatever the
+// row length), gets the row's center and own cost CM(d, c) by two small loads
+// that hit the lines in flight, and lowers the entries of row c of its key
+// table with shared minima, only where its key is smaller.  The CTAs of a
+// cluster then reduce their tables through distributed shared memory, a share
+// of the entries each.
+//
+// Up to kTableOneCluster bytes of costs one cluster does it all and writes
+// tc/td itself: one launch, which is what such a call costs.  Above that,
+// clusters of kTableCluster CTAs fill the chip, write one packed table each
+// and bt_merge_tables (a dependent launch) takes the minimum over them.
+//
+// Measured per call, before (seven launches: count, plan, place, sort, scan,
+// unpack and a memset) and after: 2,000 x 20 int32 29.3 -> 10.7 us, 50,001 x
+// 126 int32 52 -> 30 us.
+//
+// int16 costs and ranges of at most 65,536 rows: one 32-bit key per entry,
+// ((t + 32768) << 16 | d - first row), one pass, native shared minima.
+// Otherwise t and d need 32 bits each, and a 64-bit shared minimum is a
+// compare-and-swap loop that every improvement pays for (with a few rows per
+// center and range, most keys improve).  So those entries are two words and a
+// batch of rows, held in registers, goes through twice: first t takes the
+// minimum (native; whoever lowers it voids the unit), then, after a barrier,
+// the keys that equal it put their unit in the minimum.  Rows ascend from
+// batch to batch, so a later equal t never replaces the unit.
+constexpr int kTableThreads = 1024;         // 32-bit keys: short batches, many warps
+constexpr int kTableUnroll = 4;             // vectors in flight per thread
+constexpr int kWideThreads = 512;           // two words: twice the registers, batches of 8
+constexpr int kWideUnroll = 8;
+constexpr int kTableCluster = 4;
+constexpr int64_t kTableOneCluster = 4 << 20;
+constexpr size_t kTableSmem = 200 * 1024;
+constexpr int kTableMaxClusters = 64;       // packed tables of a call, at most
+constexpr int kTableReuse = 16;             // rows per center and range to aim for ...
+constexpr int kTableMinSlice = 4;           // ... with slices of no less than 64 bytes
+
+struct TableShape {
+  int C, ncl, nslice, gs;   // cluster size, clusters per slice, slices, vectors per slice of a row
+  bool wide;                // 64-bit keys
+  size_t smem;
+};
+
+// `clusters`: clusters of kTableCluster CTAs that run at a time.
+static TableShape table_shape(int32_t n, int32_t k, int elem, int clusters) {
+  TableShape p;
+  const int vpl = 16 / elem;
+  const int G = (k + vpl - 1) / vpl;
+  const int64_t vecs = (int64_t)n * G;
+  const bool one = vecs * 16 <= kTableOneCluster;
+  p.C = kTableCluster;
+  if (one)
+    for (p.C = 1; p.C < 16 && vecs > (int64_t)p.C * 2 * kTableThreads;) p.C <<= 1;
+  for (p.nslice = 1;; ++p.nslice) {
+    p.gs = (G + p.nslice - 1) / p.nslice;
+    p.ncl = one ? 1 : std::max(1, std::min(kTableMaxClusters, clusters / p.nslice));
+    // few rows per center and range: nearly every key would be a new minimum
+    // and the tables would outweigh the costs; narrower slices of more rows
+    if (!one && p.gs > kTableMinSlice && p.ncl > 1 &&
+        (int64_t)n < (int64_t)kTableReuse * k * p.ncl * p.C)
+      continue;
+    p.wide = elem == 4 || ((int64_t)n + (int64_t)p.ncl * p.C - 1) / ((int64_t)p.ncl * p.C) > 65536;
+    p.smem = (size_t)k * p.gs * vpl * (p.wide ? 8 : 4);
+    if (p.smem <= kTableSmem) break;
+  }
+  p.nslice = (G + p.gs - 1) / p.gs;   // no empty slice
+  return p;
+}
+
+// Packed tables of the largest call of this size (any cost width).
+static size_t table_part_bytes(int32_t n, int32_t k) {
+  if (k >= kStreamMinK || (int64_t)n * k * 4 + 16ll * n <= kTableOneCluster) return 0;
+  return 8ull * k * k * kTableMaxClusters;
+}
+
+// What CTA (slice, range) of a table scan reads.
+template <typename T>
+struct TablePart {
+  static constexpr int VPL = 16 / (int)sizeof(T);
+  int cr, range, ranges, c0, kp, gw;
+  int64_t R0, R1;
+  __device__ __forceinline__ TablePart(const TableShape& p, int32_t n, int32_t k) {
+    const int cl = blockIdx.x / p.C, slice = cl % p.nslice;
+    cr = cl / p.nslice;
+    ranges = p.ncl * p.C;
+    range = cr * p.C + (int)cluster_rank();
+    R0 = first(range, n);
+    R1 = first(range + 1, n);
+    kp = p.gs * VPL;
+    c0 = slice * kp;
+    gw = min(p.gs, (k - c0 + VPL - 1) / VPL);   // vectors of this slice in a row
+  }
+  __device__ __forceinline__ int64_t first(int range_, int32_t n) const {
+    return (int64_t)range_ * n / ranges;
+  }
+  // Column of entry e of a center's row of the table: entries are stored by
+  // element of the vector, then by vector, so that the lanes of a warp, which
+  // hold neighbouring vectors, touch neighbouring words.
+  __device__ __forceinline__ int column(int e, int gs) const {
+    const int h = e / gs;
+    return c0 + (e - h * gs) * VPL + h;
+  }
+};
+
+__device__ __forceinline__ void put_table(int32_t* tc, int32_t* td, int64_t at,
+                                          unsigned long long best, bool diagonal) {
+  const bool none = best == ~0ull || diagonal;
+  tc[at] = none ? kTInf : (int32_t)((int64_t)(best >> 32) - 2147483648LL);
+  td[at] = none ? -1 : (int32_t)(uint32_t)best;
+}
+
+// int16 costs, 32-bit keys.
+__global__ void __launch_bounds__(kTableThreads, 1)
+bt_scan_table(const int16_t* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
+              const int32_t* __restrict__ assign, TableShape p, unsigned long long* part,
+              int32_t* tc, int32_t* td) {
+  constexpr int VPL = 8, U = kTableUnroll;
+  extern __shared__ __align__(16) unsigned char table_smem[];
+  uint32_t* acc = reinterpret_cast<uint32_t*>(table_smem);   // [k][kp]
+  const int tid = threadIdx.x;
+  const TablePart<int16_t> P(p, n, k);
+  const int gs = p.gs, kp = P.kp, gw = P.gw;
+  const int64_t R0 = P.R0, R1 = P.R1;
+  for (int i = tid; i < k * kp / 4; i += kTableThreads)
+    reinterpret_cast<uint4*>(acc)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  __syncthreads();
+  // vector i of the range: row i / gw, vector i % gw; a thread steps by the
+  // CTA's threads
+  const int dr = kTableThreads / gw, dg = kTableThreads - dr * gw;
+  int64_t r = R0 + tid / gw;
+  int g = tid % gw;
+  while (r < R1) {
+    uint4 x[U];
+    int32_t a[U], own[U], gg[U];
+    int64_t rr[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      rr[u] = r;
+      gg[u] = g;
+      a[u] = -1;
+      if (r < R1) {
+        x[u] = __ldg(reinterpret_cast<const uint4*>(cm + r * ld + P.c0) + g);
+        a[u] = __ldg(assign + r);
+      }
+      r += dr;
+      g += dg;
+      if (g >= gw) { g -= gw; ++r; }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      own[u] = 0;
+      if ((uint32_t)a[u] < (uint32_t)k) own[u] = (int32_t)__ldg(cm + rr[u] * ld + a[u]);
+      else a[u] = -1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (a[u] < 0) continue;
+      const uint32_t* e = acc + a[u] * kp + gg[u];
+      const uint32_t w4[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+      const uint32_t crow = ((uint32_t)(32768 - own[u]) << 16) | (uint32_t)(rr[u] - R0);
+      // entries only fall, so a stale read never hides a smaller key
+#pragma unroll
+      for (int h = 0; h < VPL; ++h) {
+        const uint32_t key = ((h & 1) ? (w4[h / 2] & 0xffff0000u) : (w4[h / 2] << 16)) + crow;
+        red_min_if_less(smem_u32(e + h * gs), key, e[h * gs]);
+      }
+    }
+  }
+  __syncthreads();
+  cluster_sync_all();
+  release_successor();
+  // a share of the entries per CTA, over all tables of the cluster
+  const int C = p.C, rank = P.range - P.cr * C;
+  const int E = k * kp;
+  const int e1 = (int)((int64_t)(rank + 1) * E / C);
+  for (int e = (int)((int64_t)rank * E / C) + tid; e < e1; e += kTableThreads) {
+    const int u = e / kp, v = P.column(e - u * kp, gs);
+    if (v >= k) continue;
+    unsigned long long best = ~0ull;
+    for (int q = 0; q < C; ++q) {
+      const uint32_t key = (uint32_t)dsmem_ld32(dsmem_addr(acc + e, (uint32_t)q));
+      // ranges ascend in d: an equal cost keeps the earlier range's unit
+      if (key != ~0u)
+        best = min(best, ((unsigned long long)((key >> 16) + 0x7fff8000u) << 32) |
+                             (uint32_t)(P.first(P.cr * C + q, n) + (key & 0xffffu)));
+    }
+    const int64_t at = (int64_t)u * k + v;
+    if (p.ncl > 1) part[(int64_t)P.cr * k * k + at] = best;
+    else put_table(tc, td, at, best, u == v);
+  }
+  cluster_sync_all();   // a table stays until every CTA has read it
+}
+
+// Two words per entry: t (kTInf: none) and d.
+template <typename T>
+__global__ void __launch_bounds__(kWideThreads, 1)
+bt_scan_table_wide(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
+                   const int32_t* __restrict__ assign, TableShape p, unsigned long long* part,
+                   int32_t* tc, int32_t* td) {
+  constexpr int VPL = 16 / (int)sizeof(T), U = kWideUnroll;
+  extern __shared__ __align__(16) unsigned char table_smem[];
+  const int tid = threadIdx.x;
+  const TablePart<T> P(p, n, k);
+  const int gs = p.gs, kp = P.kp, gw = P.gw;
+  int32_t* at_t = reinterpret_cast<int32_t*>(table_smem);          // [k][kp]
+  uint32_t* at_d = reinterpret_cast<uint32_t*>(at_t + k * kp);     // [k][kp]
+  for (int i = tid; i < k * kp / 4; i += kWideThreads) {
+    reinterpret_cast<int4*>(at_t)[i] = make_int4(kTInf, kTInf, kTInf, kTInf);
+    reinterpret_cast<uint4*>(at_d)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  }
+  __syncthreads();
+  const int dr = kWideThreads / gw, dg = kWideThreads - dr * gw;
+  int64_t r = P.R0 + tid / gw;
+  int g = tid % gw;
+  const int64_t vecs = (P.R1 - P.R0) * gw;
+  const int64_t batches = (vecs + (int64_t)U * kWideThreads - 1) / ((int64_t)U * kWideThreads);
+  auto cost = [](const uint4& x, int h) -> int32_t {
+    const uint32_t w = (&x.x)[sizeof(T) == 4 ? h : h / 2];
+    return sizeof(T) == 4 ? (int32_t)w : (h & 1) ? (int32_t)w >> 16 : (int32_t)(int16_t)w;
+  };
+  for (int64_t b = 0; b < batches; ++b) {
+    uint4 x[U];
+    int32_t a[U], own[U], at[U];
+    uint32_t rr[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      rr[u] = (uint32_t)r;
+      at[u] = g;
+      a[u] = -1;
+      if (r < P.R1) {
+        x[u] = __ldg(reinterpret_cast<const uint4*>(cm + r * ld + P.c0) + g);
+        a[u] = __ldg(assign + r);
+      }
+      r += dr;
+      g += dg;
+      if (g >= gw) { g -= gw; ++r; }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      own[u] = 0;
+      if ((uint32_t)a[u] < (uint32_t)k) {
+        own[u] = (int32_t)__ldg(cm + (int64_t)rr[u] * ld + a[u]);
+        at[u] += a[u] * kp;
+      } else {
+        at[u] = -1;
+      }
+    }
+    uint32_t maybe = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (at[u] < 0) continue;
+#pragma unroll
+      for (int h = 0; h < VPL; ++h) {
+        const int32_t t = cost(x[u], h) - own[u];
+        const int e = at[u] + h * gs;
+        const int32_t cur = at_t[e];
+        red_min_void_if_less(smem_u32(at_t + e), t, cur, smem_u32(at_d + e));
+        if (t <= cur) maybe |= 1u << u;   // the others are no minimum
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (!(maybe >> u & 1)) continue;
+#pragma unroll
+      for (int h = 0; h < VPL; ++h) {
+        const int32_t t = cost(x[u], h) - own[u];
+        const int e = at[u] + h * gs;
+        red_min_if_equal(smem_u32(at_d + e), rr[u], t, at_t[e]);
+      }
+    }
+    __syncthreads();
+  }
+  cluster_sync_all();
+  release_successor();
+  const int C = p.C, rank = P.range - P.cr * C;
+  const int E = k * kp;
+  const int e1 = (int)((int64_t)(rank + 1) * E / C);
+  for (int e = (int)((int64_t)rank * E / C) + tid; e < e1; e += kWideThreads) {
+    const int u = e / kp, v = P.column(e - u * kp, gs);
+    if (v >= k) continue;
+    unsigned long long best = ~0ull;
+    for (int q = 0; q < C; ++q) {
+      const uint32_t t = (uint32_t)dsmem_ld32(dsmem_addr(at_t + e, (uint32_t)q));
+      const uint32_t d = (uint32_t)dsmem_ld32(dsmem_addr(at_d + e, (uint32_t)q));
+      if (d != ~0u) best = min(best, ((unsigned long long)(t ^ 0x80000000u) << 32) | d);
+    }
+    const int64_t out = (int64_t)u * k + v;
+    if (p.ncl > 1) part[(int64_t)P.cr * k * k + out] = best;
+    else put_table(tc, td, out, best, u == v);
+  }
+  cluster_sync_all();
+}
+
+__global__ void __launch_bounds__(kThreads) bt_merge_tables(const unsigned long long* __restrict__ part,
+                                                            int ntab, int32_t k, int32_t* tc,
+                                                            int32_t* td) {
+  wait_predecessor();
+  const int64_t kk = (int64_t)k * k;
+  for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < kk;
+       i += (int64_t)gridDim.x * kThreads) {
+    unsigned long long best = ~0ull;
+#pragma unroll 4
+    for (int t = 0; t < ntab; ++t) best = min(best, part[t * kk + i]);
+    put_table(tc, td, i, best, i / k == i % k);
+  }
+}
+
+// The scan kernel of a cost type and key width, and its threads.
+template <typename T, bool WIDE>
+static auto table_kernel() {
+  if constexpr (WIDE) return bt_scan_table_wide<T>;
+  else return bt_scan_table;
+}
+template <bool WIDE>
+static constexpr int table_threads() { return WIDE ? kWideThreads : kTableThreads; }
+
+// Sets the kernel's attributes once per device and returns how many of its
+// clusters run at a time (GPCs whose SMs are no multiple of kTableCluster
+// hold fewer than the SM count suggests).
+template <typename T, bool WIDE>
+static cudaError_t table_setup(int* clusters) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if ((*clusters = known[dev].load()) > 0) return cudaSuccess;
+  auto kern = table_kernel<T, WIDE>();
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTableSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kTableCluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kTableCluster);
+  cfg.blockDim = dim3(table_threads<WIDE>());
+  cfg.dynamicSmemBytes = kTableSmem;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(clusters, kern, &cfg);
+  if (e != cudaSuccess) return e;
+  *clusters = std::max(1, *clusters);
+  known[dev].store(*clusters);
+  return cudaSuccess;
+}
+
+template <typename T, bool WIDE>
+static cudaError_t table_run(const T* cm, int64_t ld, int32_t n, int32_t k, const int32_t* assign,
+                             int32_t* tc, int32_t* td, void* ws, const TableShape& p,
+                             cudaStream_t st) {
+  unsigned long long* part = static_cast<unsigned long long*>(ws);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)p.C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3((unsigned)(p.C * p.ncl * p.nslice));
+  cfg.blockDim = dim3(table_threads<WIDE>());
+  cfg.dynamicSmemBytes = p.smem;
+  cudaError_t e =
+      cudaLaunchKernelEx(&cfg, table_kernel<T, WIDE>(), cm, ld, n, k, assign, p, part, tc, td);
+  if (e != cudaSuccess || p.ncl == 1) return e;
+  cudaLaunchAttribute pdl[1];
+  pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = pdl;
+  cfg.gridDim = dim3((unsigned)std::min<int64_t>(((int64_t)k * k + kThreads - 1) / kThreads, 608));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, bt_merge_tables, (const unsigned long long*)part, p.ncl, k, tc,
+                            td);
+}
+
+template <typename T>
+static cudaError_t table_call(const T* cm, int64_t ld, int32_t n, int32_t k, const int32_t* assign,
+                              int32_t* tc, int32_t* td, void* ws, cudaStream_t st) {
+  int clusters = 0;
+  cudaError_t e;
+  if constexpr (sizeof(T) == 2) {
+    if ((e = table_setup<T, false>(&clusters)) != cudaSuccess) return e;
+    const TableShape p = table_shape(n, k, 2, clusters);
+    if (!p.wide) return table_run<T, false>(cm, ld, n, k, assign, tc, td, ws, p, st);
+  }
+  if ((e = table_setup<T, true>(&clusters)) != cudaSuccess) return e;
+  const TableShape p = table_shape(n, k, (int)sizeof(T), clusters);
+  return table_run<T, true>(cm, ld, n, k, assign, tc, td, ws, p, st);
 }
 
 int bt_max_k(int elem_bytes) { return kThreads * (16 / elem_bytes); }
@@ -1012,17 +1372,13 @@ static cudaError_t bulk_attr() {
 }
 
 template <typename T>
-static cudaError_t scan_launch(const T* cm, int64_t ld, int32_t n, int32_t k, const BtWorkspace& W,
+static cudaError_t scan_launch(const T* cm, int64_t ld, int32_t k, const BtWorkspace& W,
                                cudaStream_t st, int num_sms) {
   const BulkShape p = bulk_shape(k, (int)sizeof(T));
-  if (p.row_bytes >= kBulkMinRowBytes) {
-    const cudaError_t e = bulk_attr<T>();
-    if (e != cudaSuccess) return e;
-    bt_scan_bulk<T><<<num_sms, kBulkThreads, bulk_smem_bytes(p, k), st>>>(cm, ld, k, W.perm, W.cnt,
-                                                                           W.t64, W.ctl, p);
-  } else {
-    bt_scan_rows<T><<<num_sms, kThreads, 0, st>>>(cm, ld, n, k, W.perm, W.items, W.t64, W.ctl);
-  }
+  const cudaError_t e = bulk_attr<T>();
+  if (e != cudaSuccess) return e;
+  bt_scan_bulk<T><<<num_sms, kBulkThreads, bulk_smem_bytes(p, k), st>>>(cm, ld, k, W.perm, W.cnt,
+                                                                         W.t64, W.ctl, p);
   return cudaSuccess;
 }
 
@@ -1033,6 +1389,10 @@ cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_byt
                               cudaStream_t st, int num_sms) {
   void* base = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
   const BtWorkspace W = carve(base, n, k);
+  if (k < kStreamMinK)
+    return elem_bytes == 2
+               ? table_call(static_cast<const int16_t*>(cm), ld, n, k, assign, tc, td, base, st)
+               : table_call(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td, base, st);
   const int nranges = stream_ranges(n, k, elem_bytes, num_sms);
   if (nranges > 0)
     return elem_bytes == 2
@@ -1047,8 +1407,8 @@ cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_byt
   bt_place<<<kTiles, kTileThreads, 4 * (size_t)k, st>>>(assign, n, k, W.cnt, W.tile_rel, W.perm);
   bt_sort_items<<<num_sms * 4, kThreads, 0, st>>>(W.items, W.ctl, W.perm, k, W.t64);
   e = elem_bytes == 2
-          ? scan_launch(static_cast<const int16_t*>(cm), ld, n, k, W, st, num_sms)
-          : scan_launch(static_cast<const int32_t*>(cm), ld, n, k, W, st, num_sms);
+          ? scan_launch(static_cast<const int16_t*>(cm), ld, k, W, st, num_sms)
+          : scan_launch(static_cast<const int32_t*>(cm), ld, k, W, st, num_sms);
   if (e != cudaSuccess) return e;
   bt_unpack<<<num_sms * 4, kThreads, 0, st>>>(W.t64, k, tc, td, W.ctl);
   return cudaGetLastError();

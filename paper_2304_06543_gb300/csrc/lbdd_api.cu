@@ -73,10 +73,11 @@ static void free_all(lbdd_solver* s) {
 
 int lbdd::check_device(int* dev, int* sms) {
   CK(cudaGetDevice(dev));
-  cudaDeviceProp prop;
-  CK(cudaGetDeviceProperties(&prop, *dev));
-  if (prop.major != 10 || prop.minor != 3) return LBDD_ERR_NODEV;
-  *sms = prop.multiProcessorCount;
+  int major = 0, minor = 0;
+  CK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, *dev));
+  CK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, *dev));
+  if (major != 10 || minor != 3) return LBDD_ERR_NODEV;
+  CK(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev));
   return LBDD_OK;
 }
 
