@@ -18,12 +18,14 @@
 //    P(j) >= q_j(last), the penalty j's last unit pays, no negative path
 //    starts at j (Alg. 4 applies nothing), and the round ends there.
 //  * Otherwise one synchronous Bellman-Ford from j answers both: a label
-//    l(v) is expanded only while l(v) + P(v) does not exceed the best value
-//    found so far (P(j) + cycle cost for Alg. 1; min l(u) + q_n(u) for
-//    Alg. 4).  Every node of every shortest path to the sink passes that
-//    test, because l(v) + P(v) bounds the value of any completion from v, so
-//    the sink's label, hop counts and lowest-index parents are those of the
-//    full Bellman-Ford, and the path applied is the same.
+//    l(v) is expanded only while l(v) + P(v) is below the best value found so
+//    far (P(j) + cycle cost for Alg. 1; min l(u) + q_n(u) for Alg. 4).
+//    l(v) + P(v) bounds the value of any completion from v, and a completion
+//    that only equals a value already found has more hops and is not the one
+//    the full Bellman-Ford reports; so every node of the path it reports is
+//    expanded, and the sink's label, hop counts and lowest-index parents come
+//    out the same.  (Equality matters: with whole-number costs and tight
+//    prices most labels are ties.)
 //  * After a cycle was applied, Alg. 4 searches again; the bound uses the
 //    prices raised by the first search's labels, max(P(v), P(j) + L - l1(v))
 //    (L the cycle's cost), less `off`, the most by which those exceed q_n.
@@ -56,12 +58,18 @@ namespace lbdd {
 // Bits of a node in a packed (hop, node) key (k <= 8191).
 constexpr int kGNodeBits = 13;
 constexpr int kGOrd = 64;                       // prefetched (unit, center) pairs
-constexpr int kGAff = 1024;                     // affected entries per rescan chunk, at least
+constexpr int kGWideLists = 800;                // centers up to which lists are that long
+// Affected entries that an apply lists at a time.  Where the cost table does
+// not fit shared memory anyway there is room for those of eight rows, so that
+// most paths go through each phase at once.
+__host__ __device__ inline int32_t guided_list(int32_t k, int32_t elem) {
+  return (int64_t)elem * k * k > 160 * 1024 ? 8 * k : k > 1024 ? k : 1024;
+}
 
 struct GLayout {
-  uint32_t pot, lab1, lab2, hop, list, slack, pen, qn, seg, tailp, path, pathu, mid, raff, cpath, aff,
-      ord, misc, ring, base_total, tsm, total;
-  int nring;
+  uint32_t pot, lab1, lab2, hop, list, slack, pen, qn, seg, tailp, path, pathu, mid, raff, ppos, cpath, aff,
+      ord, misc, ring, base_total, tsm, total, usm, full;
+  int nring, aff_rows;
 };
 
 // Rows of CM in flight: 8 where they are short, 4 otherwise (they cover the
@@ -85,7 +93,9 @@ __host__ __device__ inline GLayout make_guided_layout(int32_t k, int32_t elem) {
   L.lab1 = take(lt * ku);
   L.lab2 = take(lt * ku);
   L.hop = take(2u * ku);
-  const uint32_t aff = ku > (uint32_t)kGAff ? ku : (uint32_t)kGAff;
+  // (large k: one row's entries, so that the layout fits)
+  const uint32_t aff = (uint32_t)(k > kGWideLists ? k : guided_list(k, elem));
+  L.aff_rows = (int)(aff / ku) < 32 ? (int)(aff / ku) : 32;
   const uint32_t lists = 2u * 2u * lt * (ku + 2);
   L.list = take(lists > 8u * aff ? lists : 8u * aff);   // also the minima of a rescan
   L.slack = take(4u * ku);
@@ -97,6 +107,7 @@ __host__ __device__ inline GLayout make_guided_layout(int32_t k, int32_t elem) {
   L.pathu = take(4u * (ku + 2));
   L.mid = take(4u * (ku + 2));
   L.raff = take(4u * (ku + 2));
+  L.ppos = take(4u * (ku + 2));
   L.cpath = take(4u * (ku + 2));
   L.aff = take(4u * aff);
   L.ord = take(8u * kGOrd);
@@ -109,6 +120,8 @@ __host__ __device__ inline GLayout make_guided_layout(int32_t k, int32_t elem) {
   L.base_total = o;
   L.tsm = take((uint32_t)elem * ku * (uint32_t)guided_stride(k, elem));
   L.total = o;
+  L.usm = take(4u * ku * ku);               // the units of T, where they fit too
+  L.full = o;
   return L;
 }
 
@@ -129,7 +142,7 @@ struct GMisc {
   uint32_t sink;      // its hop count << kGNodeBits | node, if paid < ql
   uint32_t next[3];   // parents on the way back, by hop count modulo 3
   int32_t cnt[3];     // list lengths, by sweep modulo 3
-  int32_t naff, len, bad, stop;
+  int32_t len, bad, stop;
 };
 
 template <typename T, bool TSM, bool STRICT>
@@ -147,21 +160,23 @@ struct Guided {
   int32_t max_pages;
   int32_t n, k, ws;
   int tid, flags;
-  int32_t *s_pot, *s_slack, *s_pen, *s_seg, *s_tail, *s_path, *s_pathu, *s_raff, *s_cpath,
+  int32_t *s_pot, *s_slack, *s_pen, *s_seg, *s_tail, *s_path, *s_pathu, *s_raff, *s_ppos, *s_cpath,
       *s_aff, *s_ord;
   int32_t* s_qn;      // q_n of every center: what one more unit would pay there
-  int32_t* s_mid;     // prices of a second search; positions while units move
+  int32_t* s_mid;     // prices of a second search
   LT *s_lab1, *s_lab2;
   uint16_t* s_hop;    // sweep of every label's last change in the last search
   Ent* s_list;        // [2][k + 2]
   GMisc* M;
   unsigned char* s_ring;
   uint32_t ring_row;
-  int nring;
+  int nring, aff_rows;
+  int32_t* s_td;      // [k][k] units of T in shared memory, or null: global only
   T* tt;              // [k][ws] costs of T: shared memory, or the global mirror
   Book* B;
 
-  __device__ Guided(const DevInst& inst, unsigned char* base, const GLayout& L, Book* book, int fl)
+  __device__ Guided(const DevInst& inst, unsigned char* base, const GLayout& L, bool usm, Book* book,
+                    int fl)
       : I(inst) {
     cm = static_cast<const T*>(inst.cm);
     ld = inst.ld;
@@ -191,6 +206,7 @@ struct Guided {
     s_mid = i32(L.mid);
     s_qn = i32(L.qn);
     s_raff = i32(L.raff);
+    s_ppos = i32(L.ppos);
     s_cpath = i32(L.cpath);
     s_aff = i32(L.aff);
     s_ord = i32(L.ord);
@@ -198,7 +214,9 @@ struct Guided {
     s_ring = base + L.ring;
     ring_row = align16((uint32_t)sizeof(T) * (uint32_t)k);
     nring = L.nring;
+    aff_rows = L.aff_rows;
     tt = TSM ? reinterpret_cast<T*>(base + L.tsm) : static_cast<T*>(inst.mirror);
+    s_td = usm ? i32(L.usm) : nullptr;
     B = book;
   }
 
@@ -215,9 +233,16 @@ struct Guided {
     const int32_t t = edge(u, cl);
     return vacant(u) ? min(t, 0) : t;
   }
+  // Best unit of entry (u, cl).  In global memory equal costs lower it by
+  // reductions at L2, so it is read past L1.
+  __device__ __forceinline__ int32_t unit(int32_t u, int cl) const {
+    return s_td ? s_td[u * k + cl] : __ldcg(td + (int64_t)u * k + cl);
+  }
+  // What sits in shared memory is written back when the launch ends.
   __device__ __forceinline__ void set_entry(int32_t u, int cl, int32_t t, int32_t d) {
-    tc[(int64_t)u * k + cl] = t;
-    td[(int64_t)u * k + cl] = d;
+    if (!TSM) tc[(int64_t)u * k + cl] = t;
+    if (s_td) s_td[u * k + cl] = d;
+    else td[(int64_t)u * k + cl] = d;
     tt[(int64_t)u * ws + cl] = (T)(t == kTInf ? kInf : t);
   }
   // q_c(x), x >= 1: penalty of the x-th allotment beyond capacity (Def. 4).
@@ -257,16 +282,18 @@ struct Guided {
     pos[d] = idx;
     s_seg[c] = idx + 1;
   }
-  __device__ void list_remove_at(int32_t c, int32_t idx) {
+  // last_id, last_own: the list's last member, which takes the place.
+  __device__ void list_remove_at(int32_t c, int32_t idx, int32_t last_id, int32_t last_own) {
     const int32_t len = s_seg[c], last = len - 1;
-    if (idx < 0 || idx > last || B->free_top >= I.npages) { B->err0 = ST_ERR_INVARIANT; return; }
+    if (idx < 0 || idx > last || B->free_top >= I.npages || (uint32_t)last_id >= (uint32_t)n) {
+      B->err0 = ST_ERR_INVARIANT;
+      return;
+    }
     if (idx != last) {
-      const int32_t* from = mslot(c, last, len);
       int32_t* to = mslot(c, idx, len);
-      const int32_t moved = from[0], own = from[kPage];
-      to[0] = moved;
-      to[kPage] = own;
-      pos[moved] = idx;
+      to[0] = last_id;
+      to[kPage] = last_own;
+      pos[last_id] = idx;
     }
     if ((last & (kPage - 1)) == 0) {
       I.free_stack[B->free_top++] = s_tail[c];
@@ -360,9 +387,9 @@ struct Guided {
           M->cnt[c3n] = 0;
           if (timer()) front_stat(m);
         }
-        const LT bc = cyc ? (LT)pj + min((LT)-1, lab[j]) : kFixed;
+        const LT bc = cyc ? (LT)pj + min((LT)-1, lab[j] - 1) : kFixed;
         const int32_t paid = M->paid;
-        const int32_t bp = np ? min(ql - 1, paid) : INT32_MIN;
+        const int32_t bp = np ? min(ql, paid) - 1 : INT32_MIN;
         unsigned bits = 0;
         for (int cl = tid, c0 = 0; c0 < k; c0 += nthr, cl += nthr) {
           if (!single || sweep == 1) {
@@ -375,23 +402,30 @@ struct Guided {
           const LT old = b;
           const uint32_t colb = (uint32_t)min(cl, k - 1) * (uint32_t)sizeof(T);
           LT b2 = b;
-          for (int f = 0; f < m; f += U) {
-            Ent e[U];
-            int32_t t[U];
+          // N nodes from `at`; the last batch repeats the last node
+          auto batch = [&](auto size, uint32_t at, uint32_t last) {
+            constexpr int N = decltype(size)::value;
+            Ent e[N];
+            int32_t t[N];
 #pragma unroll
-            for (int q = 0; q < U; ++q)   // past the end: the last node again
-              e[q] = entry(in + (uint32_t)min(f + q, m - 1) * (uint32_t)sizeof(Ent));
+            for (int q = 0; q < N; ++q) e[q] = entry(min(at + q * (uint32_t)sizeof(Ent), last));
 #pragma unroll
-            for (int q = 0; q < U; ++q) {
+            for (int q = 0; q < N; ++q) {
               t[q] = cost_at((STRICT ? e[q].off & ~kGVacant : e[q].off) + colb);
               if (STRICT && (e[q].off & kGVacant)) t[q] = min(t[q], 0);
             }
 #pragma unroll
-            for (int q = 0; q < U; q += 2) {
+            for (int q = 0; q < N; q += 2) {
               b = relax(e[q].l, t[q], b);
               b2 = relax(e[q + 1].l, t[q + 1], b2);
             }
-          }
+          };
+          const uint32_t last = in + (uint32_t)(m - 1) * (uint32_t)sizeof(Ent);
+          uint32_t at = in;
+          int left = m;
+          for (; left > U / 2; left -= U, at += U * (uint32_t)sizeof(Ent))
+            batch(std::integral_constant<int, U>(), at, last);
+          if (left > 0) batch(std::integral_constant<int, U / 2>(), at, last);
           b = min(b, b2);
           const bool up = b < old;
           if (up) {
@@ -402,7 +436,7 @@ struct Guided {
           if (np) {
             const int32_t vm = __reduce_min_sync(0xffffffffu, up ? clamp_sum(b, qv) : INT32_MAX);
             if (vm < paid && lane == 0) atomicMin(&M->paid, vm);
-            now = min(bp, vm);
+            now = min(bp, vm - 1);
           }
           const LT key = b + (LT)pv;
           const bool push = up && (key <= (LT)now || key <= bc);
@@ -456,27 +490,37 @@ struct Guided {
   // The canonical shortest path that ends at node `last` (the cycle through
   // j if last < 0), backwards into s_pathu: the parent of a node v with label
   // l and hop count h is the lowest-index u with l(u) + T[u][v] = l and
-  // hop(u) = h - 1.  Thread = node, one barrier per hop.  Returns its length,
-  // -1 if there is none.
+  // hop(u) = h - 1.  One warp up to kFollowWarp centers (no barrier), else
+  // thread = node and a barrier per hop.  Returns its length, -1 if there is
+  // none (the one-warp form: to warp 0 only).
+  static constexpr int kFollowWarp = 64;
+  __device__ __forceinline__ bool precedes(int u, int32_t v, int h, LT l, int32_t j,
+                                           const LT* lab) const {
+    return s_hop[u] == h - 1 && u != j && u != v && lab[u] != kNoLab && lab[u] + (LT)arc(u, v) == l;
+  }
   __device__ int follow(int32_t j, int32_t last, const LT* lab) {
+    const bool alone = k <= kFollowWarp;
     int32_t v = last < 0 ? j : last;
-    int h = s_hop[v], m = 0;
+    int h = s_hop[v], m = 0, slot = 0;
     LT l = lab[v];
     if (last >= 0) {
       if (tid == 0) s_pathu[0] = v;
       m = 1;
     }
     for (; h > 1; --h) {
-      uint32_t* slot = &M->next[h % 3];
-      for (int u = tid; u < k; u += kThreads)
-        if (s_hop[u] == h - 1 && u != j && u != v && lab[u] != kNoLab &&
-            lab[u] + (LT)arc(u, v) == l) {
-          atomicMin(slot, (uint32_t)u);
-          break;
-        }
-      __syncthreads();
-      const uint32_t best = *slot;
-      if (tid == 0) M->next[(h + 1) % 3] = ~0u;   // read before the last barrier
+      uint32_t best = ~0u;
+      for (int u = tid; u < k; u += alone ? 32 : kThreads)
+        if (precedes(u, v, h, l, j, lab)) { best = (uint32_t)u; break; }
+      if (alone) {
+        best = __reduce_min_sync(0xffffffffu, best);
+      } else {
+        if (best != ~0u) atomicMin(&M->next[slot], best);
+        __syncthreads();
+        best = M->next[slot];
+        slot = slot == 2 ? 0 : slot + 1;
+        // the slot after the next one: read before the last barrier
+        if (tid == 0) M->next[slot == 2 ? 0 : slot + 1] = ~0u;
+      }
       if (best == ~0u) return -1;
       v = (int32_t)best;
       l = lab[v];
@@ -488,279 +532,345 @@ struct Guided {
     return m + 1 < 2 ? -1 : m + 1;
   }
 
-  // Follows the parents from `last` to j and applies the transfers of that
-  // path (Alg. 1 and Alg. 4, "if cost < 0" branch): every center on it hands
-  // its best unit for the next center on; for a cycle the last one hands to
-  // j, for a path the last center only gains and j only loses a unit.  Then
-  // the rows of T of those centers.  Warp 0 moves the units while the other
-  // warps already take the arriving units into the rows (that needs no member
-  // list); what is left per call is a chain of four global latencies: the
-  // moved units, their rows, member ids, member costs.  Returns the length of
-  // the path (s_path), -1 if the walk is bad.
+  __device__ __forceinline__ int32_t arriving(bool npath, int m, int i) const {
+    return i > 0 ? s_pathu[i - 1] : (npath ? -1 : s_pathu[m - 1]);
+  }
+
+  // Applies the transfers of the path that follow() finds (Alg. 1 and Alg. 4,
+  // "if cost < 0" branch): every center on it hands its best unit for the
+  // next center on; for a cycle the last one hands to j, for a path the last
+  // center only gains and j only loses a unit.  Then the rows of T of those
+  // centers: an entry whose best unit was not the leaving one keeps its
+  // minimum over the remaining members and takes the arriving unit in; the
+  // others ("affected") are recomputed over the member list.
+  //
+  // What an apply costs is its chain of global latencies, so everything that
+  // can be in flight together is: after the affected entries are listed
+  // (shared memory only, where the units fit), the warps share the arriving
+  // units' rows and the members of the affected entries, while warp 0 loads
+  // what it needs to move the units.  Member lists change only afterwards:
+  // the scan of a list skips the leaving unit and adds the arriving one.
+  // Returns the length of the path (s_path), -1 if there is none.
   __device__ int apply(int32_t j, bool npath, int32_t last, const LT* lab, int64_t cost) {
     const uint64_t t0 = timer() ? clock_cycles() : 0;
-    const int lane = tid & 31;
-    const int m = follow(j, last, lab);
-    if (m < 0) return m;
+    const int lane = tid & 31, warp = tid >> 5;
+    int m = 0;
+    if (k > kFollowWarp || warp == 0) m = follow(j, last, lab);
     if (tid < 32) {
       __syncwarp();
-      if (lane == 0) M->naff = 0;
+      if (lane == 0) M->len = m;
       for (int i = lane; i < m; i += 32) s_path[i] = s_pathu[m - 1 - i];
       __syncwarp();
       for (int i = lane; i < m; i += 32) {
         const int32_t to = (i + 1 < m) ? s_path[i + 1] : (npath ? -1 : j);
         // a dummy unit moves where the edge's cost came from a vacancy
         const bool dummy = STRICT && vacant(s_path[i]) && edge(s_path[i], to) > 0;
-        int32_t x = to >= 0 && !dummy ? __ldcg(td + (int64_t)s_path[i] * k + to) : -1;
+        int32_t x = to >= 0 && !dummy ? unit(s_path[i], to) : -1;
         if (to >= 0 && !dummy && (uint32_t)x >= (uint32_t)n) { x = -1; B->err0 = ST_ERR_INVARIANT; }
         s_pathu[i] = x;
         s_raff[i] = 0;
       }
     }
     __syncthreads();
-    const int chunk = min(32, max(k, kGAff) / k);   // rows whose affected entries fit s_aff
+    m = M->len;
+    if (m < 0) return m;
+    // what moving the units takes, in flight while the rows are updated.
+    // Warp 0, lane = center of the path: position of its leaving unit,
+    // CM(arriving unit, center).  Paths: warp 1 takes j's unit out (position,
+    // and j's last member, which takes its place), warp 2 puts the last
+    // arriving unit in; where a page of the pool is freed or taken, warp 1
+    // does both.
+    int32_t at = -1, own = 0, last_id = 0, last_own = 0;
+    bool pages = false;
+    if (warp == 0) {
+      if (lane < m) {
+        const int32_t x_out = s_pathu[lane], x_in = arriving(npath, m, lane);
+        if (x_out >= 0) at = pos[x_out];
+        if (x_in >= 0) own = (int32_t)row(x_in)[s_path[lane]];
+      }
+      for (int i = lane + 32; i < m; i += 32) s_ppos[i] = s_pathu[i] >= 0 ? pos[s_pathu[i]] : -1;
+    } else if (npath && warp <= 2) {
+      const int32_t term = s_path[m - 1], x_in = s_pathu[m - 2];
+      pages = ((s_seg[j] - 1) & (kPage - 1)) == 0 || (s_seg[term] & (kPage - 1)) == 0;
+      if (x_in >= 0) own = (int32_t)row(x_in)[term];
+      if (warp == 1) {
+        at = s_pathu[0] >= 0 ? pos[s_pathu[0]] : -1;
+        const int32_t* sl = mslot(j, s_seg[j] - 1, s_seg[j]);
+        last_id = sl[0];
+        last_own = sl[kPage];
+      }
+    }
+    const int chunk = aff_rows;   // rows whose affected entries fit s_aff
+    const int nblk = (k + 31) >> 5;
     for (int i0 = 0; i0 < m; i0 += chunk) {
-      if (tid >= 32) merge_rows(npath, m, i0, min(m, i0 + chunk));
-      else if (i0 == 0) move_units(j, npath, m, cost);
+      const int i1 = min(m, i0 + chunk), units = (i1 - i0) * nblk;
+      list_affected(npath, m, i0, units, nblk);
       __syncthreads();
       const uint64_t t1 = timer() ? clock_cycles() : 0;
       if (timer() && i0 == 0) B->t_apply += t1 - t0;
-      if (M->naff) rescan_affected(i0, min(m, i0 + chunk));
-      __syncthreads();
-      if (timer()) B->t_rescan += clock_cycles() - t1;
-      if (i0 + chunk < m) {
-        if (tid == 0) M->naff = 0;
-        __syncthreads();
+      // lane = row: entries, list length, log2 of the entries per warp, tasks
+      const int i = i0 + lane;
+      const int na = i < i1 ? s_raff[i] : 0;
+      const int len = na > 0 ? s_seg[s_path[i]] : 0;
+      const int le = na > 16 ? 5 : na > 8 ? 4 : na > 4 ? 3 : na > 2 ? 2 : na > 1 ? 1 : 0;
+      const int parts = na > 0 ? max(1, (len + (kScanU << (5 - le)) - 1) / (kScanU << (5 - le))) : 0;
+      const bool split = __any_sync(0xffffffffu, parts > 1);
+      if (warp == 0) {
+        const int rows = __reduce_add_sync(0xffffffffu, len);
+        if (lane == 0) B->col_rows += rows;
+      } else {
+        int incl = ((na + 31) >> 5) * parts;
+        const int mine = incl;
+        if (__any_sync(0xffffffffu, na > 0)) {
+#pragma unroll
+          for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += o;
+          }
+        }
+        const int tasks = __shfl_sync(0xffffffffu, incl, 31);
+        // scan tasks first, then batches of kMergeU blocks of 32 columns
+        const int items = tasks + (units + kMergeU - 1) / kMergeU;
+        for (int t = warp - 1; t < items; t += kWarps - 1) {
+          if (t < tasks) {
+            const int r = __popc(__ballot_sync(0xffffffffu, incl <= t));
+            const int na_r = __shfl_sync(0xffffffffu, na, r), len_r = __shfl_sync(0xffffffffu, len, r);
+            const int le_r = __shfl_sync(0xffffffffu, le, r);
+            const int parts_r = __shfl_sync(0xffffffffu, parts, r);
+            const int t0r = t - __shfl_sync(0xffffffffu, incl - mine, r);
+            const int blk = t0r / parts_r;
+            scan_task(npath, m, i0, r, na_r, len_r, le_r, parts_r, blk, t0r - blk * parts_r);
+          } else {
+            merge_task(npath, m, i0, units, nblk, (t - tasks) * kMergeU);
+          }
+        }
       }
+      __syncthreads();
+      if (split) {
+        for (int r = warp; r < i1 - i0; r += kWarps) {
+          const int na_r = __shfl_sync(0xffffffffu, na, r);
+          if (__shfl_sync(0xffffffffu, parts, r) > 1)
+            for (int e = lane; e < na_r; e += 32)
+              put_entry(s_path[i0 + r], s_aff[r * k + e], best_of(r * k + e));
+        }
+      }
+      if (split || i1 < m) __syncthreads();
+      if (timer()) B->t_rescan += clock_cycles() - t1;
     }
+    move_units(j, npath, m, cost, at, own, last_id, last_own, pages);
     return m;
   }
 
-  __device__ __forceinline__ int32_t arriving(bool npath, int m, int i) const {
-    return i > 0 ? s_pathu[i - 1] : (npath ? -1 : s_pathu[m - 1]);
-  }
+  static constexpr int kScanU = 8;    // members in flight per lane
+  static constexpr int kMergeU = 4;   // column blocks in flight per warp
 
-  // Warp 0: member lists, allotment, loads and objective.
-  __device__ void move_units(int32_t j, bool npath, int m, int64_t cost) {
+  // The affected entries of rows i0...: s_aff[row][...] columns, their number
+  // in s_raff, their running minima reset.
+  __device__ void list_affected(bool npath, int m, int i0, int units, int nblk) {
     const int lane = tid & 31;
-    int32_t pos0 = -1, ownl = 0;   // of j's leaving unit and the last arriving unit (paths)
-    for (int b = 0; b < m; b += 32) {
-      const int i = b + lane;
-      int32_t c = 0, x_out = -1, x_in = -1, at = -1, own = 0;
-      if (i < m) {
-        c = s_path[i];
-        x_out = s_pathu[i];
-        x_in = arriving(npath, m, i);
-        if (x_out >= 0) at = pos[x_out];
-        if (x_in >= 0) own = (int32_t)row(x_in)[c];   // CM(x_in, its new center)
-        if (x_out >= 0) I.assign[x_out] = (i + 1 < m) ? s_path[i + 1] : j;
-      }
-      if (b == 0) pos0 = __shfl_sync(0xffffffffu, at, 0);
-      if (m - 1 >= b && m - 1 < b + 32) ownl = __shfl_sync(0xffffffffu, own, m - 1 - b);
-      if (i < m) s_mid[i] = at;
-      __syncwarp();   // every position of this batch is read before any is replaced
-      if (x_out >= 0 && x_in >= 0) {
-        if (at >= 0 && at < s_seg[c]) {
-          int32_t* slot = mslot(c, at, s_seg[c]);
-          slot[0] = x_in;
-          slot[kPage] = own;
-        } else {
-          s_mid[i] = -1;
-          B->err0 = ST_ERR_INVARIANT;
-        }
-      }
-    }
-    __syncwarp();
-    for (int i = lane; i < m; i += 32) {   // positions, once all old ones were read
-      const int32_t x_in = arriving(npath, m, i);
-      if (s_pathu[i] >= 0 && x_in >= 0 && s_mid[i] >= 0) pos[x_in] = s_mid[i];
-    }
-    __syncwarp();
-    if (STRICT && lane == 0) {
-      // centers that only lose or only gain a real unit: a dummy is on the
-      // other side of their pair of edges
-      for (int i = 0; i < m; ++i) {
-        const int32_t c = s_path[i], x_out = s_pathu[i], x_in = arriving(npath, m, i);
-        if (x_out >= 0 && x_in < 0) {
-          list_remove_at(c, s_mid[i]);
-          shift_load(c, -1);
-        } else if (x_out < 0 && x_in >= 0) {
-          list_append(c, x_in, (int32_t)row(x_in)[c]);
-          shift_load(c, 1);
-        }
-      }
-    }
-    if (lane == 0) {
-      if (npath) {
-        const int32_t term = s_path[m - 1];
-        list_remove_at(j, pos0);
-        if (s_pathu[m - 2] >= 0) list_append(term, s_pathu[m - 2], ownl);
-        else B->err0 = ST_ERR_INVARIANT;
-        shift_load(j, -1);
-        shift_load(term, 1);
-        B->paths++;
-        B->moves += m - 1;
-      } else {
-        B->cycles++;
-        B->moves += m;
-      }
-      B->delta += cost;
-    }
-  }
-
-  // Warps 1..15: rows i0..i1 of the path.  Center s_path[i] lost unit
-  // s_pathu[i] and gained the one before it (either may be absent): an entry
-  // whose best unit was not the leaving one keeps its minimum over the
-  // remaining members and only takes the arriving unit in; the others are
-  // listed in s_aff.  All rows go through together, so that their loads
-  // overlap.
-  __device__ void merge_rows(bool npath, int m, int i0, int i1) {
-    constexpr int U = 4, W = kWarps - 1;
-    const int nblk = (k + 31) >> 5, lane = tid & 31;   // a warp takes 32 columns of one row
-    int r = 0, blk = (tid >> 5) - 1;
-    while (blk >= nblk) { blk -= nblk; ++r; }
-    while (i0 + r < i1) {
-      int32_t bd[U], ct[U], ow[U], rr[U], vv[U];
+    const int dr = kWarps / nblk, db = kWarps - dr * nblk;
+    int w = tid >> 5;
+    int r = w / nblk, blk = w - r * nblk;
+    while (w < units) {
+      int32_t bd[kMergeU], rr[kMergeU], vv[kMergeU];
 #pragma unroll
-      for (int q = 0; q < U; ++q) {
-        const int i = i0 + r, v = blk * 32 + lane;
-        rr[q] = r;
-        vv[q] = v;
-        bd[q] = -2;   // no item
-        ct[q] = ow[q] = 0;
-        if (i < i1) {
-          const int32_t c = s_path[i], x_in = arriving(npath, m, i);
-          if (v < k && v != c) {
-            bd[q] = __ldcg(td + (int64_t)c * k + v);
-            if (x_in >= 0) {
-              const T* rx = row(x_in);
-              ct[q] = (int32_t)rx[v];
-              ow[q] = (int32_t)rx[c];
-            }
-          }
-          blk += W;
-          while (blk >= nblk) { blk -= nblk; ++r; }
-        }
+      for (int q = 0; q < kMergeU; ++q) {
+        rr[q] = w < units ? r : -1;
+        vv[q] = blk * 32 + lane;
+        bd[q] = -1;
+        if (rr[q] >= 0 && vv[q] < k && s_pathu[i0 + r] >= 0) bd[q] = unit(s_path[i0 + r], vv[q]);
+        w += kWarps;
+        r += dr;
+        blk += db;
+        if (blk >= nblk) { blk -= nblk; ++r; }
       }
 #pragma unroll
-      for (int q = 0; q < U; ++q) {
-        const int i = i0 + rr[q], v = vv[q];
-        if (i >= i1) break;
-        const int32_t c = s_path[i], x_out = s_pathu[i], x_in = arriving(npath, m, i);
-        const bool hit = bd[q] >= 0 && bd[q] == x_out;
-        if (!hit && bd[q] != -2 && x_in >= 0) {
-          const int32_t t = ct[q] - ow[q];
-          const int32_t e = edge(c, v);
-          const int32_t bt = e == kInf ? kTInf : e;
-          if (lex_less(t, x_in, bt, bd[q])) set_entry(c, v, t, x_in);
-        }
+      for (int q = 0; q < kMergeU; ++q) {
+        if (rr[q] < 0) break;
+        const int i = i0 + rr[q];
+        const bool hit = bd[q] >= 0 && bd[q] == s_pathu[i] && vv[q] != s_path[i];
         const unsigned bits = __ballot_sync(0xffffffffu, hit);
         if (bits) {
           int at = 0;
           const int leader = __ffs(bits) - 1;
-          if (lane == leader) {
-            at = atomicAdd(&s_raff[i], __popc(bits));
-            M->naff = 1;
+          if (lane == leader) at = atomicAdd(&s_raff[i], __popc(bits));
+          at = __shfl_sync(0xffffffffu, at, leader) + __popc(bits & ((1u << lane) - 1u));
+          if (hit) {
+            s_aff[rr[q] * k + at] = vv[q];
+            best_of(rr[q] * k + at) = ~0ull;
           }
-          at = __shfl_sync(0xffffffffu, at, leader);
-          if (hit) s_aff[rr[q] * k + at + __popc(bits & ((1u << lane) - 1u))] = v;
         }
       }
     }
   }
-
-  // The listed entries of rows i0..i1, each the minimum over its center's
-  // members.  A warp takes a block of at most 32 entries of one row and a
-  // part of the member list: lane = (entry, member of eight in flight), with
-  // as many lanes per entry as the block leaves, so that few entries of a
-  // long list (a large center) still fill the warps and many entries of a
-  // short one read neighbouring columns of the same rows.  Lists of more
-  // than one part meet in a 64-bit shared minimum per entry.
-  __device__ void rescan_affected(int i0, int i1) {
-    constexpr int U = 8;
-    const int lane = tid & 31, warp = tid >> 5;
-    unsigned long long* s_best = reinterpret_cast<unsigned long long*>(s_list);   // [rows][k]
-    // lane = row: entries, list length, log2 of the entries per warp, tasks
-    const int i = i0 + lane;
-    const int na = i < i1 ? s_raff[i] : 0;
-    const int len = na > 0 ? s_seg[s_path[i]] : 0;
-    const int le = na > 16 ? 5 : na > 8 ? 4 : na > 4 ? 3 : na > 2 ? 2 : na > 1 ? 1 : 0;
-    const int parts = na > 0 ? max(1, (len + (U << (5 - le)) - 1) / (U << (5 - le))) : 0;
-    int incl = ((na + 31) >> 5) * parts;
-    const int mine = incl;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int o = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += o;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const bool split = __any_sync(0xffffffffu, parts > 1);
-    if (warp == 0) {
-      const int rows = __reduce_add_sync(0xffffffffu, len);
-      if (lane == 0) B->col_rows += rows;
-    }
-    if (split) {
-      for (int r = warp; r < i1 - i0; r += kWarps) {
-        const int na_r = __shfl_sync(0xffffffffu, na, r);
-        for (int e = lane; e < na_r; e += 32) s_best[r * k + e] = ~0ull;
-      }
-      __syncthreads();
-    }
-    for (int t = warp; t < total; t += kWarps) {
-      const int r = __popc(__ballot_sync(0xffffffffu, incl <= t));
-      const int na_r = __shfl_sync(0xffffffffu, na, r), len_r = __shfl_sync(0xffffffffu, len, r);
-      const int le_r = __shfl_sync(0xffffffffu, le, r), parts_r = __shfl_sync(0xffffffffu, parts, r);
-      const int t0 = t - __shfl_sync(0xffffffffu, incl - mine, r);
-      const int blk = t0 / parts_r, part = t0 - blk * parts_r;
-      const int e = (blk << 5) + (lane & ((1 << le_r) - 1)), sub = lane >> le_r;
-      const int step = 32 >> le_r;
-      const int32_t c = s_path[i0 + r];
-      const int32_t v = e < na_r ? s_aff[r * k + e] : 0;
-      const int32_t base = part * U * step + sub;
-      unsigned long long best = ~0ull;
-      if (e < na_r && base < len_r) {
-        // a part is a power of two of at most a page's entries: one page
-        const int32_t* sl = mslot(c, base, len_r);
-        const int left = (len_r - base + step - 1) >> (5 - le_r);
-        const T* cv = cm + v;
-        int32_t id[U], ow[U], x[U];
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-          const int32_t at = (q < left ? q : 0) << (5 - le_r);   // past the end: the first again
-          id[q] = sl[at];
-          ow[q] = sl[at + kPage];
-        }
-#pragma unroll
-        for (int q = 0; q < U; ++q) {
-          if ((uint32_t)id[q] >= (uint32_t)n) id[q] = 0;   // guard: corrupt entry
-          x[q] = (int32_t)cv[(int64_t)id[q] * ld];
-        }
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-          best = min(best, ((unsigned long long)((uint32_t)(x[q] - ow[q]) ^ 0x80000000u) << 32) |
-                               (uint32_t)id[q]);
-      }
-      for (int s = 1 << le_r; s < 32; s <<= 1)
-        best = min(best, (unsigned long long)__shfl_xor_sync(0xffffffffu, best, s));
-      if (e < na_r && sub == 0) {
-        if (parts_r > 1) atomicMin(&s_best[r * k + e], best);
-        else put_entry(c, v, best);
-      }
-    }
-    if (split) {
-      __syncthreads();
-      for (int r = warp; r < i1 - i0; r += kWarps) {
-        const int na_r = __shfl_sync(0xffffffffu, na, r);
-        if (__shfl_sync(0xffffffffu, parts, r) > 1)
-          for (int e = lane; e < na_r; e += 32)
-            put_entry(s_path[i0 + r], s_aff[r * k + e], s_best[r * k + e]);
-      }
-    }
+  // 64-bit running minimum of a listed entry (the frontier lists' space).
+  __device__ __forceinline__ unsigned long long& best_of(int e) const {
+    return reinterpret_cast<unsigned long long*>(s_list)[e];
+  }
+  static __device__ __forceinline__ unsigned long long entry_key(int32_t t, int32_t d) {
+    return ((unsigned long long)((uint32_t)t ^ 0x80000000u) << 32) | (uint32_t)d;
   }
   __device__ __forceinline__ void put_entry(int32_t c, int32_t v, unsigned long long best) {
     if (best == ~0ull) set_entry(c, v, kTInf, -1);
-    else set_entry(c, v, (int32_t)((int64_t)(best >> 32) - 2147483648LL),
-                   (int32_t)(best & 0xffffffffu));
+    else set_entry(c, v, (int32_t)((uint32_t)(best >> 32) ^ 0x80000000u), (int32_t)(uint32_t)best);
+  }
+
+  // A block of at most 32 affected entries of row i0 + r over one part of its
+  // center's member list: lane = (entry, member of eight in flight), with as
+  // many lanes per entry as the block leaves, so that few entries of a long
+  // list (a large center) still fill the warps and many entries of a short
+  // one read neighbouring columns of the same rows.  Lists of more than one
+  // part meet in the entry's running minimum.
+  __device__ void scan_task(bool npath, int m, int i0, int r, int na, int len, int le, int parts,
+                            int blk, int part) {
+    constexpr int U = kScanU;
+    const int lane = tid & 31;
+    const int e = (blk << 5) + (lane & ((1 << le) - 1)), sub = lane >> le;
+    const int step = 32 >> le;
+    const int32_t c = s_path[i0 + r], x_out = s_pathu[i0 + r];
+    const int32_t v = e < na ? s_aff[r * k + e] : 0;
+    const int32_t base = part * U * step + sub;
+    unsigned long long best = ~0ull;
+    if (e < na && part == 0 && sub == 0) {
+      const int32_t x_in = arriving(npath, m, i0 + r);
+      if (x_in >= 0) best = entry_key((int32_t)row(x_in)[v] - (int32_t)row(x_in)[c], x_in);
+    }
+    if (e < na && base < len) {
+      // a part is a power of two of at most a page's entries: one page
+      const int32_t* sl = mslot(c, base, len);
+      const int left = (len - base + step - 1) >> (5 - le);
+      const T* cv = cm + v;
+      int32_t id[U], ow[U], x[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int32_t at = (q < left ? q : 0) << (5 - le);   // past the end: the first again
+        id[q] = sl[at];
+        ow[q] = sl[at + kPage];
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if ((uint32_t)id[q] >= (uint32_t)n) id[q] = x_out;   // guard: corrupt entry
+        x[q] = (int32_t)cv[(int64_t)id[q] * ld];
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (id[q] != x_out) best = min(best, entry_key(x[q] - ow[q], id[q]));
+    }
+    for (int s = 1 << le; s < 32; s <<= 1)
+      best = min(best, (unsigned long long)__shfl_xor_sync(0xffffffffu, best, s));
+    if (e < na && sub == 0) {
+      if (parts > 1) atomicMin(&best_of(r * k + e), best);
+      else put_entry(c, v, best);
+    }
+  }
+
+  // The arriving units into the entries that are not affected: kMergeU blocks
+  // of 32 columns from block w of rows i0....
+  __device__ void merge_task(bool npath, int m, int i0, int units, int nblk, int w) {
+    const int lane = tid & 31;
+    int r = w / nblk, blk = w - r * nblk;
+    int32_t ct[kMergeU], ow[kMergeU], bd[kMergeU], rr[kMergeU], vv[kMergeU];
+#pragma unroll
+    for (int q = 0; q < kMergeU; ++q) {
+      rr[q] = -1;
+      vv[q] = blk * 32 + lane;
+      ct[q] = ow[q] = bd[q] = 0;
+      if (w + q < units && vv[q] < k) {
+        const int i = i0 + r;
+        const int32_t c = s_path[i], x_in = arriving(npath, m, i);
+        if (x_in >= 0 && vv[q] != c) {
+          rr[q] = r;
+          const T* rx = row(x_in);
+          ct[q] = (int32_t)rx[vv[q]];
+          ow[q] = (int32_t)rx[c];
+          bd[q] = unit(c, vv[q]);
+        }
+      }
+      if (++blk == nblk) { blk = 0; ++r; }
+    }
+#pragma unroll
+    for (int q = 0; q < kMergeU; ++q) {
+      if (rr[q] < 0) continue;
+      const int i = i0 + rr[q];
+      const int32_t c = s_path[i], x_out = s_pathu[i];
+      if (x_out >= 0 && bd[q] == x_out) continue;   // affected
+      const int32_t x_in = arriving(npath, m, i);
+      const int32_t t = ct[q] - ow[q];
+      const int32_t e = edge(c, vv[q]);
+      const int32_t bt = e == kInf ? kTInf : e;
+      if (lex_less(t, x_in, bt, bd[q])) set_entry(c, vv[q], t, x_in);
+    }
+  }
+
+  // Member lists, allotment, loads and objective, by a few warps at once (see
+  // apply for who holds what); the others may already prepare the next search.
+  __device__ void move_units(int32_t j, bool npath, int m, int64_t cost, int32_t at, int32_t own,
+                             int32_t last_id, int32_t last_own, bool pages) {
+    const int lane = tid & 31, warp = tid >> 5;
+    if (warp == 0) {
+      for (int b = 0; b < m; b += 32) {
+        const int i = b + lane;
+        int32_t c = 0, x_out = -1, x_in = -1;
+        if (i < m) {
+          c = s_path[i];
+          x_out = s_pathu[i];
+          x_in = arriving(npath, m, i);
+          if (b > 0) {   // (warps 1 and 2 may have written the positions meanwhile)
+            at = s_ppos[i];
+            own = x_in >= 0 ? (int32_t)row(x_in)[c] : 0;
+          }
+          if (x_out >= 0) I.assign[x_out] = (i + 1 < m) ? s_path[i + 1] : j;
+          s_ppos[i] = at;
+        }
+        if (x_out >= 0 && x_in >= 0) {
+          if (at >= 0 && at < s_seg[c]) {
+            int32_t* slot = mslot(c, at, s_seg[c]);
+            slot[0] = x_in;
+            slot[kPage] = own;
+          } else {
+            s_ppos[i] = -1;
+            B->err0 = ST_ERR_INVARIANT;
+          }
+        }
+      }
+      __syncwarp();
+      for (int i = lane; i < m; i += 32) {   // positions, once all old ones were read
+        const int32_t x_in = arriving(npath, m, i);
+        if (s_pathu[i] >= 0 && x_in >= 0 && s_ppos[i] >= 0) pos[x_in] = s_ppos[i];
+      }
+      __syncwarp();
+      if (STRICT && lane == 0) {
+        // centers that only lose or only gain a real unit: a dummy is on the
+        // other side of their pair of edges
+        for (int i = 0; i < m; ++i) {
+          const int32_t c = s_path[i], x_out = s_pathu[i], x_in = arriving(npath, m, i);
+          if (x_out >= 0 && x_in < 0) {
+            const int32_t* sl = mslot(c, s_seg[c] - 1, s_seg[c]);
+            list_remove_at(c, s_ppos[i], sl[0], sl[kPage]);
+            shift_load(c, -1);
+          } else if (x_out < 0 && x_in >= 0) {
+            list_append(c, x_in, (int32_t)row(x_in)[c]);
+            shift_load(c, 1);
+          }
+        }
+      }
+    } else if (npath && warp <= 2 && lane == 0) {
+      if (warp == 1) {
+        list_remove_at(j, at, last_id, last_own);
+        shift_load(j, -1);
+      }
+      if (warp == (pages ? 1 : 2)) {
+        const int32_t term = s_path[m - 1];
+        if (s_pathu[m - 2] >= 0) list_append(term, s_pathu[m - 2], own);
+        else B->err0 = ST_ERR_INVARIANT;
+        shift_load(term, 1);
+      }
+    } else if (warp == 3 && lane == 0) {
+      if (npath) B->paths++;
+      else B->cycles++;
+      B->moves += npath ? m - 1 : m;
+      B->delta += cost;
+    }
   }
 
   // Rows list[0..m) of T against the prices: sets M->bad if an entry breaks
@@ -812,6 +922,20 @@ struct Guided {
       if (__syncthreads_or(any) == 0) return true;
     }
     return false;   // a negative cycle in Gamma: Lemmas 1/2 broken
+  }
+
+  // P(v) up to d1 - l1(v) and, after a second search, d2 - l2(v); P(j) up to d2.
+  __device__ void raise_prices(int32_t j, int64_t d2, int64_t d1, bool second) {
+    for (int v = tid; v < k; v += kThreads) {
+      int64_t p = s_pot[v];
+      if (v == j) {
+        p = max(p, d2);
+      } else {
+        if (s_lab1[v] != kNoLab) p = max(p, d1 - (int64_t)s_lab1[v]);
+        if (second && s_lab2[v] != kNoLab) p = max(p, d2 - (int64_t)s_lab2[v]);
+      }
+      s_pot[v] = clamp32(p);
+    }
   }
 
   // ----------------------------------------------------------- the loop --
@@ -883,7 +1007,6 @@ struct Guided {
       for (int h = 0; h < 6; ++h) B->front_hist[h] = 0;
       M->bad = 0;
       M->stop = 0;
-      M->naff = 0;
     }
     if (TSM || I.ctl[CTL_MIRROR] == 0)
       for (int64_t u = 0; u < k; ++u)
@@ -891,6 +1014,8 @@ struct Guided {
           const int32_t t = cl < k ? tc[u * k + cl] : kTInf;
           tt[u * ws + cl] = (T)(t == kTInf ? kInf : t);
         }
+    if (s_td)
+      for (int64_t i = tid; i < (int64_t)k * k; i += kThreads) s_td[i] = td[i];
     if (tid < kGOrd) load_order(r_begin + tid, r_end, tid);
     __syncthreads();
     bool prices_ok = I.ctl[CTL_POT] != 0;
@@ -935,11 +1060,14 @@ struct Guided {
         const int32_t t = (int32_t)r[cl] - own;
         const int32_t e = edge(j, cl);
         const int32_t bt = e == kInf ? kTInf : e;
-        // equal costs take the lower unit: a reduction nobody waits for (so
-        // td is read past L1 everywhere)
-        if (t < bt) set_entry(j, cl, t, d);
-        else if (t == bt)
-          atomicMin(reinterpret_cast<unsigned*>(td + (int64_t)j * k + cl), (unsigned)d);
+        // equal costs take the lower unit: in global memory a reduction that
+        // nobody waits for
+        if (t < bt) {
+          set_entry(j, cl, t, d);
+        } else if (t == bt) {
+          if (s_td) s_td[j * k + cl] = min(s_td[j * k + cl], d);
+          else atomicMin(reinterpret_cast<unsigned*>(td + (int64_t)j * k + cl), (unsigned)d);
+        }
         viol |= (int64_t)t + s_pot[cl] < (int64_t)pj;
       }
       viol = __syncthreads_or(viol) != 0;
@@ -954,69 +1082,56 @@ struct Guided {
         if (tid == 0) B->skipped++;
         if (!over || pj >= ql) continue;
       }
-      // Alg. 1 and Alg. 4 at j
+      // Alg. 1 and Alg. 4 at j: one search for both, and a second one for
+      // Alg. 4 if a cycle was applied
       if (STRICT) __syncthreads();   // j's vacancy counts the allotment
-      const uint64_t ts0 = timer() ? clock_cycles() : 0;
-      search(j, viol, over, s_lab1, s_pot, ql);
-      if (timer()) B->t_relax += clock_cycles() - ts0;
-      if (M->bad) { status = ST_ERR_INVARIANT; break; }
-      const int64_t cycv = viol ? (int64_t)s_lab1[j] : 0;
-      const uint32_t sink1 = M->sink;
-      const int64_t D1 = over ? (int64_t)M->paid : INT32_MAX;   // exact below ql
-      bool bad = false;
-      if (cycv >= 0) {
-        const int64_t dd = over ? min(D1, (int64_t)ql) : (int64_t)pj;
-        for (int v = tid; v < k; v += kThreads) {
-          if (v == j) s_pot[v] = (int32_t)max((int64_t)pj, dd);
-          else if (s_lab1[v] != kNoLab) s_pot[v] = (int32_t)max((int64_t)s_pot[v], dd - (int64_t)s_lab1[v]);
+      int64_t cycv = 0, d1 = 0;
+      int mc = 0, m2 = 0;
+      bool failed = false;
+      for (int stage = 0; stage < 2; ++stage) {
+        const uint64_t ts0 = timer() ? clock_cycles() : 0;
+        LT* lab = stage ? s_lab2 : s_lab1;
+        search(j, stage == 0 && viol, over, lab, stage ? s_mid : s_pot, ql);
+        if (timer()) B->t_relax += clock_cycles() - ts0;
+        const uint32_t sink = M->sink;
+        const int64_t paid = over ? (int64_t)M->paid : INT32_MAX;   // exact below ql
+        if (stage == 0 && viol) cycv = min((int64_t)0, (int64_t)lab[j]);
+        const bool cycle = stage == 0 && cycv < 0;
+        const bool path = !cycle && over && paid < ql;
+        if (stage == 0) d1 = paid;
+        if (!cycle) {
+          // prices up to the cheapest paid slot, over the labels of both searches
+          const int64_t d2 = over ? min(paid, (int64_t)ql) : (int64_t)pj;
+          raise_prices(j, d2, d2 + cycv, stage == 1);
+          if (stage == 0 && over && tid == 0) B->npath_reused++;
         }
-        if (over && tid == 0) B->npath_reused++;
-        if (over && D1 < ql) {
-          const int m = apply(j, true, (int32_t)(sink1 & ((1u << kGNodeBits) - 1)), s_lab1, D1 - ql);
-          if (m < 0) { status = ST_ERR_INVARIANT; break; }
-          bad = broken_rows(s_path, m);
+        if (M->bad) { failed = true; break; }
+        if (!cycle && !path) break;
+        const int m = apply(j, path, path ? (int32_t)(sink & ((1u << kGNodeBits) - 1)) : -1, lab,
+                            cycle ? cycv : paid - ql);
+        if (m < 0) { failed = true; break; }
+        if (path) {
+          m2 = m;
+          break;
         }
-      } else {
-        const int mc = apply(j, false, -1, s_lab1, cycv);
-        if (mc < 0) { status = ST_ERR_INVARIANT; break; }
+        mc = m;
         for (int i = tid; i < mc; i += kThreads) s_cpath[i] = s_path[i];
-        int64_t d2 = 0, D2 = 0;
-        int m2 = 0;
-        if (over) {
-          const int64_t dt = pj + cycv;
-          const uint64_t ts1 = timer() ? clock_cycles() : 0;
-          const int64_t off = max((int64_t)0, dt - D1);
-          for (int v = tid; v < k; v += kThreads) {
-            int64_t p = s_pot[v];
-            if (v != j && s_lab1[v] != kNoLab) p = max(p, dt - (int64_t)s_lab1[v]);
-            s_mid[v] = (int32_t)max(p - off, (int64_t)-kGPenLimit);
-          }
-          search(j, false, true, s_lab2, s_mid, ql);
-          if (timer()) B->t_relax += clock_cycles() - ts1;
-          if (M->bad) { status = ST_ERR_INVARIANT; break; }
-          D2 = M->paid;
-          d2 = min((int64_t)ql, D2);
+        if (!over) {
+          raise_prices(j, pj, pj + cycv, false);
+          break;
         }
-        const uint32_t sink2 = M->sink;
-        if (!over) d2 = pj;
-        const int64_t dd = cycv + d2;
+        // bounds for the second search: prices raised by the first labels,
+        // less the most by which those exceed q_n
+        const int64_t dt = pj + cycv, off = max((int64_t)0, dt - d1);
         for (int v = tid; v < k; v += kThreads) {
           int64_t p = s_pot[v];
-          if (v == j) {
-            p = max((int64_t)pj, d2);
-          } else {
-            if (s_lab1[v] != kNoLab) p = max(p, dd - (int64_t)s_lab1[v]);
-            if (over && s_lab2[v] != kNoLab) p = max(p, d2 - (int64_t)s_lab2[v]);
-          }
-          s_pot[v] = clamp32(p);
+          if (v != j && s_lab1[v] != kNoLab) p = max(p, dt - (int64_t)s_lab1[v]);
+          s_mid[v] = (int32_t)max(p - off, (int64_t)-kGPenLimit);
         }
-        if (over && D2 < ql) {
-          m2 = apply(j, true, (int32_t)(sink2 & ((1u << kGNodeBits) - 1)), s_lab2, D2 - ql);
-          if (m2 < 0) { status = ST_ERR_INVARIANT; break; }
-        }
-        __syncthreads();   // prices and rows are final
-        bad = broken_rows(s_cpath, mc) | broken_rows(s_path, m2);
       }
+      if (failed) { status = ST_ERR_INVARIANT; break; }
+      __syncthreads();   // prices, loads and rows are final
+      const bool bad = broken_rows(s_cpath, mc) | broken_rows(s_path, m2);
       if (__syncthreads_or(bad)) prices_ok = false;   // rebuilt before the next round
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -1026,6 +1141,14 @@ struct Guided {
       I.load[v] = s_slack[v] + __ldg(I.cap + v);
       I.seg_size[v] = s_seg[v];
     }
+    if (s_td)
+      for (int64_t i = tid; i < (int64_t)k * k; i += kThreads) td[i] = s_td[i];
+    if (TSM)
+      for (int64_t u = 0; u < k; ++u)
+        for (int cl = tid; cl < k; cl += kThreads) {
+          const int32_t t = tt[u * ws + cl];
+          tc[u * k + cl] = t == kInf ? kTInf : t;
+        }
     if (tid == 0) {
       I.ctl[CTL_POT] = prices_ok && status == ST_OK ? 1 : 0;
       if (count > 0) I.ctl[CTL_MIRROR] = TSM ? 0 : 1;

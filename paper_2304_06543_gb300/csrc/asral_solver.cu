@@ -1619,14 +1619,19 @@ asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_coun
       S.c1 = min(S.k, S.c0 + S.w);
       S.wr = max(0, S.c1 - S.c0);
       S.s_red = smem + L.ring;
-      S.prologue();   // every CTA has read CTL_PROLOGUE by its cluster barriers
+      // the mirror of an empty table (a share per CTA; the cluster barriers of
+      // the prologue publish it, and every CTA has read CTL_PROLOGUE by then)
+      const int64_t ents = (int64_t)s_inst.k * guided_stride(s_inst.k, (int)sizeof(T));
+      for (int64_t i = (int64_t)rank * kThreads + tid; i < ents; i += (int64_t)C * kThreads)
+        static_cast<T*>(s_inst.mirror)[i] = (T)Solver<T>::kTsInf;
+      S.prologue();
       for (int v = tid; v < s_inst.k && rank == 0; v += kThreads) s_inst.pot[v] = 0;
       if (rank == 0 && tid == 0) {
         s_inst.ctl[CTL_FREE_TOP] = s_inst.npages;
         s_inst.ctl[CTL_ROUNDS] = 0;
         s_inst.ctl[CTL_DELTA] = 0;
         s_inst.ctl[CTL_POT] = 1;
-        s_inst.ctl[CTL_MIRROR] = 0;
+        s_inst.ctl[CTL_MIRROR] = 1;
         s_inst.ctl[CTL_PROLOGUE] = 1;
         s_inst.ctl[CTL_T_PROLOGUE] += gtimer_ns() - t0;
       }
@@ -1634,23 +1639,27 @@ asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_coun
     }
     if (rank != 0) continue;   // waits at the next instance's barrier
     const bool tsm = L.total <= avail && !(flags & OPT_NO_TC_SMEM);
+    const bool usm = tsm && L.full <= avail;
     auto rounds = [&](auto G) { G.run_rounds(s_deadline); };
     if (flags & OPT_STRICT) {
-      if (tsm) rounds(Guided<T, true, true>(s_inst, smem, L, &s_book, flags));
-      else rounds(Guided<T, false, true>(s_inst, smem, L, &s_book, flags));
+      if (tsm) rounds(Guided<T, true, true>(s_inst, smem, L, usm, &s_book, flags));
+      else rounds(Guided<T, false, true>(s_inst, smem, L, false, &s_book, flags));
     } else {
-      if (tsm) rounds(Guided<T, true, false>(s_inst, smem, L, &s_book, flags));
-      else rounds(Guided<T, false, false>(s_inst, smem, L, &s_book, flags));
+      if (tsm) rounds(Guided<T, true, false>(s_inst, smem, L, usm, &s_book, flags));
+      else rounds(Guided<T, false, false>(s_inst, smem, L, false, &s_book, flags));
     }
   }
 }
 
-// Shared memory of a guided CTA for k centers (with the cost slice of T
-// when that fits `limit`), 0 if it does not fit.
+// Shared memory of a guided CTA for k centers (with the costs and the units
+// of T as far as they fit `limit`), 0 if it does not fit.
 size_t guided_smem_bytes(int32_t k, int elem_bytes, size_t limit) {
   if (k >= 1 << kGNodeBits) return 0;
   const GLayout L = make_guided_layout(k, elem_bytes);
-  return L.total <= limit ? L.total : L.base_total <= limit ? L.base_total : 0;
+  return L.full <= limit         ? L.full
+         : L.total <= limit      ? L.total
+         : L.base_total <= limit ? L.base_total
+                                 : 0;
 }
 
 int32_t guided_pen_limit() { return kGPenLimit; }
