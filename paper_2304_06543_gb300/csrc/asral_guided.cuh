@@ -149,6 +149,9 @@ template <typename T, bool TSM, bool STRICT>
 struct Guided {
   using LT = typename Solver<T>::LT;
   using Ent = GEnt<LT>;
+  // Sums of a label, a price and a penalty: 32 bits with int16 costs (labels
+  // stay below 2^28, the others below 2^30).
+  using PT = LT;
   static constexpr int VPL = 16 / (int)sizeof(T);
   static constexpr int32_t kInf = Solver<T>::kTsInf;
   static constexpr LT kNoLab = Solver<T>::kNoLab;
@@ -604,7 +607,7 @@ struct Guided {
     const int nblk = (k + 31) >> 5;
     for (int i0 = 0; i0 < m; i0 += chunk) {
       const int i1 = min(m, i0 + chunk), units = (i1 - i0) * nblk;
-      list_affected(npath, m, i0, units, nblk);
+      list_affected(i0, units, nblk);
       __syncthreads();
       const uint64_t t1 = timer() ? clock_cycles() : 0;
       if (timer() && i0 == 0) B->t_apply += t1 - t0;
@@ -612,13 +615,16 @@ struct Guided {
       const int i = i0 + lane;
       const int na = i < i1 ? s_raff[i] : 0;
       const int len = na > 0 ? s_seg[s_path[i]] : 0;
-      const int le = na > 16 ? 5 : na > 8 ? 4 : na > 4 ? 3 : na > 2 ? 2 : na > 1 ? 1 : 0;
+      // (at least two entries' lanes: a part then stays within a page)
+      const int le = na > 16 ? 5 : na > 8 ? 4 : na > 4 ? 3 : na > 2 ? 2 : 1;
+      static_assert((kScanU << 4) <= kPage, "a part of a member list lies in one page");
       const int parts = na > 0 ? max(1, (len + (kScanU << (5 - le)) - 1) / (kScanU << (5 - le))) : 0;
       const bool split = __any_sync(0xffffffffu, parts > 1);
       if (warp == 0) {
         const int rows = __reduce_add_sync(0xffffffffu, len);
         if (lane == 0) B->col_rows += rows;
-      } else {
+      }
+      {
         int incl = ((na + 31) >> 5) * parts;
         const int mine = incl;
         if (__any_sync(0xffffffffu, na > 0)) {
@@ -631,7 +637,7 @@ struct Guided {
         const int tasks = __shfl_sync(0xffffffffu, incl, 31);
         // scan tasks first, then batches of kMergeU blocks of 32 columns
         const int items = tasks + (units + kMergeU - 1) / kMergeU;
-        for (int t = warp - 1; t < items; t += kWarps - 1) {
+        for (int t = warp; t < items; t += kWarps) {
           if (t < tasks) {
             const int r = __popc(__ballot_sync(0xffffffffu, incl <= t));
             const int na_r = __shfl_sync(0xffffffffu, na, r), len_r = __shfl_sync(0xffffffffu, len, r);
@@ -661,44 +667,47 @@ struct Guided {
     return m;
   }
 
-  static constexpr int kScanU = 8;    // members in flight per lane
+  static constexpr int kScanU = 16;   // members in flight per lane
   static constexpr int kMergeU = 4;   // column blocks in flight per warp
 
   // The affected entries of rows i0...: s_aff[row][...] columns, their number
   // in s_raff, their running minima reset.
-  __device__ void list_affected(bool npath, int m, int i0, int units, int nblk) {
+  __device__ void list_affected(int i0, int units, int nblk) {
+    if (s_td) list_affected_by<1>(i0, units, nblk);
+    else list_affected_by<kMergeU>(i0, units, nblk);
+  }
+  // U blocks of 32 entries in flight per warp (the units' latency).
+  template <int U>
+  __device__ __forceinline__ void list_affected_by(int i0, int units, int nblk) {
     const int lane = tid & 31;
     const int dr = kWarps / nblk, db = kWarps - dr * nblk;
     int w = tid >> 5;
     int r = w / nblk, blk = w - r * nblk;
+#pragma unroll 1
     while (w < units) {
-      int32_t bd[kMergeU], rr[kMergeU], vv[kMergeU];
+      int32_t bd[U], rr[U], vv[U];
 #pragma unroll
-      for (int q = 0; q < kMergeU; ++q) {
+      for (int q = 0; q < U; ++q) {
         rr[q] = w < units ? r : -1;
         vv[q] = blk * 32 + lane;
         bd[q] = -1;
-        if (rr[q] >= 0 && vv[q] < k && s_pathu[i0 + r] >= 0) bd[q] = unit(s_path[i0 + r], vv[q]);
+        if (rr[q] >= 0 && vv[q] < k && s_pathu[i0 + r] >= 0)
+          bd[q] = U == 1 ? s_td[s_path[i0 + r] * k + vv[q]]
+                         : __ldcg(td + (int64_t)s_path[i0 + r] * k + vv[q]);
         w += kWarps;
         r += dr;
         blk += db;
         if (blk >= nblk) { blk -= nblk; ++r; }
       }
 #pragma unroll
-      for (int q = 0; q < kMergeU; ++q) {
+      for (int q = 0; q < U; ++q) {
         if (rr[q] < 0) break;
         const int i = i0 + rr[q];
         const bool hit = bd[q] >= 0 && bd[q] == s_pathu[i] && vv[q] != s_path[i];
-        const unsigned bits = __ballot_sync(0xffffffffu, hit);
-        if (bits) {
-          int at = 0;
-          const int leader = __ffs(bits) - 1;
-          if (lane == leader) at = atomicAdd(&s_raff[i], __popc(bits));
-          at = __shfl_sync(0xffffffffu, at, leader) + __popc(bits & ((1u << lane) - 1u));
-          if (hit) {
-            s_aff[rr[q] * k + at] = vv[q];
-            best_of(rr[q] * k + at) = ~0ull;
-          }
+        if (hit) {
+          const int at = rr[q] * k + atomicAdd(&s_raff[i], 1);
+          s_aff[at] = vv[q];
+          best_of(at) = ~0ull;
         }
       }
     }
@@ -716,7 +725,7 @@ struct Guided {
   }
 
   // A block of at most 32 affected entries of row i0 + r over one part of its
-  // center's member list: lane = (entry, member of eight in flight), with as
+  // center's member list: lane = (entry, member of sixteen in flight), with as
   // many lanes per entry as the block leaves, so that few entries of a long
   // list (a large center) still fill the warps and many entries of a short
   // one read neighbouring columns of the same rows.  Lists of more than one
@@ -884,7 +893,7 @@ struct Guided {
       const int32_t c = list[i];
       if (v < k && v != c) {
         const int32_t t = arc(c, v);
-        if (t != kInf && (int64_t)s_pot[c] > (int64_t)t + s_pot[v]) bad = true;
+        if (t != kInf && (PT)s_pot[c] > (PT)t + s_pot[v]) bad = true;
       } else if (v == c && !STRICT && s_pot[c] > s_qn[c]) {
         bad = true;
       }
@@ -925,16 +934,16 @@ struct Guided {
   }
 
   // P(v) up to d1 - l1(v) and, after a second search, d2 - l2(v); P(j) up to d2.
-  __device__ void raise_prices(int32_t j, int64_t d2, int64_t d1, bool second) {
+  __device__ void raise_prices(int32_t j, PT d2, PT d1, bool second) {
     for (int v = tid; v < k; v += kThreads) {
-      int64_t p = s_pot[v];
+      PT p = s_pot[v];
       if (v == j) {
         p = max(p, d2);
       } else {
-        if (s_lab1[v] != kNoLab) p = max(p, d1 - (int64_t)s_lab1[v]);
-        if (second && s_lab2[v] != kNoLab) p = max(p, d2 - (int64_t)s_lab2[v]);
+        if (s_lab1[v] != kNoLab) p = max(p, d1 - (PT)s_lab1[v]);
+        if (second && s_lab2[v] != kNoLab) p = max(p, d2 - (PT)s_lab2[v]);
       }
-      s_pot[v] = clamp32(p);
+      s_pot[v] = (int32_t)p;
     }
   }
 
@@ -1068,7 +1077,7 @@ struct Guided {
           if (s_td) s_td[j * k + cl] = min(s_td[j * k + cl], d);
           else atomicMin(reinterpret_cast<unsigned*>(td + (int64_t)j * k + cl), (unsigned)d);
         }
-        viol |= (int64_t)t + s_pot[cl] < (int64_t)pj;
+        viol |= (PT)t + s_pot[cl] < (PT)pj;
       }
       viol = __syncthreads_or(viol) != 0;
       if (tid == kThreads - 32) {
@@ -1085,7 +1094,7 @@ struct Guided {
       // Alg. 1 and Alg. 4 at j: one search for both, and a second one for
       // Alg. 4 if a cycle was applied
       if (STRICT) __syncthreads();   // j's vacancy counts the allotment
-      int64_t cycv = 0, d1 = 0;
+      PT cycv = 0, d1 = 0;
       int mc = 0, m2 = 0;
       bool failed = false;
       for (int stage = 0; stage < 2; ++stage) {
@@ -1094,14 +1103,14 @@ struct Guided {
         search(j, stage == 0 && viol, over, lab, stage ? s_mid : s_pot, ql);
         if (timer()) B->t_relax += clock_cycles() - ts0;
         const uint32_t sink = M->sink;
-        const int64_t paid = over ? (int64_t)M->paid : INT32_MAX;   // exact below ql
-        if (stage == 0 && viol) cycv = min((int64_t)0, (int64_t)lab[j]);
+        const PT paid = over ? (PT)M->paid : (PT)kGNever;   // exact below ql
+        if (stage == 0 && viol) cycv = min((PT)0, (PT)lab[j]);
         const bool cycle = stage == 0 && cycv < 0;
         const bool path = !cycle && over && paid < ql;
         if (stage == 0) d1 = paid;
         if (!cycle) {
           // prices up to the cheapest paid slot, over the labels of both searches
-          const int64_t d2 = over ? min(paid, (int64_t)ql) : (int64_t)pj;
+          const PT d2 = over ? min(paid, (PT)ql) : (PT)pj;
           raise_prices(j, d2, d2 + cycv, stage == 1);
           if (stage == 0 && over && tid == 0) B->npath_reused++;
         }
@@ -1122,11 +1131,11 @@ struct Guided {
         }
         // bounds for the second search: prices raised by the first labels,
         // less the most by which those exceed q_n
-        const int64_t dt = pj + cycv, off = max((int64_t)0, dt - d1);
+        const PT dt = pj + cycv, off = max((PT)0, dt - d1);
         for (int v = tid; v < k; v += kThreads) {
-          int64_t p = s_pot[v];
-          if (v != j && s_lab1[v] != kNoLab) p = max(p, dt - (int64_t)s_lab1[v]);
-          s_mid[v] = (int32_t)max(p - off, (int64_t)-kGPenLimit);
+          PT p = s_pot[v];
+          if (v != j && s_lab1[v] != kNoLab) p = max(p, dt - (PT)s_lab1[v]);
+          s_mid[v] = (int32_t)max(p - off, (PT)-kGPenLimit);
         }
       }
       if (failed) { status = ST_ERR_INVARIANT; break; }

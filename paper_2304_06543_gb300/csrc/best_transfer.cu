@@ -983,8 +983,8 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
 // batch to batch, so a later equal t never replaces the unit.
 constexpr int kTableThreads = 1024;         // 32-bit keys: short batches, many warps
 constexpr int kTableUnroll = 4;             // vectors in flight per thread
-constexpr int kWideThreads = 512;           // two words: twice the registers, batches of 8
-constexpr int kWideUnroll = 8;
+constexpr int kWideThreads = 640;           // two words: two batches of 4 in registers
+constexpr int kWideUnroll = 4;
 constexpr int kTableCluster = 4;
 constexpr int64_t kTableOneCluster = 4 << 20;
 constexpr size_t kTableSmem = 200 * 1024;
@@ -1175,22 +1175,35 @@ bt_scan_table_wide(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
     const uint32_t w = (&x.x)[sizeof(T) == 4 ? h : h / 2];
     return sizeof(T) == 4 ? (int32_t)w : (h & 1) ? (int32_t)w >> 16 : (int32_t)(int16_t)w;
   };
+  uint4 xn[U];          // the next batch, in flight while this one goes through
+  int32_t an[U], gn[U];
+  uint32_t rn[U];
+  auto fetch = [&]() {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      rn[u] = (uint32_t)r;
+      gn[u] = g;
+      an[u] = -1;
+      if (r < P.R1) {
+        xn[u] = __ldg(reinterpret_cast<const uint4*>(cm + r * ld + P.c0) + g);
+        an[u] = __ldg(assign + r);
+      }
+      r += dr;
+      g += dg;
+      if (g >= gw) { g -= gw; ++r; }
+    }
+  };
+  fetch();
   for (int64_t b = 0; b < batches; ++b) {
     uint4 x[U];
     int32_t a[U], own[U], at[U];
     uint32_t rr[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      rr[u] = (uint32_t)r;
-      at[u] = g;
-      a[u] = -1;
-      if (r < P.R1) {
-        x[u] = __ldg(reinterpret_cast<const uint4*>(cm + r * ld + P.c0) + g);
-        a[u] = __ldg(assign + r);
-      }
-      r += dr;
-      g += dg;
-      if (g >= gw) { g -= gw; ++r; }
+      x[u] = xn[u];
+      a[u] = an[u];
+      at[u] = gn[u];
+      rr[u] = rn[u];
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -1202,6 +1215,7 @@ bt_scan_table_wide(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
         at[u] = -1;
       }
     }
+    fetch();
     uint32_t maybe = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {

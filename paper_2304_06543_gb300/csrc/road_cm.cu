@@ -102,6 +102,30 @@ static size_t road_smem_bytes(int32_t V) {
 // decides whether the neighbour is listed; one that was lowered further in
 // between is listed all the same).  65,536 nodes, 109 centers: 6.6 ms per
 // call with one list and marks in global memory, 1.8 ms now.
+// Sets `bit` of a bitmap word where `on`; returns the word as it was (all ones
+// where not).  Predicated instead of branched around, so that the atomics of
+// a node's edges are in flight together.
+template <bool SMEM>
+__device__ __forceinline__ uint32_t mark_if(bool on, uint32_t* word, uint32_t bit) {
+  uint32_t old;
+  if constexpr (SMEM)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.u32 %0, 0xffffffff;\n\t"
+        "@p atom.shared.or.b32 %0, [%1], %2;\n\t}"
+        : "=r"(old) : "r"(smem_u32(word)), "r"(bit), "r"((uint32_t)on) : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.u32 %0, 0xffffffff;\n\t"
+        "@p atom.global.or.b32 %0, [%1], %2;\n\t}"
+        : "=r"(old) : "l"(word), "r"(bit), "r"((uint32_t)on) : "memory");
+  return old;
+}
+__device__ __forceinline__ void lower_if(bool on, int32_t* label, int32_t v) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.global.min.s32 [%0], %1;\n\t}"
+               ::"l"(label), "r"(v), "r"((uint32_t)on) : "memory");
+}
+
+template <bool SMEM>
 __global__ void __launch_bounds__(kRoadThreads)
 road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
           const int32_t* __restrict__ w, const int2* __restrict__ adj, int32_t k,
@@ -112,8 +136,7 @@ road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restr
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t words = road_bitmap_words(V);
   int32_t* sq = reinterpret_cast<int32_t*>(road_smem);            // [3][kRoadQueue]
-  uint32_t* bits = V <= kRoadSmemNodes ? road_smem + 3 * kRoadQueue
-                                       : marks + 3 * words * blockIdx.x;   // [3][words]
+  uint32_t* bits = SMEM ? road_smem + 3 * kRoadQueue : marks + 3 * words * blockIdx.x;   // [3][words]
   uint32_t* far_bits = bits + 2 * words;
   int32_t* gq = queues + (int64_t)blockIdx.x * 3 * V;             // [3][V]
   auto item = [&](int list, int i) {
@@ -214,15 +237,21 @@ road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restr
         for (;;) {
 #pragma unroll
           for (int q = 0; q < U; ++q) dv[q] = v[q] >= 0 ? __ldcg(d + v[q]) : INT32_MIN;
-          unsigned near = 0, far = 0;
+          uint32_t old[U];
 #pragma unroll
           for (int q = 0; q < U; ++q) {
             nd[q] += du;
-            if (nd[q] < dv[q]) {
-              atomicMin(d + v[q], nd[q]);
-              const uint32_t bit = 1u << (v[q] & 31);
-              if (nd[q] < T) near |= (atomicOr(bout + (v[q] >> 5), bit) & bit) == 0 ? 1u << q : 0u;
-              else far |= (atomicOr(far_bits + (v[q] >> 5), bit) & bit) == 0 ? 1u << q : 0u;
+            const bool on = nd[q] < dv[q];
+            const int32_t x = on ? v[q] : 0;
+            lower_if(on, d + x, nd[q]);
+            old[q] = mark_if<SMEM>(on, (nd[q] < T ? bout : far_bits) + (x >> 5), 1u << (x & 31));
+          }
+          unsigned near = 0, far = 0;
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            if (!(old[q] >> (v[q] & 31) & 1)) {   // all ones where nothing was lowered
+              if (nd[q] < T) near |= 1u << q;
+              else far |= 1u << q;
             }
           }
           int an = near ? atomicAdd(&s_near[c3], __popc(near)) : 0;
@@ -299,15 +328,10 @@ extern "C" int lbdd_road_cm(int32_t V, const int32_t* row_ptr, const int32_t* co
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int grid = std::min(k, sms);
-  int32_t *dist = nullptr, *queues = nullptr;
-  int2* adj = nullptr;
-  uint32_t* marks = nullptr;   // frontier bitmaps that shared memory does not hold
+  unsigned char* base = nullptr;
   int* err = nullptr;
   auto release = [&]() {
-    cudaFreeAsync(dist, st);
-    cudaFreeAsync(queues, st);
-    cudaFreeAsync(adj, st);
-    if (marks) cudaFreeAsync(marks, st);
+    if (base) cudaFreeAsync(base, st);
     cudaFreeAsync(err, st);
     cudaStreamSynchronize(st);
   };
@@ -323,11 +347,16 @@ extern "C" int lbdd_road_cm(int32_t V, const int32_t* row_ptr, const int32_t* co
   if (e) { rc = cuda_fail(e, "lbdd_road_cm check"); release(); return rc; }
   // labels are int32: every path length must fit
   if (h[0] != 0 || (int64_t)h[1] * (V - 1) >= (int64_t)kRoadInf) { release(); return LBDD_ERR_ARG; }
-  e = cudaMallocAsync(reinterpret_cast<void**>(&dist), 4ull * k * V, st);
-  if (!e) e = cudaMallocAsync(reinterpret_cast<void**>(&queues), 12ull * grid * V, st);
-  if (!e) e = cudaMallocAsync(reinterpret_cast<void**>(&adj), sizeof(int2) * kRoadDeg * (size_t)V, st);
-  if (!e && V > kRoadSmemNodes)
-    e = cudaMallocAsync(reinterpret_cast<void**>(&marks), 12ull * grid * road_bitmap_words(V), st);
+  // one allocation for all scratch
+  auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  const size_t o_queues = al(4ull * k * V), o_adj = o_queues + al(12ull * grid * V);
+  const size_t o_marks = o_adj + al(sizeof(int2) * kRoadDeg * (size_t)V);
+  const size_t o_end = o_marks + (V > kRoadSmemNodes ? 12ull * grid * road_bitmap_words(V) : 0);
+  e = cudaMallocAsync(reinterpret_cast<void**>(&base), o_end, st);
+  int32_t* dist = reinterpret_cast<int32_t*>(base);
+  int32_t* queues = reinterpret_cast<int32_t*>(base + o_queues);
+  int2* adj = reinterpret_cast<int2*>(base + o_adj);
+  uint32_t* marks = reinterpret_cast<uint32_t*>(base + o_marks);   // bitmaps past shared memory
   const size_t smem = road_smem_bytes(V);
   // threshold step: four mean lengths (1.05 to 1.1 relaxations per node on
   // grids; half as much takes a fifth more steps, twice as much 1.2
@@ -336,13 +365,14 @@ extern "C" int lbdd_road_cm(int32_t V, const int32_t* row_ptr, const int32_t* co
   std::memcpy(&sum, h + 4, sizeof(sum));
   const uint64_t roads = (uint64_t)std::max(1, h[6]);
   const int32_t delta = (int32_t)std::min<uint64_t>(1u << 30, std::max<uint64_t>(1, 4 * sum / roads));
+  auto sssp = V <= kRoadSmemNodes ? road_sssp<true> : road_sssp<false>;
   if (!e)   // the largest any graph asks for
-    e = cudaFuncSetAttribute(road_sssp, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(sssp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)road_smem_bytes(kRoadSmemNodes));
   if (!e) {
     road_pack<<<sms * 8, 256, 0, st>>>(V, row_ptr, col, w, adj);
-    road_sssp<<<grid, kRoadThreads, smem, st>>>(V, row_ptr, col, w, adj, k, centers, delta, dist,
-                                                queues, marks, err);
+    sssp<<<grid, kRoadThreads, smem, st>>>(V, row_ptr, col, w, adj, k, centers, delta, dist, queues,
+                                           marks, err);
     e = cudaGetLastError();
   }
   if (!e) {
