@@ -61,13 +61,15 @@ typedef struct lbdd_stats {
   int64_t rounds;           /* rounds of Alg. 2 completed */
   int64_t cycles_applied;   /* negative cycles removed (Alg. 1) */
   int64_t paths_applied;    /* negative paths removed (Alg. 4) */
-  int64_t bf_calls;         /* Bellman-Ford runs to convergence */
+  int64_t bf_calls;         /* Bellman-Ford runs (one pruned run may answer Alg. 1
+                               and Alg. 4 of a round) */
   int64_t bf_sweeps;        /* synchronous sweeps over all those runs */
   int64_t bf_max_sweeps;    /* longest run, in sweeps */
   int64_t moves;            /* demand units transferred between centers */
   int64_t ncyc_skipped;     /* Alg. 1 calls answered without Bellman-Ford because
-                               the new unit lowered no best-transfer cost */
-  int64_t rows_scanned;     /* CM rows read by best-transfer segment rescans */
+                               the new unit's edges break no price of a center, or
+                               it lowered no best-transfer cost */
+  int64_t rows_scanned;     /* CM rows read by whole-row segment rescans */
   int64_t cm_elem_bytes;    /* 2 or 4: element size of the stored CM */
   int64_t cluster_size;     /* CTAs per thread-block cluster used by solves */
   /* Device-side phase timers of the cluster's first CTA, nanoseconds summed
@@ -84,8 +86,8 @@ typedef struct lbdd_stats {
   int64_t relax_reduce_ns;  /* part of relax_ns: loop + cross-warp reduction and record */
   int64_t cost_slice_in_smem; /* 1 if the last solve kept each CTA's best-transfer cost
                                  columns in shared memory */
-  int64_t npath_reused;     /* Alg. 4 calls answered from the labels of an Alg. 1
-                               Bellman-Ford that applied nothing (exact: same graph
+  int64_t npath_reused;     /* Alg. 4 calls answered from the labels of Alg. 1's
+                               Bellman-Ford, which applied nothing (exact: same graph
                                except for the sink edges) */
   int64_t col_rows;         /* member rows read by column-subset rescans */
   int64_t front_sum;        /* sum over sweeps of the Bellman-Ford frontier size */
@@ -96,14 +98,14 @@ typedef struct lbdd_stats {
 typedef enum lbdd_option {
   LBDD_OPT_CLUSTER = 1,     /* CTAs per cluster for lbdd_solve: 1, 2, 4, 8 or 16
                                (0 = auto) */
-  LBDD_OPT_NCYC_SKIP = 2,   /* 1 (default): skip Alg. 1's Bellman-Ford when the new
-                               unit lowers no best-transfer cost (exact by Lemma 1);
-                               0: always run it */
+  LBDD_OPT_NCYC_SKIP = 2,   /* 1 (default): skip or prune Alg. 1's Bellman-Ford where
+                               prices of the centers, or an unchanged table, show that
+                               it cannot change the result; 0: always run it in full */
   LBDD_OPT_TC_SMEM = 4,     /* 1 (default): keep each CTA's best-transfer cost columns in
                                shared memory when they fit; 0: read them from global memory */
   LBDD_OPT_NPATH_REUSE = 3, /* 1 (default): answer Alg. 4 from the converged labels of
                                an Alg. 1 run that applied nothing; 0: always run a
-                               separate Bellman-Ford */
+                               separate, unpruned Bellman-Ford */
   LBDD_OPT_PHASE_TIMERS = 5,/* 0 (default): only the total time of the rounds is kept;
                                1: also time every phase (the *_ns fields of lbdd_stats
                                and the frontier counters), which slows the rounds */
@@ -411,7 +413,7 @@ int lbdd_best_transfer_noalloc(int32_t n, int32_t k, const void* cm_dev, int cm_
  *   cm (n x ld)  : output, int32, CM[d * ld + s] = shortest path length from
  *                  centers[s] to demand[d] (ld >= k).
  * All arrays are device memory; work is ordered on `stream` and the call
- * waits for it.  Scratch (k x V labels and per-CTA frontier queues) is
+ * waits for it.  Scratch (k x V labels, per-CTA lists, packed edges) is
  * allocated from the stream-ordered pool and freed before returning.
  * Errors: LBDD_ERR_ARG (bad graph or ids, lengths that could overflow, a
  * demand node no center reaches, a demand node that is a center's node:

@@ -39,18 +39,28 @@
 //
 // What this buys (counted on instances of the city shape, 8,000 x 500, and of
 // the batched mix, 6,007 x 126): 48 sweeps of 180 labels and 19 sweeps of 52
-// per round become 22 sweeps of 12 labels and 8 of 12; half of the mix's
-// rounds run no sweep at all.
+// per round become 10 sweeps of about 30 labels and 3 of about 16; half of the
+// mix's rounds run no sweep at all.  Per call, against the cluster solver on
+// the CTAs it did best on: 317 -> 44 ms for the mix instance, 1,230 -> 289 ms
+// for the city, 37.0 -> 10.3 ms for 2,000 x 20, 540 -> 38 ms for 24 mixed
+// instances in one launch (a cluster each before, a CTA each now).
+//
+// Bound by the chain of dependent instructions and reads of a round: a warp
+// that runs alone issues about one instruction in five cycles, a dependent
+// global read takes about half a microsecond.  A round that ends at the tests
+// takes about 1 us, a sweep 0.6 to 1.4 us, an applied path 4 to 10 us.
 //
 // Layout.  A frontier of a dozen labels is too little work to spread over a
 // cluster: one CTA runs the whole round.  Thread t owns columns t, t + 512,
 // ...; every thread reads the whole frontier list (broadcast loads) and keeps
 // its own column's minimum, so a sweep needs one barrier of the ceil(k / 32)
-// warps that own a column and no cross-warp reduction.  Labels that improved
-// are appended to the next list by one shared-memory atomic per warp (order
-// inside a list does not matter: equal labels take the lower node).  The
-// costs of T sit in shared memory as T (int16 or int32) when they fit beside
-// the rest, otherwise they are read from the global table through L1.
+// warps that own a column and no cross-warp reduction.  A label that improved
+// is appended to the next list by its own lane's shared-memory atomic; the
+// order inside a list does not matter, because only labels and hop counts are
+// kept and `follow` looks up the lowest parent of each node of the one path
+// that is applied.  The costs of T sit in shared memory as T (int16 or int32)
+// when they fit beside the rest, otherwise they are read from the global
+// table through L1; its units too, where both fit.
 #pragma once
 
 namespace lbdd {
@@ -1103,7 +1113,7 @@ struct Guided {
         search(j, stage == 0 && viol, over, lab, stage ? s_mid : s_pot, ql);
         if (timer()) B->t_relax += clock_cycles() - ts0;
         const uint32_t sink = M->sink;
-        const PT paid = over ? (PT)M->paid : (PT)kGNever;   // exact below ql
+        const PT paid = over ? (PT)min(M->paid, kGNever) : (PT)kGNever;   // exact below ql
         if (stage == 0 && viol) cycv = min((PT)0, (PT)lab[j]);
         const bool cycle = stage == 0 && cycv < 0;
         const bool path = !cycle && over && paid < ql;

@@ -220,7 +220,7 @@ constexpr int32_t kGuidedMaxK = 1024;
 
 static int fits(const lbdd_solver* s, int C) { return fits_k(s->k, s->elem, C) ? 1 : 0; }
 
-size_t lbdd::solver_footprint(int32_t n, int32_t k, int in_elem, int elem) {
+size_t lbdd::solver_footprint(int32_t n, int32_t k, int in_elem, int elem, bool guided) {
   auto a = [](size_t b) { return (std::max<size_t>(b, 16) + 511) / 512 * 512; };
   const int dt_in = in_elem == 2 ? LBDD_CM_I16 : LBDD_CM_I32;
   const int dt = elem == 2 ? LBDD_CM_I16 : LBDD_CM_I32;
@@ -235,14 +235,14 @@ size_t lbdd::solver_footprint(int32_t n, int32_t k, int in_elem, int elem) {
   b += 3 * a(4ull * k);                       // load, seg_size, pot
   b += a(4ull * k * max_pages) + a(4ull * npages * kPageWords) + a(4ull * npages);
   b += 2 * a(4ull * k * k);                   // tc, td
-  if (guided_smem_bytes(k, elem, kMaxSmem) > 0) b += a(guided_mirror_bytes(k, elem));
+  if (guided && guided_smem_bytes(k, elem, kMaxSmem) > 0) b += a(guided_mirror_bytes(k, elem));
   b += a(8ull * CTL_COUNT) + a(16) + a(sizeof(DevInst));
   return b;
 }
 
 static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, int cm_dtype,
                        int cm_is_device, int64_t cm_ld, const int32_t* cap, const int32_t* pen,
-                       void* cuda_stream) {
+                       void* cuda_stream, bool guided = true) {
   if (!out) return LBDD_ERR_ARG;
   *out = nullptr;
   if (n < 1 || k < 1 || !cm || !cap || !pen) return LBDD_ERR_ARG;
@@ -280,8 +280,10 @@ static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, 
   if (!rc) rc = dalloc(s, &s->tc, (size_t)k * k);
   if (!rc) rc = dalloc(s, &s->td, (size_t)k * k);
   if (!rc) rc = dalloc(s, &s->pot, k);
-  if (!rc && guided_smem_bytes(k, s->elem, kMaxSmem) > 0)
-    rc = dev_alloc(s, &s->mirror, guided_mirror_bytes(k, s->elem));
+  // the guided rounds' mirror is optional: without it (no memory left for it)
+  // the solver runs unguided
+  if (!rc && guided && guided_smem_bytes(k, s->elem, kMaxSmem) > 0)
+    (void)dev_alloc(s, &s->mirror, guided_mirror_bytes(k, s->elem));
   if (!rc) rc = dalloc(s, &s->ctl, CTL_COUNT);
   if (!rc) rc = dalloc(s, &s->counter, 4);
   if (!rc) rc = dalloc(s, &s->d_inst, 1);
@@ -315,6 +317,12 @@ extern "C" int lbdd_create(lbdd_solver** out, int32_t n, int32_t k, const void* 
                            int cm_is_device, const int32_t* cap, const int32_t* pen,
                            void* cuda_stream) {
   return create_impl(out, n, k, cm, cm_dtype, cm_is_device, k, cap, pen, cuda_stream);
+}
+
+int lbdd::create_unguided(lbdd_solver** out, int32_t n, int32_t k, const void* cm, int cm_dtype,
+                          int cm_is_device, const int32_t* cap, const int32_t* pen,
+                          void* cuda_stream) {
+  return create_impl(out, n, k, cm, cm_dtype, cm_is_device, k, cap, pen, cuda_stream, false);
 }
 
 // Extended cost matrix of Alg. 5: the caller's n x k costs widened to int32,

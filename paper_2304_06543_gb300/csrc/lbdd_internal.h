@@ -92,7 +92,11 @@ int status_to_rc(int64_t st);
 // Device bytes lbdd_create allocates for an n x k instance whose costs are
 // stored with elem-byte entries (in_elem: entry size of the caller's CM,
 // which is held alongside the narrowed copy while it is made).
-size_t solver_footprint(int32_t n, int32_t k, int in_elem, int elem);
+// `guided`: with the mirror that the guided rounds use.
+size_t solver_footprint(int32_t n, int32_t k, int in_elem, int elem, bool guided);
+// lbdd_create without that mirror.
+int create_unguided(lbdd_solver** out, int32_t n, int32_t k, const void* cm, int cm_dtype,
+                    int cm_is_device, const int32_t* cap, const int32_t* pen, void* cuda_stream);
 // A new solver on the same device holding a copy of src's instance (costs,
 // capacities, penalties), in the initial state.
 int clone_solver(const lbdd_solver* src, lbdd_solver** out);

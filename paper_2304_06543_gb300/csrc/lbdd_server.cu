@@ -69,6 +69,7 @@ struct Request {
   std::vector<int32_t> cap, pen;
   int32_t* assign_out = nullptr;
   size_t footprint = 0;
+  bool guided = true;     // false: the budget has no room for the mirror
   lbdd_solver* solver = nullptr;
   int64_t rounds = 0;
   int stalled = 0;        // passes in a row without progress
@@ -117,8 +118,8 @@ struct lbdd_server {
 
 // Device bytes a request may hold: int32 input is narrowed to int16 when
 // every cost fits, and both copies exist while the narrow one is made.
-static size_t request_footprint(int32_t n, int32_t k, int dtype) {
-  return solver_footprint(n, k, dtype == LBDD_CM_I16 ? 2 : 4, 2);
+static size_t request_footprint(int32_t n, int32_t k, int dtype, bool guided) {
+  return solver_footprint(n, k, dtype == LBDD_CM_I16 ? 2 : 4, 2, guided);
 }
 
 static void finish(lbdd_server* S, Request* r, int state, int status) {
@@ -195,8 +196,9 @@ static void admit_loop(lbdd_server* S) {
     }
     lk.unlock();
     lbdd_solver* s = nullptr;
-    const int rc = lbdd_create(&s, r->n, r->k, r->cm, r->dtype, r->cm_is_device, r->cap.data(),
-                               r->pen.data(), S->admit_st);
+    const auto create = r->guided ? lbdd_create : create_unguided;
+    const int rc = create(&s, r->n, r->k, r->cm, r->dtype, r->cm_is_device, r->cap.data(),
+                          r->pen.data(), S->admit_st);
     lk.lock();
     if (rc) {
       S->bytes -= r->footprint;
@@ -335,7 +337,13 @@ extern "C" int lbdd_server_submit_ex(lbdd_server* S, int32_t n, int32_t k, const
   r->cap.assign(cap, cap + k);
   r->pen.assign(pen, pen + k);
   r->assign_out = assign_out;
-  r->footprint = request_footprint(n, k, cm_dtype);
+  // a request that fits the budget only without the guided rounds' mirror is
+  // served without it
+  r->footprint = request_footprint(n, k, cm_dtype, true);
+  if (r->footprint > S->cfg.budget_bytes) {
+    r->guided = false;
+    r->footprint = request_footprint(n, k, cm_dtype, false);
+  }
   std::lock_guard<std::mutex> lk(S->mu);
   if (S->stop) { delete r; return LBDD_ERR_STATE; }
   r->id = S->next_id++;
