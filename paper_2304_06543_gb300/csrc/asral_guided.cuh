@@ -68,7 +68,9 @@ namespace lbdd {
 // Bits of a node in a packed (hop, node) key (k <= 8191).
 constexpr int kGNodeBits = 13;
 constexpr int kGOrd = 64;                       // prefetched (unit, center) pairs
-constexpr int kGWideLists = 800;                // centers up to which lists are that long
+// Centers up to which the lists of affected entries are as long as
+// guided_list says; beyond, one row's, so that the layout still fits.
+constexpr int kGWideLists = 800;
 // Affected entries that an apply lists at a time.  Where the cost table does
 // not fit shared memory anyway there is room for those of eight rows, so that
 // most paths go through each phase at once.
@@ -503,8 +505,9 @@ struct Guided {
   // The canonical shortest path that ends at node `last` (the cycle through
   // j if last < 0), backwards into s_pathu: the parent of a node v with label
   // l and hop count h is the lowest-index u with l(u) + T[u][v] = l and
-  // hop(u) = h - 1.  One warp up to kFollowWarp centers (no barrier), else
-  // thread = node and a barrier per hop.  Returns its length, -1 if there is
+  // hop(u) = h - 1.  One warp up to kFollowWarp centers (two strided passes and
+  // no barrier), else thread = node and a barrier per hop (one warp up to 192
+  // centers measured slower at 126).  Returns its length, -1 if there is
   // none (the one-warp form: to warp 0 only).
   static constexpr int kFollowWarp = 64;
   __device__ __forceinline__ bool precedes(int u, int32_t v, int h, LT l, int32_t j,
