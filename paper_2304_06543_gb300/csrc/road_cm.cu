@@ -92,16 +92,6 @@ static size_t road_smem_bytes(int32_t V) {
   return 12 * (size_t)kRoadQueue + (V <= kRoadSmemNodes ? 12 * road_bitmap_words(V) : 0);
 }
 
-// A step is a chain of memory latencies (node, its label and row, edges,
-// neighbour labels), so there should be few steps and little in each: the
-// threshold keeps a node from being relaxed again for every detour that
-// reaches it first (65,536 nodes in a grid: 1.1 relaxations per node instead
-// of up to 12, in about as many steps).  The lists and the marks live in
-// shared memory, a thread has eight edges of a node in flight together, and a
-// label is lowered by a reduction that returns nothing (the label read before
-// decides whether the neighbour is listed; one that was lowered further in
-// between is listed all the same).  65,536 nodes, 109 centers: 6.6 ms per
-// call with one list and marks in global memory, 1.8 ms now.
 // Sets `bit` of a bitmap word where `on`; returns the word as it was (all ones
 // where not).  Predicated instead of branched around, so that the atomics of
 // a node's edges are in flight together.
@@ -125,6 +115,18 @@ __device__ __forceinline__ void lower_if(bool on, int32_t* label, int32_t v) {
                ::"l"(label), "r"(v), "r"((uint32_t)on) : "memory");
 }
 
+// A step is a chain of memory latencies (node, its label and row, edges,
+// neighbour labels), so there should be few steps and little in each: the
+// threshold keeps a node from being relaxed again for every detour that
+// reaches it first (65,536 nodes in a grid: 1.1 relaxations per node instead
+// of up to 12, in about as many steps).  The lists and the marks live in
+// shared memory, a thread has eight edges of a node in flight together, and a
+// label is lowered by a reduction that returns nothing (the label read before
+// decides whether the neighbour is listed; one that was lowered further in
+// between is listed all the same).  65,536 nodes, 109 centers: 6.6 ms per
+// call with one list and marks in global memory, 1.74 ms now.  (Marks spread over
+// banks, and one atomic per warp instead of one per node for a list's length,
+// measured no faster: what a step issues counts for more than its conflicts.)
 template <bool SMEM>
 __global__ void __launch_bounds__(kRoadThreads)
 road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
