@@ -220,7 +220,10 @@ road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restr
       for (int i = tid; i < na; i += kRoadThreads) {
         const int32_t u = item(ln, i);
         const int4* row = reinterpret_cast<const int4*>(adj + (int64_t)u * kRoadDeg);
-        int32_t v[U], nd[U], dv[U];
+        // sums and labels as unsigned words: a label is a simple path's length
+        // (below 2^31, checked by the host), one road more may reach 2^32 - 1
+        int32_t v[U];
+        uint32_t nd[U], dv[U];
 #pragma unroll
         for (int q = 0; q < U; q += 2) {
           const int4 x = __ldg(row + q / 2);
@@ -233,19 +236,19 @@ road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restr
         bin[u >> 5] = 0;   // every set bit of this map is in the list being read
         int32_t rest = 0, end = 0;
         if (v[U - 1] == -2) {
-          rest = nd[U - 1];
+          rest = (int32_t)nd[U - 1];
           end = __ldg(row_ptr + u + 1);
         }
         for (;;) {
 #pragma unroll
-          for (int q = 0; q < U; ++q) dv[q] = v[q] >= 0 ? __ldcg(d + v[q]) : INT32_MIN;
+          for (int q = 0; q < U; ++q) dv[q] = v[q] >= 0 ? (uint32_t)__ldcg(d + v[q]) : 0u;
           uint32_t old[U];
 #pragma unroll
           for (int q = 0; q < U; ++q) {
-            nd[q] += du;
+            nd[q] += (uint32_t)du;
             const bool on = nd[q] < dv[q];
             const int32_t x = on ? v[q] : 0;
-            lower_if(on, d + x, nd[q]);
+            lower_if(on, d + x, (int32_t)nd[q]);
             old[q] = mark_if<SMEM>(on, (nd[q] < T ? bout : far_bits) + (x >> 5), 1u << (x & 31));
           }
           unsigned near = 0, far = 0;
@@ -268,7 +271,7 @@ road_sssp(int32_t V, const int32_t* __restrict__ row_ptr, const int32_t* __restr
           for (int q = 0; q < U; ++q) {
             const bool on = rest + q < end;
             v[q] = on ? __ldg(col + rest + q) : -1;
-            nd[q] = on ? __ldg(w + rest + q) : 0;
+            nd[q] = on ? (uint32_t)__ldg(w + rest + q) : 0u;
           }
           rest += U;
         }

@@ -66,3 +66,26 @@ def test_road_graph_matches_dijkstra(gpu_lib, name):
     rc, ref = oracle.road_cm(g.row_ptr, g.col, g.w, g.centers, g.demand)
     assert rc == 0
     assert np.array_equal(gpu_cm(gpu_lib, g), ref)
+
+
+def test_longest_accepted_lengths(gpu_lib):
+    """Roads back from a node whose distance is close to 2^31: the sum one road
+    further passes 2^31 and must not lower a label."""
+    t = lambda *a: np.array(a, np.int32)
+    x = 700_000_000
+    ring = SimpleNamespace(V=4, row_ptr=t(0, 1, 2, 3, 4), col=t(1, 2, 3, 0), w=t(x, x, x, x),
+                           centers=t(0), demand=t(1, 2, 3))
+    y = 1_000_000_000
+    line = SimpleNamespace(V=3, row_ptr=t(0, 1, 3, 4), col=t(1, 0, 2, 1), w=t(y, y, y, y),
+                           centers=t(0, 2), demand=t(1))
+    z = 2**31 - 2
+    pair = SimpleNamespace(V=2, row_ptr=t(0, 1, 2), col=t(1, 0), w=t(z, z), centers=t(0),
+                           demand=t(1))
+    # a node of 9 roads: the last ones are read from its CSR row
+    m = 200_000_000
+    hub = both(np.zeros(9, int), 1 + np.arange(9), np.full(9, m))
+    star = csr(10, *hub, 1, 2)
+    for g in (ring, line, pair, star):
+        rc, ref = oracle.road_cm(g.row_ptr, g.col, g.w, g.centers, g.demand)
+        assert rc == 0
+        assert np.array_equal(gpu_cm(gpu_lib, g), ref)
