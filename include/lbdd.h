@@ -219,14 +219,17 @@ void lbdd_batch_destroy(lbdd_batch* b);
 int lbdd_solve_batch(lbdd_solver* const* solvers, int m, int64_t max_rounds,
                      int cluster_size, int max_clusters, void* stream);
 
-/* Autotuner of the batch plan: for every (cost width, k bucket
+/* Autotuner of the batch plan: for every (kind of rounds, cost width, k bucket
  * 2^(b-1) < k <= 2^b) present among the m solvers, takes the instance with
  * the most units, builds a scaled-down copy (its first probe_rounds units,
- * capacities scaled by the same ratio) and times a complete solve of it on
- * one cluster of each size that fits; the ns per round are kept per device for
- * the process's lifetime and used by every later batch plan and server pass.
- * The solvers themselves are not modified.  lbdd_tune_get reads one entry
- * (0 = not measured); lbdd_tune_clear forgets all. */
+ * capacities scaled by the same ratio, the same options) and times a complete
+ * solve of it on one cluster of each size that fits; the ns per round are kept
+ * per device for the process's lifetime and used by every later batch plan and
+ * server pass of solvers of that kind.  The two kinds are the price-guided
+ * rounds and the full Bellman-Fords (a shortcut switched off, a penalty of 2^30
+ * or more, more centers than the guided form holds).  The solvers themselves
+ * are not modified.  lbdd_tune_get reads one entry, of the guided rounds where
+ * both kinds were measured (0 = not measured); lbdd_tune_clear forgets all. */
 int lbdd_autotune(lbdd_solver* const* solvers, int m, int probe_rounds, void* stream);
 int lbdd_tune_get(int cm_dtype, int32_t k, int cluster_size, double* ns_per_round);
 int lbdd_tune_clear(void);

@@ -436,8 +436,13 @@ int lbdd::clone_prefix(const lbdd_solver* src, int32_t n_sub, lbdd_solver** out)
     cap[c] = std::max<int32_t>(1, (int32_t)((int64_t)cap[c] * n_sub / src->n));
   }
   int rc = create_impl(out, n_sub, src->k, src->cm, src->elem == 2 ? LBDD_CM_I16 : LBDD_CM_I32,
-                       1, src->ld, cap.data(), pen.data(), src->st);
+                       1, src->ld, cap.data(), pen.data(), src->st, src->mirror != nullptr);
   if (rc == LBDD_OK && Q > 1) rc = lbdd_set_penalty_table(*out, q.data(), Q);
+  if (rc == LBDD_OK) {   // the same kind of rounds as src
+    (*out)->ncyc_skip = src->ncyc_skip;
+    (*out)->npath_reuse = src->npath_reuse;
+    (*out)->tc_smem = src->tc_smem;
+  }
   return rc;
 }
 

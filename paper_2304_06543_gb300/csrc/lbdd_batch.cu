@@ -11,7 +11,7 @@
 //    Larger C shortens a round (lower latency) but costs C SMs; for a batch
 //    the SM-time per round, t(k, C) * C, decides throughput.  The autotuner
 //    (lbdd_autotune) measures t(k, C) on a clone of one instance per
-//    (cost width, k bucket) and keeps the table per device.  The plan starts
+//    (kind of rounds, cost width, k bucket) and keeps the table per device.  The plan starts
 //    every instance at its throughput-best C and moves the instances that
 //    would outlast the rest of the batch to faster (larger) clusters.
 //  * Groups.  Instances with the same cost width and C form a group: one
@@ -66,8 +66,11 @@ __global__ void batch_gather(const DevInst* __restrict__ insts, int m, int64_t* 
 constexpr int kMaxDevices = 64;
 constexpr int kBuckets = 17;            // bucket b: 2^(b-1) < k <= 2^b
 constexpr int kNC = 5;                  // cluster sizes 1, 2, 4, 8, 16
+// [guided]: the guided rounds take about the same time on every C, the full
+// Bellman-Fords gain from larger clusters, so the times of one kind say
+// nothing about the other.
 struct TuneTable {
-  double ns[2][kBuckets][kNC];          // ns per round; 0 = not measured
+  double ns[2][2][kBuckets][kNC];       // [guided][width]: ns per round; 0 = not measured
 };
 static std::mutex g_tune_mu;
 static TuneTable g_tune[kMaxDevices];
@@ -129,9 +132,10 @@ static int choose_sizes(lbdd_solver* const* v, int m, int forced_C, int dev,
       (*est)[i] = Est{forced_C, (double)s->k / forced_C + 1.0};
       continue;
     }
-    const double* row = tab.ns[wid(s->elem)][bucket_of(s->k)];
-    for (int C = 1; C <= 16; C <<= 1)
-      if (row[cidx(C)] > 0 && solver_fits(s, C)) (*cands)[i].push_back({C, row[cidx(C)]});
+    for (int C = 1; C <= 16; C <<= 1) {
+      const double t = tab.ns[solver_guided(s, C)][wid(s->elem)][bucket_of(s->k)][cidx(C)];
+      if (t > 0 && solver_fits(s, C)) (*cands)[i].push_back({C, t});
+    }
     if ((*cands)[i].empty()) {
       const int C = default_cluster(s);
       if (!solver_fits(s, C)) return LBDD_ERR_ARG;
@@ -550,14 +554,16 @@ extern "C" int lbdd_autotune(lbdd_solver* const* solvers, int m, int probe_round
   int rc = check_device(&dev, &sms);
   if (rc) return rc;
   if (dev >= kMaxDevices) return LBDD_ERR_NODEV;
-  // one representative per (cost width, k bucket): the instance with most units
-  std::vector<int> rep(2 * kBuckets, -1);
+  // one representative per (kind of rounds, cost width, k bucket): the instance
+  // with most units
+  std::vector<int> rep(4 * kBuckets, -1);
   for (int i = 0; i < m; ++i) {
     if (!solvers[i]) return LBDD_ERR_ARG;
-    const int key = wid(solvers[i]->elem) * kBuckets + bucket_of(solvers[i]->k);
+    const int key = (2 * solver_guided(solvers[i], 1) + wid(solvers[i]->elem)) * kBuckets +
+                    bucket_of(solvers[i]->k);
     if (rep[key] < 0 || solvers[i]->n > solvers[rep[key]]->n) rep[key] = i;
   }
-  for (int key = 0; key < 2 * kBuckets; ++key) {
+  for (int key = 0; key < 4 * kBuckets; ++key) {
     if (rep[key] < 0) continue;
     // a whole solve of a scaled-down copy (first probe_rounds units,
     // capacities scaled alike) passes through the filling and the overload
@@ -565,7 +571,7 @@ extern "C" int lbdd_autotune(lbdd_solver* const* solvers, int m, int probe_round
     lbdd_solver* tmp = nullptr;
     rc = clone_prefix(solvers[rep[key]], probe_rounds, &tmp);
     if (rc) return rc;
-    double row[kNC] = {0, 0, 0, 0, 0};
+    double row[2][kNC] = {};
     const int64_t rounds = tmp->n;
     for (int C = 1; C <= 16 && rc == LBDD_OK; C <<= 1) {
       if (!solver_fits(tmp, C)) continue;
@@ -573,12 +579,15 @@ extern "C" int lbdd_autotune(lbdd_solver* const* solvers, int m, int probe_round
       rc = lbdd_reset(tmp);
       if (!rc) rc = solve_timed(tmp, 0, C, &ms);          // prologue only
       if (!rc) rc = solve_timed(tmp, rounds, C, &ms);
-      if (!rc) row[cidx(C)] = ms * 1e6 / (double)rounds;
+      if (!rc) row[solver_guided(tmp, C)][cidx(C)] = ms * 1e6 / (double)rounds;
     }
     lbdd_destroy(tmp);
     if (rc) return rc;
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    std::memcpy(g_tune[dev].ns[key / kBuckets][key % kBuckets], row, sizeof(row));
+    for (int kind = 0; kind < 2; ++kind)
+      if (*std::max_element(row[kind], row[kind] + kNC) > 0)
+        std::memcpy(g_tune[dev].ns[kind][key / kBuckets % 2][key % kBuckets], row[kind],
+                    sizeof(row[kind]));
   }
   return LBDD_OK;
 }
@@ -595,7 +604,9 @@ extern "C" int lbdd_tune_get(int cm_dtype, int32_t k, int cluster_size, double* 
   }
   if (dev >= kMaxDevices) return LBDD_ERR_NODEV;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  *ns_per_round = g_tune[dev].ns[cm_dtype == LBDD_CM_I16 ? 0 : 1][bucket_of(k)][cidx(cluster_size)];
+  const int w = cm_dtype == LBDD_CM_I16 ? 0 : 1, b = bucket_of(k), c = cidx(cluster_size);
+  const double guided = g_tune[dev].ns[1][w][b][c];
+  *ns_per_round = guided > 0 ? guided : g_tune[dev].ns[0][w][b][c];
   return LBDD_OK;
 }
 
