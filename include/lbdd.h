@@ -191,9 +191,10 @@ int lbdd_reset(lbdd_solver* s);
  *     round, least first; instances that would outlast the rest of the
  *     batch move to faster clusters); without measurements about k/128
  *     CTAs; cluster_size > 0 forces one size for all;
- *   - instances with the same cost width, C and solver options (strict,
- *     lbdd_option flags) form a group, at most 16 groups per batch (more:
- *     LBDD_ERR_ARG): one persistent launch whose clusters take instances
+ *   - instances with the same cost width, C, solver options (strict,
+ *     lbdd_option flags) and kind of rounds (guided or not; dropped where it
+ *     would make more than 16 groups: a mixed group then runs unguided) form a
+ *     group, at most 16 groups per batch (more: LBDD_ERR_ARG): one persistent launch whose clusters take instances
  *     from a device-side queue, the longest estimated solve first; the SMs
  *     are shared between the groups
  *     in proportion to their estimated SM-time (max_clusters > 0 caps each

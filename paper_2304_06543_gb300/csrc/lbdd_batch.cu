@@ -97,6 +97,8 @@ static int default_cluster(const lbdd_solver* s) {
 
 // ------------------------------------------------------------------ plan ---
 
+constexpr int kMaxGroups = 16;          // launches of a pass, at most
+
 struct Group {
   int elem = 4, C = 1, ncl = 1;
   size_t smem = 0;
@@ -154,16 +156,19 @@ static int choose_sizes(lbdd_solver* const* v, int m, int forced_C, int dev,
 // Order of instances inside a group's work queue.
 enum Order { LONGEST_FIRST = 0, SHORTEST_FIRST = 1 };
 
-// Groups of instances with equal (cost width, cluster size, options).
+// Groups of instances with equal (cost width, cluster size, options, kind of
+// rounds).  merge_kinds: instances that differ in the kind alone share a group,
+// whose rounds are then guided only if all of them can be.
 static int build_groups(lbdd_solver* const* v, const int64_t* rem, int m,
                         const std::vector<Est>& est, Order order, const uint8_t* first,
-                        std::vector<Group>* groups) {
+                        bool merge_kinds, std::vector<Group>* groups) {
   groups->clear();
+  const int same = merge_kinds ? ~OPT_GUIDED : ~0;
   for (int i = 0; i < m; ++i) {
     Group* g = nullptr;
     const int fl = launch_flags(v[i], est[i].C);
     for (auto& x : *groups)
-      if (x.elem == v[i]->elem && x.C == est[i].C && x.flags == fl) g = &x;
+      if (x.elem == v[i]->elem && x.C == est[i].C && ((x.flags ^ fl) & same) == 0) g = &x;
     if (!g) {
       groups->push_back(Group{});
       g = &groups->back();
@@ -171,6 +176,7 @@ static int build_groups(lbdd_solver* const* v, const int64_t* rem, int m,
       g->C = est[i].C;
       g->flags = fl;
     }
+    g->flags &= fl | same;
     g->idx.push_back(i);
     const double len = (double)rem[i] * est[i].t;
     g->work += len * est[i].C;
@@ -188,7 +194,11 @@ static int build_groups(lbdd_solver* const* v, const int64_t* rem, int m,
       return order == LONGEST_FIRST ? la > lb : la < lb;
     });
     g.smem = 0;
-    for (int i : g.idx) g.smem = std::max(g.smem, launch_smem_of(v[i], g.C));
+    for (int i : g.idx) {
+      const bool full = (g.flags & OPT_GUIDED) == 0;
+      if (full && !fits_k(v[i]->k, g.elem, g.C)) return LBDD_ERR_ARG;
+      g.smem = std::max(g.smem, full ? launch_smem(v[i]->k, g.C, g.elem) : launch_smem_of(v[i], g.C));
+    }
     if (g.smem > kMaxSmem) return LBDD_ERR_ARG;
   }
   return LBDD_OK;
@@ -274,7 +284,11 @@ static int make_plan(lbdd_solver* const* v, const int64_t* rem, int m, int force
     if (next.C == 0) { cands[top].clear(); continue; }
     est[top] = next;
   }
-  rc = build_groups(v, rem, m, est, order, first, groups);
+  // one launch per group; when there are more groups than the batch launches,
+  // the kind of rounds makes no group of its own
+  rc = build_groups(v, rem, m, est, order, first, false, groups);
+  if (!rc && groups->size() > (size_t)kMaxGroups)
+    rc = build_groups(v, rem, m, est, order, first, true, groups);
   if (!rc) rc = allocate_proportional(groups, max_clusters, sms);
   if (rc) return rc;
   cluster_of->assign(m, 0);
@@ -285,8 +299,6 @@ static int make_plan(lbdd_solver* const* v, const int64_t* rem, int m, int force
 }  // namespace lbdd
 
 // ----------------------------------------------------------- the batch ---
-
-constexpr int kMaxGroups = 16;          // one per (cost width, cluster size, solver options)
 
 struct lbdd_batch {
   int capacity = 0;                 // instances the buffers hold

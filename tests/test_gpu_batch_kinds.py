@@ -42,3 +42,26 @@ def test_tuning_of_one_kind_leaves_plans_of_the_other(gpu_lib, full):
             assert plan(gpu_lib, g) == plan_g
     finally:
         gpu_lib.tune_clear()
+
+
+def test_sixteen_option_sets_with_both_kinds(gpu_lib):
+    """Sixteen combinations of options form sixteen groups, the most a batch
+    takes; a penalty past the guided limit in four of them adds none."""
+    combos = [(a, b, c, d) for a in (0, 1) for b in (0, 1) for c in (0, 1) for d in (0, 1)]
+    solvers, refs = [], []
+    try:
+        for i, (ncyc, npath, tc, timers) in enumerate(combos + [x for x in combos if x[0] and x[1]]):
+            inst = L.random_small(9950 + i, n=90, k=7, cm_max=30, cap_frac=0.6, pen=(3, 40))
+            pen = inst.pen.copy()
+            if i >= len(combos):
+                pen[0] = 1 << 30
+            refs.append(oracle.asral(inst.cm, inst.cap, pen))
+            solvers.append(gpu_lib.Solver(inst.cm, inst.cap, pen, ncyc_skip=bool(ncyc),
+                                          npath_reuse=bool(npath), tc_smem=bool(tc),
+                                          phase_timers=bool(timers)))
+        gpu_lib.solve_batch([s.h for s in solvers], cluster_size=1)
+        for s, ref in zip(solvers, refs):
+            assert s.objective == ref.delta and np.array_equal(s.assignment(), ref.assign)
+    finally:
+        for s in solvers:
+            s.close()
