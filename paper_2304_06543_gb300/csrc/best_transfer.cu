@@ -101,10 +101,13 @@ static BtWorkspace carve(void* base, int32_t n, int32_t k) {
 
 static size_t table_part_bytes(int32_t n, int32_t k);
 
+// The least a call accepts, and what it makes full use of: the packed tables of
+// short rows take the place of everything else, as many as there is room for.
+size_t bt_workspace_min(int32_t n, int32_t k) {
+  return n < 1 || k < 1 ? 0 : carve(nullptr, n, k).bytes + 256;
+}
 size_t bt_workspace_bytes(int32_t n, int32_t k) {
-  if (n < 1 || k < 1) return 0;
-  // the packed tables of short rows take the place of everything else
-  return std::max(carve(nullptr, n, k).bytes, table_part_bytes(n, k)) + 256;
+  return n < 1 || k < 1 ? 0 : std::max(bt_workspace_min(n, k), table_part_bytes(n, k) + 256);
 }
 
 // ------------------------------------------------------------- grouping ---
@@ -1010,19 +1013,25 @@ struct TableShape {
   size_t smem;
 };
 
-// `clusters`: clusters of kTableCluster CTAs that run at a time.
-static TableShape table_shape(int32_t n, int32_t k, int elem, int clusters) {
+// `clusters`: clusters of kTableCluster CTAs that run at a time; `tables`:
+// packed tables that the workspace holds.  With room for few of them, larger
+// clusters and more slices keep the SMs busy.
+static TableShape table_shape(int32_t n, int32_t k, int elem, int clusters, int tables) {
   TableShape p;
   const int vpl = 16 / elem;
   const int G = (k + vpl - 1) / vpl;
   const int64_t vecs = (int64_t)n * G;
   const bool one = vecs * 16 <= kTableOneCluster;
-  p.C = kTableCluster;
   if (one)
     for (p.C = 1; p.C < 16 && vecs > (int64_t)p.C * 2 * kTableThreads;) p.C <<= 1;
   for (p.nslice = 1;; ++p.nslice) {
     p.gs = (G + p.nslice - 1) / p.nslice;
-    p.ncl = one ? 1 : std::max(1, std::min(kTableMaxClusters, clusters / p.nslice));
+    p.ncl = one ? 1 : std::max(1, std::min({kTableMaxClusters, tables, clusters / p.nslice}));
+    if (!one)
+      for (p.C = kTableCluster; p.C < 16 && 2 * p.C * p.ncl * p.nslice <= kTableCluster * clusters;)
+        p.C <<= 1;
+    if (!one && p.gs > kTableMinSlice && 2 * p.C * p.ncl * p.nslice <= kTableCluster * clusters)
+      continue;
     // few rows per center and range: nearly every key would be a new minimum
     // and the tables would outweigh the costs; narrower slices of more rows
     if (!one && p.gs > kTableMinSlice && p.ncl > 1 &&
@@ -1365,16 +1374,18 @@ static cudaError_t table_run(const T* cm, int64_t ld, int32_t n, int32_t k, cons
 
 template <typename T>
 static cudaError_t table_call(const T* cm, int64_t ld, int32_t n, int32_t k, const int32_t* assign,
-                              int32_t* tc, int32_t* td, void* ws, cudaStream_t st) {
+                              int32_t* tc, int32_t* td, void* ws, size_t ws_bytes,
+                              cudaStream_t st) {
   int clusters = 0;
+  const int tables = (int)std::min<size_t>(kTableMaxClusters, ws_bytes / (8ull * k * k));
   cudaError_t e;
   if constexpr (sizeof(T) == 2) {
     if ((e = table_setup<T, false>(&clusters)) != cudaSuccess) return e;
-    const TableShape p = table_shape(n, k, 2, clusters);
+    const TableShape p = table_shape(n, k, 2, clusters, tables);
     if (!p.wide) return table_run<T, false>(cm, ld, n, k, assign, tc, td, ws, p, st);
   }
   if ((e = table_setup<T, true>(&clusters)) != cudaSuccess) return e;
-  const TableShape p = table_shape(n, k, (int)sizeof(T), clusters);
+  const TableShape p = table_shape(n, k, (int)sizeof(T), clusters, tables);
   return table_run<T, true>(cm, ld, n, k, assign, tc, td, ws, p, st);
 }
 
@@ -1412,13 +1423,14 @@ static cudaError_t scan_launch(const T* cm, int64_t ld, int32_t k, const BtWorks
 // by the caller.
 cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_bytes, int64_t ld,
                               const int32_t* assign, int32_t* tc, int32_t* td, void* ws,
-                              cudaStream_t st, int num_sms) {
+                              size_t ws_bytes, cudaStream_t st, int num_sms) {
   void* base = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
   const BtWorkspace W = carve(base, n, k);
+  const size_t room = ws_bytes - (size_t)(static_cast<char*>(base) - static_cast<char*>(ws));
   if (k < kStreamMinK)
     return elem_bytes == 2
-               ? table_call(static_cast<const int16_t*>(cm), ld, n, k, assign, tc, td, base, st)
-               : table_call(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td, base, st);
+               ? table_call(static_cast<const int16_t*>(cm), ld, n, k, assign, tc, td, base, room, st)
+               : table_call(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td, base, room, st);
   const int nranges = stream_ranges(n, k, elem_bytes, num_sms);
   if (nranges > 0)
     return elem_bytes == 2

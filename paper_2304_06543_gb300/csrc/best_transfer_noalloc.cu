@@ -19,7 +19,7 @@ size_t bt_workspace_bytes(int32_t n, int32_t k);
 int bt_max_k(int elem_bytes);
 cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_bytes, int64_t ld,
                               const int32_t* assign, int32_t* tc, int32_t* td, void* ws,
-                              cudaStream_t st, int num_sms);
+                              size_t ws_bytes, cudaStream_t st, int num_sms);
 int cuda_fail(cudaError_t e, const char* what);
 }  // namespace lbdd
 
@@ -81,6 +81,7 @@ extern "C" int lbdd_best_transfer_noalloc(int32_t n, int32_t k, const void* cm_d
   // bounds via cudaMemsetAsync, the packed table filled with its identity),
   // so nothing left by an earlier call can leak into this one.
   const cudaError_t e = lbdd::best_transfer_run(n, k, cm_dev, elem, ld, assign_dev, tc_dev, td_dev,
-                                                scratch, static_cast<cudaStream_t>(stream), sms);
+                                                scratch, kStaticScratchBytes,
+                                                static_cast<cudaStream_t>(stream), sms);
   return e == cudaSuccess ? LBDD_OK : lbdd::cuda_fail(e, "lbdd_best_transfer_noalloc");
 }

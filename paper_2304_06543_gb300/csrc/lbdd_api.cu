@@ -878,11 +878,11 @@ extern "C" int lbdd_best_transfer(int32_t n, int32_t k, const void* cm_dev, int 
   if (ld < k || (ld * elem) % 16 != 0 || (reinterpret_cast<uintptr_t>(cm_dev) & 15) != 0)
     return LBDD_ERR_ARG;
   if (k > bt_max_k(elem)) return LBDD_ERR_ARG;
-  if (workspace_bytes < bt_workspace_bytes(n, k)) return LBDD_ERR_ARG;
+  if (workspace_bytes < bt_workspace_min(n, k)) return LBDD_ERR_ARG;
   int dev = 0, sms = 0;
   int rc = check_device(&dev, &sms);
   if (rc) return rc;
-  CK(best_transfer_run(n, k, cm_dev, elem, ld, assign_dev, tc_dev, td_dev, workspace,
+  CK(best_transfer_run(n, k, cm_dev, elem, ld, assign_dev, tc_dev, td_dev, workspace, workspace_bytes,
                        static_cast<cudaStream_t>(stream), sms));
   return LBDD_OK;
 }

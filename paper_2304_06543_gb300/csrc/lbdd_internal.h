@@ -25,10 +25,11 @@ cudaError_t launch_solver(const DevInst* d_insts, int ninst, int* d_counter, int
                           cudaStream_t st, uint64_t quantum_ns = 0, bool set_attrs = true);
 // best_transfer.cu
 size_t bt_workspace_bytes(int32_t n, int32_t k);
+size_t bt_workspace_min(int32_t n, int32_t k);   // ws_bytes is at least this
 int bt_max_k(int elem_bytes);
 cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_bytes, int64_t ld,
                               const int32_t* assign, int32_t* tc, int32_t* td, void* ws,
-                              cudaStream_t st, int num_sms);
+                              size_t ws_bytes, cudaStream_t st, int num_sms);
 
 // Dynamic shared memory a solver CTA may request: the 227 KB a block may
 // opt into, less 1 KB for the kernel's static shared variables (400 bytes
