@@ -371,10 +371,11 @@ const char* lbdd_last_cuda_error(void);
  *   tc_dev, td_dev : device int32[k*k] outputs.
  *   workspace  : device scratch of lbdd_best_transfer_workspace(n, k) bytes,
  *                owned by the caller; contents on entry are ignored.  With
- *                fewer than 256 centers this counts 40 packed k x k tables
- *                (8k^2 bytes each); a size with room for fewer of them, down
- *                to 4n + n/4 + 8k^2 + 276k bytes and 2 KB, gives the same
- *                table by fewer, larger clusters.
+ *                fewer than 256 centers and more than 4 MB of int32 costs
+ *                this counts 40 packed k x k tables (8k^2 bytes each); a size
+ *                with room for fewer of them, down to 4n + n/4 + 8k^2 + 276k
+ *                bytes and 2 KB, gives the same table by fewer, larger
+ *                clusters.
  *   stream     : cudaStream_t or NULL.  Asynchronous: results are ready
  *                when the stream reaches this point.
  * Errors: LBDD_ERR_ARG (sizes, alignment, workspace too small),

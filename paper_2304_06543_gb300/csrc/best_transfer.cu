@@ -978,10 +978,30 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
 // cluster then reduce their tables through distributed shared memory, a share
 // of the entries each.
 //
-// Up to kTableOneCluster bytes of costs one cluster does it all and writes
-// tc/td itself: one launch, which is what such a call costs.  Above that,
-// clusters of kTableCluster CTAs fill the chip, write one packed table each
-// and bt_merge_tables (a dependent launch) takes the minimum over them.
+// Up to kTableOneClusterK centers and kTableOneCluster entries one cluster does
+// it all and writes tc/td itself: one launch, which is what such a call costs.
+// Otherwise clusters of kTableCluster CTAs fill the chip, write one packed
+// table each and bt_merge_tables (a dependent launch) takes the minimum over
+// them.  Room for few tables (small workspaces, or up to kTablesInWorkspace
+// bytes of int32 costs, where that is all the workspace holds) makes clusters of
+// up to 8 CTAs and more slices; room for one table needs no merge, so such a
+// call is one launch too.
+//
+// Where the one cluster ends, measured (us per call, one cluster against many):
+// 40 centers int16 512 KB of costs 12.4 / 13.3, 768 KB 13.1 / 12.9, 1 MB 14.4 /
+// 12.1, int32 1 MB 12.3 / 12.2, 2 MB 16.4 / 11.8.  The time of its reduction
+// grows with k^2: 512 KB of int16 costs of 64, 100, 126 and 200 centers 12.4 /
+// 13.2, 14.4 / 12.0, 14.4 / 11.3 and 22.5 / 10.4 (with one cluster up to 4 MB,
+// calls of 200 centers took longer than the seven launches: 32 KB 32.7 against
+// 28.7, 3.6 MB 34.0 against 32.3).
+//
+// The other limits, us per call (50,001 x 126, 200,000 x 126 and 30,000 x 200
+// int32 unless said): clusters of 2, 4, 8 CTAs 24.6, 24.6, 28.8; 110.5, 66.8,
+// 77.9; 26.7, 28.8, 37.2.  kTableReuse 4, 16, 64: 26.1, 24.6, 24.6; 70.6, 66.8,
+// 70.6; 24.7, 28.8, 28.8 (400,000 x 64 int16 32.8, 32.8, 41.0).  kTableMinSlice 2,
+// 4, 8, 16: 20,011 x 255 32.9, 24.6, 24.6, 24.7, int16 22.6, 22.6, 22.6, 26.7.
+// kWideThreads 512, 640, 768, 1,024: 24.7, 24.6, 24.6, 24.7; 74.0, 66.8, 63.5,
+// 63.6; 30.8, 28.8, 28.7, 30.7; 1,000,000 x 20 49.2, 45.2, 45.1, 47.7.
 //
 // Measured per call, before (seven launches: count, plan, place, sort, scan,
 // unpack and a memset) and after: 2,000 x 20 int32 29.3 -> 10.7 us, 50,001 x
@@ -1001,7 +1021,9 @@ constexpr int kTableUnroll = 4;             // vectors in flight per thread
 constexpr int kWideThreads = 640;           // two words: two batches of 4 in registers
 constexpr int kWideUnroll = 4;
 constexpr int kTableCluster = 4;
-constexpr int64_t kTableOneCluster = 4 << 20;
+constexpr int kTableOneClusterK = 64;       // centers and ...
+constexpr int64_t kTableOneCluster = 384 << 10;   // ... entries up to which one cluster runs
+constexpr int64_t kTablesInWorkspace = 4 << 20;   // bytes of int32 costs from which they count
 constexpr size_t kTableSmem = 200 * 1024;
 constexpr int kTableMaxClusters = 40;       // packed tables of a call, at most
 constexpr int kTableReuse = 16;             // rows per center and range to aim for ...
@@ -1021,15 +1043,14 @@ static TableShape table_shape(int32_t n, int32_t k, int elem, int clusters, int 
   const int vpl = 16 / elem;
   const int G = (k + vpl - 1) / vpl;
   const int64_t vecs = (int64_t)n * G;
-  const bool one = vecs * 16 <= kTableOneCluster;
+  const bool one = k <= kTableOneClusterK && vecs * vpl <= kTableOneCluster;
   if (one)
     for (p.C = 1; p.C < 16 && vecs > (int64_t)p.C * 2 * kTableThreads;) p.C <<= 1;
   for (p.nslice = 1;; ++p.nslice) {
     p.gs = (G + p.nslice - 1) / p.nslice;
     p.ncl = one ? 1 : std::max(1, std::min({kTableMaxClusters, tables, clusters / p.nslice}));
-    if (!one)
-      for (p.C = kTableCluster; p.C < 16 && 2 * p.C * p.ncl * p.nslice <= kTableCluster * clusters;)
-        p.C <<= 1;
+    if (!one)   // (clusters of 8 leave some SMs of a GPC unused)
+      for (p.C = kTableCluster; p.C < 8 && 2 * p.C * p.ncl * p.nslice <= 3 * clusters;) p.C <<= 1;
     if (!one && p.gs > kTableMinSlice && 2 * p.C * p.ncl * p.nslice <= kTableCluster * clusters)
       continue;
     // few rows per center and range: nearly every key would be a new minimum
@@ -1045,9 +1066,13 @@ static TableShape table_shape(int32_t n, int32_t k, int elem, int clusters, int 
   return p;
 }
 
-// Packed tables of the largest call of this size (any cost width).
+// Packed tables of the largest call of this size (any cost width); fewer costs
+// make do with those that the grouped scan's workspace has room for.
+static bool tables_in_workspace(int32_t n, int32_t k) {
+  return k < kStreamMinK && (int64_t)n * k * 4 + 16ll * n > kTablesInWorkspace;
+}
 static size_t table_part_bytes(int32_t n, int32_t k) {
-  if (k >= kStreamMinK || (int64_t)n * k * 4 + 16ll * n <= kTableOneCluster) return 0;
+  if (!tables_in_workspace(n, k)) return 0;
   return 8ull * k * k * kTableMaxClusters;
 }
 
@@ -1377,7 +1402,10 @@ static cudaError_t table_call(const T* cm, int64_t ld, int32_t n, int32_t k, con
                               int32_t* tc, int32_t* td, void* ws, size_t ws_bytes,
                               cudaStream_t st) {
   int clusters = 0;
-  const int tables = (int)std::min<size_t>(kTableMaxClusters, ws_bytes / (8ull * k * k));
+  // (the same route whatever a caller's workspace has beyond the size asked for)
+  const size_t room = tables_in_workspace(n, k)
+                          ? ws_bytes : std::min(ws_bytes, bt_workspace_min(n, k) - 256);
+  const int tables = (int)std::min<size_t>(kTableMaxClusters, room / (8ull * k * k));
   cudaError_t e;
   if constexpr (sizeof(T) == 2) {
     if ((e = table_setup<T, false>(&clusters)) != cudaSuccess) return e;

@@ -1,4 +1,6 @@
-"""A workspace of the size that the grouped scan needed is enough for every size."""
+"""Scans of fewer than 256 centers by the room for packed tables: a workspace
+of the size that the grouped scan needed is enough, and the sizes where one
+cluster ends."""
 import numpy as np
 import pytest
 
@@ -13,9 +15,24 @@ SIZES = [(50001, 126, 375296), (20011, 255, 676608), (9001, 126, 200960), (30000
          (9000, 200, 414208), (5000, 255, 612864)]
 
 
+# around 64 centers and 393,216 entries, and calls of one table and several
+EDGES = [(6144, 64), (6145, 64), (6049, 65), (90, 65), (16384, 24), (16385, 24), (49152, 8),
+         (49153, 8), (80, 200), (1300, 200), (2000, 100), (3, 255)]
+
+
+@pytest.mark.parametrize("dtype", ["i16", "i32"])
+@pytest.mark.parametrize("n,k", EDGES)
+def test_scan_where_one_cluster_ends(gpu_lib, dtype, n, k):
+    run(gpu_lib, dtype, n, k, gpu_lib.best_transfer_workspace(n, k))
+
+
 @pytest.mark.parametrize("dtype", ["i16", "i32"])
 @pytest.mark.parametrize("n,k,size", SIZES)
 def test_scan_with_the_smaller_workspace(gpu_lib, dtype, n, k, size):
+    run(gpu_lib, dtype, n, k, size)
+
+
+def run(gpu_lib, dtype, n, k, size):
     import torch
     inst = L.random_small(9300 + k, n=n, k=k, cm_max=90)
     assign = np.random.default_rng(k).integers(-1, k, n).astype(np.int32)
