@@ -117,9 +117,12 @@ struct lbdd_server {
 };
 
 // Device bytes a request may hold: int32 input is narrowed to int16 when
-// every cost fits, and both copies exist while the narrow one is made.
+// every cost fits, and both copies exist while the narrow one is made;
+// otherwise one copy stays, and the guided rounds' mirror holds int32 costs
+// too, which is more where n is less than k.
 static size_t request_footprint(int32_t n, int32_t k, int dtype, bool guided) {
-  return solver_footprint(n, k, dtype == LBDD_CM_I16 ? 2 : 4, 2, guided);
+  if (dtype == LBDD_CM_I16) return solver_footprint(n, k, 2, 2, guided);
+  return std::max(solver_footprint(n, k, 4, 2, guided), solver_footprint(n, k, 4, 4, guided));
 }
 
 static void finish(lbdd_server* S, Request* r, int state, int status) {
