@@ -30,17 +30,22 @@ int lbdd::cuda_fail(cudaError_t e, const char* what) {
 // Device memory of a solver comes from the stream-ordered pool on the
 // solver's stream: allocating and freeing never waits for kernels running on
 // other streams (a server admits and retires requests while others solve).
-static int dev_alloc(lbdd_solver* s, void** p, size_t bytes) {
+static cudaError_t try_alloc(lbdd_solver* s, void** p, size_t bytes) {
   bytes = std::max<size_t>(bytes, 16);
-  cudaError_t e = cudaMallocAsync(p, bytes, s->st);
+  const cudaError_t e = cudaMallocAsync(p, bytes, s->st);
   if (e != cudaSuccess) {
     *p = nullptr;
-    return cuda_fail(e, "cudaMallocAsync");
+    return e;
   }
   s->allocs.push_back(*p);
   s->sizes.push_back(bytes);
   s->bytes += bytes;
-  return LBDD_OK;
+  return e;
+}
+
+static int dev_alloc(lbdd_solver* s, void** p, size_t bytes) {
+  const cudaError_t e = try_alloc(s, p, bytes);
+  return e == cudaSuccess ? LBDD_OK : cuda_fail(e, "cudaMallocAsync");
 }
 
 template <typename P>
@@ -286,13 +291,14 @@ static int create_impl(lbdd_solver** out, int32_t n, int32_t k, const void* cm, 
   if (!rc) rc = dalloc(s, &s->tc, (size_t)k * k);
   if (!rc) rc = dalloc(s, &s->td, (size_t)k * k);
   if (!rc) rc = dalloc(s, &s->pot, k);
-  // the guided rounds' mirror is optional: without it (no memory left for it)
-  // the solver runs unguided
-  if (!rc && guided && guided_smem_bytes(k, s->elem, kMaxSmem) > 0)
-    (void)dev_alloc(s, &s->mirror, guided_mirror_bytes(k, s->elem));
   if (!rc) rc = dalloc(s, &s->ctl, CTL_COUNT);
   if (!rc) rc = dalloc(s, &s->counter, 4);
   if (!rc) rc = dalloc(s, &s->d_inst, 1);
+  // the guided rounds' mirror is optional, so it comes last and its failure is
+  // no error: without it (no memory left for it) the solver runs unguided
+  if (!rc && guided && guided_smem_bytes(k, s->elem, kMaxSmem) > 0 &&
+      try_alloc(s, &s->mirror, guided_mirror_bytes(k, s->elem)) != cudaSuccess)
+    (void)cudaGetLastError();
   if (rc) { free_all(s); delete s; return rc; }
   DevInst& I = s->h_inst;
   I.cm = s->cm; I.ld = s->ld; I.n = n; I.k = k; I.cap = s->cap; I.pen = s->pen; I.Q = 1;
