@@ -1597,7 +1597,8 @@ namespace lbdd {
 
 // The guided rounds.  CTA 0 of every cluster runs them; the others share the
 // prologue (a scan of every row of CM), which is all there is to share: a
-// round's frontier is a dozen labels.
+// round's frontier is a dozen labels.  A launch with OPT_PROLOGUE runs the
+// prologues that are due and worth its cluster, and no rounds.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 1)
 asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_counter, int flags,
@@ -1620,8 +1621,10 @@ asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_coun
           if (it >= ninst) break;
           const int64_t* c = insts[it].ctl;
           const int64_t target = min((int64_t)insts[it].n, __ldcg(c + CTL_TARGET));
+          const bool due = __ldcg(c + CTL_PROLOGUE) == 0;
           if (__ldcg(c + CTL_STATUS) == 0 &&
-              (__ldcg(c + CTL_PROLOGUE) == 0 || __ldcg(c + CTL_ROUNDS) < target))
+              (flags & OPT_PROLOGUE ? due && wide_prologue(insts[it].n, insts[it].k)
+                                    : due || __ldcg(c + CTL_ROUNDS) < target))
             break;
         }
       }
@@ -1669,7 +1672,7 @@ asral_guided_kernel(const DevInst* __restrict__ insts, int ninst, int* work_coun
       }
       __syncthreads();
     }
-    if (rank != 0) continue;   // waits at the next instance's barrier
+    if (rank != 0 || (flags & OPT_PROLOGUE)) continue;   // waits at the next instance's barrier
     const bool tsm = L.total <= avail && !(flags & OPT_NO_TC_SMEM);
     const bool usm = tsm && L.full <= avail;
     auto rounds = [&](auto G) { G.run_rounds(s_deadline); };

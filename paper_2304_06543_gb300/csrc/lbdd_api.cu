@@ -225,9 +225,19 @@ extern "C" int32_t lbdd_max_centers(void) {
 // rounds without the prologue: 49.6 ms on one CTA, 50.2 on 16); the other CTAs
 // only shorten the prologue (2.2 against 0.36 ms; whole solves: below 1 %) and
 // hold their SMs for as long as the solve runs, which other streams could use.
-// Past this many centers the prologue is a larger share of a short solve (and
-// at 1,500 one CTA no longer holds the full Bellman-Ford form to fall back on).
+// (At 1,500 centers one CTA no longer holds the full Bellman-Ford form to fall
+// back on.)
 constexpr int32_t kGuidedMaxK = 1024;
+
+// Rounds below n / kShortCall are a short call: it begins with the prologue on
+// a cluster of its own, which is given back before the rounds.  Longer calls
+// leave it to the CTA of the rounds (below 1 % of their time) and need no
+// cluster.  First call of five rounds (solver on up to 16 CTAs with the full
+// Bellman-Fords / all on one CTA / this way): 200,000 x 1,000 3.40 / 9.40 /
+// 2.23 ms, 200,000 x 500 2.41 / 6.14 / 1.79, 50,000 x 126 0.89 / 1.16 / 0.51.
+// Eight CTAs: 16 shorten the prologue by a fifth to a third more, but find
+// their SMs free in one GPC less often.
+constexpr int64_t kShortCall = 16;
 
 static int fits(const lbdd_solver* s, int C) { return fits_k(s->k, s->elem, C) ? 1 : 0; }
 
@@ -555,6 +565,17 @@ size_t lbdd::launch_smem_of(const lbdd_solver* s, int C) {
                              : launch_smem(s->k, C, s->elem);
 }
 
+bool lbdd::prologue_first(const lbdd_solver* s, int C, int64_t rounds, uint64_t quantum_ns) {
+  if (!s->fresh || C >= kPrologueCluster || !wide_prologue(s->n, s->k) || !solver_guided(s, C) ||
+      !solver_guided(s, kPrologueCluster))
+    return false;
+  if (rounds >= 0 && rounds < s->n / kShortCall) return true;
+  // one CTA's prologue, measured over 500 to 200,000 units and 20 to 1,000
+  // centers: 21 ns a unit, 50 GB/s of costs, k^2 / 5 ns for the tables
+  const double ns = 21.0 * s->n + (double)s->n * s->k * s->elem / 50 + 0.2 * s->k * s->k;
+  return quantum_ns > 0 && ns > quantum_ns / 4.0;
+}
+
 int lbdd::choose_cluster(lbdd_solver* s) {
   if (s->cluster == 0 && s->k <= kGuidedMaxK && solver_guided(s, 1)) return 1;
   int C = pick_cluster(s);
@@ -569,11 +590,15 @@ extern "C" int lbdd_solve(lbdd_solver* s, int64_t max_rounds) {
   const int C = choose_cluster(s);
   if (C < 1) return LBDD_ERR_ARG;
   const size_t smem = launch_smem_of(s, C);
-  CK(cudaMemsetAsync(s->counter, 0, sizeof(int32_t), s->st));
+  CK(cudaMemsetAsync(s->counter, 0, 2 * sizeof(int32_t), s->st));
+  if (s->cluster == 0 && prologue_first(s, C, max_rounds, 0))
+    CK(launch_solver(s->d_inst, 1, s->counter + 1, kPrologueCluster, 1, s->elem, smem,
+                     launch_flags(s, C) | OPT_PROLOGUE, s->st));
   CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, launch_flags(s, C), s->st));
   int64_t st = 0;
   CK(cudaMemcpyAsync(&st, s->ctl + CTL_STATUS, sizeof(int64_t), cudaMemcpyDeviceToHost, s->st));
   CK(cudaStreamSynchronize(s->st));
+  s->fresh = false;
   return status_to_rc(st);
 }
 
@@ -748,6 +773,7 @@ extern "C" int lbdd_insert(lbdd_solver* s, const void* row, int cm_dtype, int32_
 
 extern "C" int lbdd_reset(lbdd_solver* s) {
   if (!s) return LBDD_ERR_ARG;
+  s->fresh = true;
   CK(cudaMemsetAsync(s->ctl, 0, sizeof(int64_t) * CTL_COUNT, s->st));
   CK(cudaMemsetAsync(s->assign, 0xff, 4ull * s->n, s->st));
   CK(cudaMemsetAsync(s->load, 0, 4ull * s->k, s->st));

@@ -313,7 +313,7 @@ struct lbdd_batch {
   cudaEvent_t join[kMaxGroups - 1] = {};
   DevInst* d_insts = nullptr;
   DevInst* h_insts = nullptr;       // pinned staging of d_insts
-  int* d_counters = nullptr;
+  int* d_counters = nullptr;        // a work queue per group, then one per group's prologues
   int64_t* d_params = nullptr;
   int64_t* d_out = nullptr;
   int64_t* h_params = nullptr;      // pinned
@@ -321,6 +321,7 @@ struct lbdd_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   uint64_t quantum_ns = 0;
+  int launches = 0;                 // kernels of the last pass
   int dev = 0, sms = 0;
 };
 
@@ -389,7 +390,7 @@ int batch_alloc(lbdd_batch** out, int capacity, uint64_t quantum_ns, void* strea
   cudaError_t e;
   auto cf = [&](cudaError_t err, const char* w) { batch_free(b); return cuda_fail(err, w); };
   if ((e = cudaMalloc(&b->d_insts, sizeof(DevInst) * capacity))) return cf(e, "batch insts");
-  if ((e = cudaMalloc(&b->d_counters, sizeof(int) * kMaxGroups))) return cf(e, "batch counters");
+  if ((e = cudaMalloc(&b->d_counters, sizeof(int) * 2 * kMaxGroups))) return cf(e, "batch counters");
   if ((e = cudaMalloc(&b->d_params, sizeof(int64_t) * 2))) return cf(e, "batch params");
   if ((e = cudaMalloc(&b->d_out, sizeof(int64_t) * 2 * capacity))) return cf(e, "batch out");
   if ((e = cudaMallocHost(&b->h_insts, sizeof(DevInst) * capacity))) return cf(e, "batch insts (host)");
@@ -462,10 +463,35 @@ int batch_capture(lbdd_batch* b) {
   return LBDD_OK;
 }
 
+// A short pass, or one whose quantum a prologue would fill, begins with the
+// prologues that are due, on larger clusters (prologue_first), unless there
+// are so many that an SM each serves them as well.
+static int batch_prologues(lbdd_batch* b, int64_t max_rounds) {
+  for (size_t g = 0; g < b->groups.size(); ++g) {
+    const Group& G = b->groups[g];
+    if (!(G.flags & OPT_GUIDED)) continue;
+    int due = 0;
+    for (int i : G.idx)
+      due += prologue_first(b->solvers[i], G.C, max_rounds, b->quantum_ns) ? 1 : 0;
+    const int most = b->sms / kPrologueCluster;
+    if (due == 0 || due > most) continue;
+    int* queue = b->d_counters + kMaxGroups + g;
+    CK(cudaMemsetAsync(queue, 0, sizeof(int), b->st));
+    CK(launch_solver(b->d_insts + b->offset[g], (int)G.idx.size(), queue, kPrologueCluster,
+                     std::min(most, (int)G.idx.size()), G.elem, G.smem, G.flags | OPT_PROLOGUE,
+                     b->st));
+    b->launches++;
+  }
+  return LBDD_OK;
+}
+
 // Starts one pass (max_rounds more rounds for every instance) on b->st.
 int batch_launch(lbdd_batch* b, int64_t max_rounds) {
   b->h_params[0] = max_rounds;
   for (auto& g : b->groups) CK(prepare_solver(g.C, g.elem, g.smem, g.flags));
+  b->launches = 2 + (int)b->groups.size();
+  const int rc = batch_prologues(b, max_rounds);
+  if (rc) return rc;
   if (b->exec) {
     CK(cudaGraphLaunch(b->exec, b->st));
     return LBDD_OK;
@@ -478,6 +504,7 @@ int batch_wait(lbdd_batch* b, int* first_rc) {
   CK(cudaStreamSynchronize(b->st));
   int first = LBDD_OK;
   for (size_t i = 0; i < b->solvers.size(); ++i) {
+    if (b->h_out[2 * b->slot_of[i] + 1] > 0) b->solvers[i]->fresh = false;
     const int r = status_to_rc(b->h_out[2 * b->slot_of[i]]);
     if (r && first == LBDD_OK) first = r;
   }
@@ -492,7 +519,7 @@ void batch_detach(lbdd_batch* b) {
   b->solvers.clear();
 }
 
-int batch_launches(const lbdd_batch* b) { return 2 + (int)b->groups.size(); }
+int batch_launches(const lbdd_batch* b) { return b->launches; }
 int64_t batch_rounds(const lbdd_batch* b, int i) { return b->h_out[2 * b->slot_of[i] + 1]; }
 int64_t batch_status(const lbdd_batch* b, int i) { return b->h_out[2 * b->slot_of[i]]; }
 void batch_destroy(lbdd_batch* b) {

@@ -72,8 +72,15 @@ enum : int {
   OPT_NO_TC_SMEM = 4,     // keep the owned cost slice in global memory only
   OPT_PHASE_TIMERS = 8,   // time the phases of every round (CTA 0, thread 0)
   OPT_STRICT = 32,        // strict-LBDD (Alg. 5): vacancies as zero-cost dummy units
-  OPT_GUIDED = 64,        // one-CTA launch of the price-guided rounds (set by the host)
+  OPT_GUIDED = 64,        // the price-guided rounds: CTA 0 runs them (set by the host)
+  OPT_PROLOGUE = 128,     // guided launch that runs no rounds, only due prologues (host)
 };
+
+// Whether a prologue is worth a launch of its own on a larger cluster (about
+// 60 us on one CTA, 20 to 40 us more than on eight).
+__host__ __device__ inline bool wide_prologue(int64_t n, int64_t k) {
+  return 100 * n + k * k >= 300000;
+}
 
 // Device view of one instance.  Pointers are device memory owned by the
 // library (lbdd_solver).

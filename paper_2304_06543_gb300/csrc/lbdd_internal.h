@@ -62,6 +62,7 @@ struct lbdd_solver {
   int32_t n_cap = 0;       // units the unit-indexed arrays and the page pool hold (>= n)
   int32_t max_cost = 0;    // largest cost at creation
   int32_t max_pen = 0;     // largest penalty (guided rounds need it below guided_pen_limit())
+  bool fresh = true;       // no round has run: the next ones begin with the prologue
   int in_batches = 0;      // batches that hold a copy of this solver's device view
   int32_t* ins_row = nullptr;  // k costs of a unit being inserted (device staging)
   size_t bytes = 0;        // device bytes held now
@@ -86,6 +87,11 @@ int solver_flags(const lbdd_solver* s);
 bool solver_guided(const lbdd_solver* s, int C);
 // Whether s runs on C-CTA clusters, guided or not.
 bool solver_fits(const lbdd_solver* s, int C);
+// A prologue ahead of rounds on smaller clusters: its cluster size, and whether
+// s's next `rounds` (< 0: all) rounds on C CTAs, in a pass of quantum_ns (0:
+// unlimited), are preceded by it.
+constexpr int kPrologueCluster = 8;
+bool prologue_first(const lbdd_solver* s, int C, int64_t rounds, uint64_t quantum_ns);
 // Launch flags and dynamic shared memory of s's rounds on C-CTA clusters.
 int launch_flags(const lbdd_solver* s, int C);
 size_t launch_smem_of(const lbdd_solver* s, int C);
