@@ -186,6 +186,11 @@ def kernel_source_hash(files=None) -> str:
     return h.hexdigest()[:16]
 
 
+def solver_kernel(solver) -> str:
+    """The kernel that ran a solver's rounds."""
+    return "asral_guided_kernel" if solver.guided_rounds > 0 else "asral_cluster_kernel"
+
+
 def committed_traffic(kernel: str, workload: str = "city"):
     """DRAM bytes per launch from a committed ncu summary, if it was taken on
     the kernel's current sources (the files listed with it) and on this
@@ -390,16 +395,15 @@ def run_ours(args):
     alg_bytes = (rows_full * inst.k * w + dstat("col_rows") * (w + 4)) / steps
     achieved = alg_bytes / (ms_per_step / 1000.0) / 1e9
     # the committed figure is for whole solves of its own workload
-    traffic = (committed_traffic("asral_guided_kernel", args.workload)
-               if args.max_rounds < 0 else None)
-    roofline = {"kernel": "asral_guided_kernel", "bound": "hbm", "achieved": achieved,
+    kernel = solver_kernel(solver)
+    traffic = committed_traffic(kernel, args.workload) if args.max_rounds < 0 else None
+    roofline = {"kernel": kernel, "bound": "hbm", "achieved": achieved,
                 "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                 "peak_kind": peak_kind,
                 "traffic": traffic["dram_bytes_per_launch"] if traffic else None,
                 "algorithmic_bytes_per_launch": alg_bytes,
-                "note": "persistent kernel, one CTA runs the rounds; latency bound (pruned "
-                        "Bellman-Ford sweeps, dependent reads of an apply), see phase "
-                        "breakdown"}
+                "note": "persistent kernel, latency bound (Bellman-Ford sweeps, dependent reads "
+                        "of an apply), see phase breakdown; guided: one CTA runs the rounds"}
     # phase breakdown from one more solve with the phase timers on (they
     # slow the rounds, so they are off in the timed steps)
     lb.set_option(solver.h, lb.OPT_PHASE_TIMERS, 1)
@@ -1146,14 +1150,15 @@ def city_measure(lb, hbm_peak, peak_kind):
     ms = e0.elapsed_time(e1)
     st = solver.stats()
     obj = solver.objective
+    kernel = solver_kernel(solver)
     solver.close()
     with open(os.path.join(ROOT, "tests", "golden", "city_oracle.json")) as f:
         gold = json.load(f)
     w = st.cm_elem_bytes
     alg = (st.rows_scanned + 2 * inst.n) * inst.k * w + st.col_rows * (w + 4)
     achieved = alg / (ms / 1000.0) / 1e9
-    traffic = committed_traffic("asral_guided_kernel", "city")
-    roof = {"kernel": "asral_guided_kernel", "bound": "hbm", "achieved": achieved,
+    traffic = committed_traffic(kernel, "city")
+    roof = {"kernel": kernel, "bound": "hbm", "achieved": achieved,
             "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak, "peak_kind": peak_kind,
             "traffic": traffic["dram_bytes_per_launch"] if traffic else None,
             "algorithmic_bytes_per_launch": alg,

@@ -336,6 +336,13 @@ int lbdd_loads(const lbdd_solver* s, int32_t* out);
 
 int lbdd_rounds_done(const lbdd_solver* s, int64_t* out);
 
+/* How many of those rounds ran price-guided (asral_guided_kernel) instead of
+ * with full Bellman-Fords (asral_cluster_kernel).  Guided rounds need both
+ * LBDD_OPT_NCYC_SKIP and LBDD_OPT_NPATH_REUSE on, penalties below 2^30 (strict
+ * solvers: costs below 2^30), at most 2,680 centers with int16 and 1,954 with
+ * int32 costs, and device memory for one more copy of the best-transfer costs.  Either way the result is the same; only the time differs. */
+int lbdd_guided_rounds(const lbdd_solver* s, int64_t* out);
+
 /* Counters of the solve so far (host struct). */
 int lbdd_get_stats(const lbdd_solver* s, lbdd_stats* out);
 

@@ -94,6 +94,7 @@ def load():
         lib.lbdd_insert.argtypes = [P, P, c_int, ctypes.POINTER(i32)]
         lib.lbdd_solve_batch.argtypes = [ctypes.POINTER(P), c_int, i64, c_int, c_int, P]
         lib.lbdd_objective.argtypes = [P, ctypes.POINTER(i64)]
+        lib.lbdd_guided_rounds.argtypes = [P, ctypes.POINTER(i64)]
         lib.lbdd_assignment.argtypes = [P, P, c_int]
         lib.lbdd_loads.argtypes = [P, P]
         lib.lbdd_rounds_done.argtypes = [P, ctypes.POINTER(i64)]
@@ -323,6 +324,13 @@ def rounds_done(h) -> int:
     return v.value
 
 
+def guided_rounds(h) -> int:
+    """lbdd_guided_rounds: rounds that ran price-guided."""
+    v = ctypes.c_int64()
+    _check(load().lbdd_guided_rounds(h, ctypes.byref(v)), "lbdd_guided_rounds")
+    return v.value
+
+
 def assignment(h, n: int, out=None):
     """Host numpy copy (default) or into a CUDA int32 tensor `out`."""
     if out is None:
@@ -449,6 +457,10 @@ class Solver:
     @property
     def rounds(self) -> int:
         return rounds_done(self.h)
+
+    @property
+    def guided_rounds(self) -> int:
+        return guided_rounds(self.h)
 
     def assignment(self, out=None):
         return assignment(self.h, self.n, out)

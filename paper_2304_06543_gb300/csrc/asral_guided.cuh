@@ -1175,6 +1175,7 @@ struct Guided {
       I.ctl[CTL_POT] = prices_ok && status == ST_OK ? 1 : 0;
       if (count > 0) I.ctl[CTL_MIRROR] = TSM ? 0 : 1;
       I.ctl[CTL_ROUNDS] = r_begin + q;
+      I.ctl[CTL_GUIDED] += q;
       I.ctl[CTL_DELTA] = B->delta;
       I.ctl[CTL_FREE_TOP] = B->free_top;
       I.ctl[CTL_STATUS] = status != ST_OK ? status : B->err0;

@@ -798,6 +798,11 @@ extern "C" int lbdd_rounds_done(const lbdd_solver* s, int64_t* out) {
   return read_ctl(s, CTL_ROUNDS, out);
 }
 
+extern "C" int lbdd_guided_rounds(const lbdd_solver* s, int64_t* out) {
+  if (!s || !out) return LBDD_ERR_ARG;
+  return read_ctl(s, CTL_GUIDED, out);
+}
+
 extern "C" int lbdd_assignment(const lbdd_solver* s, int32_t* out, int out_is_device) {
   if (!s || !out) return LBDD_ERR_ARG;
   CK(cudaMemcpyAsync(out, s->assign, 4ull * s->n,

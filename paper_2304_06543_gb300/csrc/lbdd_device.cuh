@@ -55,6 +55,7 @@ enum CtlIndex {
   CTL_FRONT_HIST,      // 6 bins of frontier sizes: 1, 2-4, 5-16, 17-64, 65-256, >256
   CTL_POT = CTL_FRONT_HIST + 6,  // 1: the prices hold for the current table (guided rounds)
   CTL_MIRROR,          // 1: the global mirror of T's costs is current (guided rounds)
+  CTL_GUIDED,          // rounds that ran guided
   CTL_COUNT
 };
 

@@ -41,7 +41,7 @@ lib = lb.load()
 inst = L.random_small(9500, n=300, k=400, cm_max=50, cap_frac=0.5, pen=(5, 60))
 with lb.Solver(inst.cm.astype(np.int16), inst.cap, inst.pen) as s:
     s.solve()
-    print(json.dumps({"objective": s.objective, "assign": s.assignment().tolist(),
+    print(json.dumps({"objective": s.objective, "guided": s.guided_rounds, "assign": s.assignment().tolist(),
                       "error": lib.lbdd_last_cuda_error().decode()}))
 """
 
@@ -63,4 +63,4 @@ def test_mirror_without_memory(gpu_lib, tmp_path):
     ref = oracle.asral(inst.cm, inst.cap, inst.pen)
     assert ref.stats["moves"] > 0
     assert got["objective"] == ref.delta and np.array_equal(got["assign"], ref.assign)
-    assert got["error"] == "no error"
+    assert got["error"] == "no error" and got["guided"] == 0
