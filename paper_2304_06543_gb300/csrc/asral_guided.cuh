@@ -453,7 +453,8 @@ struct Guided {
             if (vm < paid && lane == 0) atomicMin(&M->paid, vm);
             now = min(bp, vm - 1);
           }
-          const LT key = b + (LT)pv;
+          // (unsigned: a label that is not reached wraps, and is not used)
+          const LT key = (LT)((std::make_unsigned_t<LT>)b + (std::make_unsigned_t<LT>)(LT)pv);
           const bool push = up && (key <= (LT)now || key <= bc);
           if (nthr == 32) bits = __ballot_sync(0xffffffffu, push);
           if (push) {
