@@ -63,7 +63,9 @@ typedef struct lbdd_stats {
   int64_t paths_applied;    /* negative paths removed (Alg. 4) */
   int64_t bf_calls;         /* Bellman-Ford runs (one pruned run may answer Alg. 1
                                and Alg. 4 of a round) */
-  int64_t bf_sweeps;        /* synchronous sweeps over all those runs */
+  int64_t bf_sweeps;        /* synchronous sweeps over all those runs (guided rounds:
+                               this, bf_max_sweeps, front_sum and front_hist may differ
+                               a little from run to run; results do not) */
   int64_t bf_max_sweeps;    /* longest run, in sweeps */
   int64_t moves;            /* demand units transferred between centers */
   int64_t ncyc_skipped;     /* Alg. 1 calls answered without Bellman-Ford because

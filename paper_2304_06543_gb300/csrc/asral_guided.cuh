@@ -29,21 +29,29 @@
 //  * After a cycle was applied, Alg. 4 searches again; the bound uses the
 //    prices raised by the first search's labels, max(P(v), P(j) + L - l1(v))
 //    (L the cycle's cost), less `off`, the most by which those exceed q_n.
+//    These bounds are not tested against the rows that the cycle has just
+//    changed: the table is that of a minimum-cost flow again, for which the
+//    raised prices hold.
 //  * The round ends by raising prices: P(v) = max(P(v), D - l1(v), D2 -
 //    l2(v)), D the shortest way from d to a paid slot (L + D2 after a
 //    cycle, D2 from j).  For a row of T that did not change this keeps both
 //    inequalities by l(v) <= l(u) + T[u][v]; the rows that did change are
-//    tested entry by entry (verify).  Should one ever fail, the prices are
-//    rebuilt from the table by reverse Bellman-Ford sweeps before the next
-//    round, so the pruning never rests on an untested bound.
+//    tested entry by entry (broken_rows), and P(v) <= q_n(v) at the centers of
+//    the applied paths.  Should one ever fail, the prices are rebuilt from the
+//    table by reverse Bellman-Ford sweeps before the next round.
+//  * Which of two equally good bounds a lane sees (the value found so far may
+//    fall during a sweep) changes neither labels nor hop counts of the path,
+//    but how many other labels are expanded: sweep and frontier counters and
+//    prices may differ from run to run, results do not.
 //
 // What this buys (counted on instances of the city shape, 8,000 x 500, and of
 // the batched mix, 6,007 x 126): 48 sweeps of 180 labels and 19 sweeps of 52
 // per round become 10 sweeps of about 30 labels and 3 of about 16; half of the
 // mix's rounds run no sweep at all.  Per call, against the cluster solver on
-// the CTAs it did best on: 317 -> 44 ms for the mix instance, 1,230 -> 289 ms
-// for the city, 37.0 -> 10.3 ms for 2,000 x 20, 540 -> 38 ms for 24 mixed
-// instances in one launch (a cluster each before, a CTA each now).
+// the CTAs it did best on: 317 -> 43 to 46 ms for the mix instance, 1,230 -> 268
+// to 277 ms for the city, 37 -> 10.5 to 11.5 ms for 2,000 x 20, 540 -> 36 to 38
+// ms for 24 mixed instances in one launch (a cluster each before, a CTA each
+// now); 1,000,000 x 500, whose largest center holds 112,000 units, 146 -> 56 s.
 //
 // Bound by the chain of dependent instructions and reads of a round: a warp
 // that runs alone issues about one instruction in five cycles, a dependent
@@ -69,7 +77,9 @@ namespace lbdd {
 constexpr int kGNodeBits = 13;
 constexpr int kGOrd = 64;                       // prefetched (unit, center) pairs
 // Centers up to which the lists of affected entries are as long as
-// guided_list says; beyond, one row's, so that the layout still fits.
+// guided_list says; beyond, one row's.  (The layout would hold eight rows' up to
+// 1,356 centers with int16 and 1,296 with int32 costs, four up to 2,002 and
+// 1,773, at the expense of the L1 that serves the mirror: not measured.)
 constexpr int kGWideLists = 800;
 // Affected entries that an apply lists at a time.  Where the cost table does
 // not fit shared memory anyway there is room for those of eight rows, so that
@@ -105,7 +115,6 @@ __host__ __device__ inline GLayout make_guided_layout(int32_t k, int32_t elem) {
   L.lab1 = take(lt * ku);
   L.lab2 = take(lt * ku);
   L.hop = take(2u * ku);
-  // (large k: one row's entries, so that the layout fits)
   const uint32_t aff = (uint32_t)(k > kGWideLists ? k : guided_list(k, elem));
   L.aff_rows = (int)(aff / ku) < 32 ? (int)(aff / ku) : 32;
   const uint32_t lists = 2u * 2u * lt * (ku + 2);

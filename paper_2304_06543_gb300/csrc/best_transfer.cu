@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(kThreads) bt_unpack(const unsigned long long* 
 // 40 cycles of its pipe per 512 bytes), then the partial tables.  Slices of
 // 64 bytes instead of 128 with int16 costs halve the ranges, their tables and
 // the share of keys that lower an entry: 200,000 x 500 int16 64.0 -> 62.1 us
-// per call.
+// per call on inputs that were read before; on inputs new to L2 no difference.
 constexpr int kStreamThreads = 1024;    // 4 or 8 threads per row slice, 256 or 128 rows at a time
 constexpr int kStreamStages = 5;        // rows in flight per thread (cp.async stages)
 
@@ -1004,7 +1004,7 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
 // 63.6; 30.8, 28.8, 28.7, 30.7; 1,000,000 x 20 49.2, 45.2, 45.1, 47.7.
 //
 // Measured per call, before (seven launches: count, plan, place, sort, scan,
-// unpack and a memset) and after: 2,000 x 20 int32 29.3 -> 10.7 us, 50,001 x
+// unpack and a memset) and after: 2,000 x 20 int32 29.3 -> 10.1 to 12 us, 50,001 x
 // 126 int32 52 -> 24.6 us (28.7 without the next batch in flight).
 //
 // int16 costs and ranges of at most 65,536 rows: one 32-bit key per entry,
