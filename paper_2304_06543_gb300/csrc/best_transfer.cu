@@ -621,8 +621,8 @@ __global__ void __launch_bounds__(kThreads) bt_unpack(const unsigned long long* 
 //
 // Rows of kStreamMinK..kStreamMaxK centers (512 bytes to 2 KB) are short for
 // row gathers, so this path reads the CM in row order instead and needs no
-// grouping.  CTA (j, r) owns the column slice j (32 columns: 64 bytes of int16,
-// 128 of int32 costs) and the row range r, and keeps in shared memory one key per
+// grouping.  CTA (j, r) owns the column slice j (32 or 64 columns of int16, 32
+// of int32 costs: stream_cols) and the row range r, and keeps in shared memory one key per
 // (center, column of the slice): ((t + 32768) << 16) | (d - first row of the
 // range) in 32 bits for int16, ((t + 2^31) << 32) | (d - first row) in 64
 // bits for int32, so the smaller key is the lexicographically smaller (t, d)
@@ -644,6 +644,7 @@ __global__ void __launch_bounds__(kThreads) bt_unpack(const unsigned long long* 
 // 64 bytes instead of 128 with int16 costs halve the ranges, their tables and
 // the share of keys that lower an entry: 200,000 x 500 int16 64.0 -> 62.1 us
 // per call on inputs that were read before; on inputs new to L2 no difference.
+// From about 400,000 rows on the wider slices are the faster ones.
 constexpr int kStreamThreads = 1024;    // 4 or 8 threads per row slice, 256 or 128 rows at a time
 constexpr int kStreamStages = 5;        // rows in flight per thread (cp.async stages)
 
@@ -673,18 +674,15 @@ __device__ __forceinline__ void red_min_if_equal(uint32_t at, uint32_t d, int32_
                ::"r"(at), "r"(d), "r"(t), "r"(cur) : "memory");
 }
 
-// Per cost type: columns per slice, the key, and the key's split into cost
-// and row offset.
+// Per cost type: the key, and the key's split into cost and row offset.
 template <typename T> struct StreamKey;
 template <> struct StreamKey<int16_t> {
   using K = uint32_t;                    // ((t + 32768) << 16) | row offset
-  static constexpr int kCols = 32;       // 64 bytes of a row
   static __device__ __forceinline__ int32_t cost(K key) { return (int32_t)(key >> 16) - 32768; }
   static __device__ __forceinline__ uint32_t offset(K key) { return key & 0xffffu; }
 };
 template <> struct StreamKey<int32_t> {
   using K = unsigned long long;          // ((t + 2^31) << 32) | row offset
-  static constexpr int kCols = 32;       // 128 bytes of a row
   static __device__ __forceinline__ int32_t cost(K key) {
     return (int32_t)((int64_t)(key >> 32) - 2147483648LL);
   }
@@ -699,9 +697,9 @@ __device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontro
 __device__ __forceinline__ void release_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Dynamic shared memory of bt_scan_stream: the key table, then the stages.
-template <typename T>
+template <typename T, int COLS>
 static size_t stream_smem_bytes(int32_t k) {
-  return (size_t)StreamKey<T>::kCols * sizeof(typename StreamKey<T>::K) * (size_t)k +
+  return (size_t)COLS * sizeof(typename StreamKey<T>::K) * (size_t)k +
          (size_t)kStreamStages * kStreamThreads * 16;
 }
 
@@ -709,15 +707,34 @@ static size_t stream_smem_bytes(int32_t k) {
 // int16 keys hold a 16-bit row offset (ranges of at most kStreamRowSpan
 // rows); int32 keys are twice as wide, so at most half as many ranges fit the
 // partial tables' bytes.
-static int stream_ranges(int32_t n, int32_t k, int elem, int num_sms) {
+static int stream_ranges(int32_t n, int32_t k, int elem, int cols, int num_sms) {
   if (k < kStreamMinK || k > kStreamMaxK) return 0;
-  const int cols = elem == 2 ? StreamKey<int16_t>::kCols : StreamKey<int32_t>::kCols;
   const int64_t need = elem == 2 ? ((int64_t)n + kStreamRowSpan - 1) / kStreamRowSpan : 1;
   const int64_t cap = elem == 2 ? std::min<int64_t>(kStreamMaxRanges, n)
                                 : std::min<int64_t>(kStreamMaxRanges / 2, n / 2);
   if (cap < 1 || need > cap) return 0;
   const int nslice = (k + cols - 1) / cols;
   return (int)std::min<int64_t>(cap, std::max<int64_t>(need, num_sms / nslice));
+}
+
+// Columns per slice: int32 32 (128 bytes), int16 32 or 64 (64 or 128 bytes).  A
+// scan takes its waves times the rows of a range times the columns; slices of
+// 64 columns fill the SMs better or worse, need fewer waves where the 65,536
+// rows of a range force many ranges, and write and merge more tables.  They are
+// taken where the time they save, in bytes of the CM, outweighs the tables (us
+// per call, 32 / 64 columns: 200,000 x 500 62.8 / 63.6, 400,000 x 500 104.7 /
+// 100.9, 1,000,000 x 500 265 / 214, 1,000,000 x 300 246 / 147, 1,000,000 x 256
+// 124 / 137, 2,000,000 x 400 402 / 454).
+static int stream_cols(int32_t n, int32_t k, int elem, int num_sms) {
+  if (elem == 4) return 32;
+  const int r32 = stream_ranges(n, k, 2, 32, num_sms), r64 = stream_ranges(n, k, 2, 64, num_sms);
+  if (r32 < 1 || r64 < 1) return 32;
+  auto time = [&](int cols, int ranges) {
+    const int64_t ctas = (int64_t)((k + cols - 1) / cols) * ranges;
+    return (double)((ctas + num_sms - 1) / num_sms) * cols / ranges;
+  };
+  const double saved = 2.0 * n * k * (1.0 - time(64, r64) / time(32, r32));
+  return saved >= 8.0 * k * k * (r64 - r32) ? 64 : 32;
 }
 
 template <typename T>
@@ -735,13 +752,12 @@ __global__ void __launch_bounds__(kThreads) bt_own(const int32_t* __restrict__ a
   }
 }
 
-template <typename T>
+template <typename T, int COLS>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 bt_scan_stream(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
                const int32_t* __restrict__ assign, const int32_t* __restrict__ own, int nslice,
                int nranges, typename StreamKey<T>::K* part) {
   using K = typename StreamKey<T>::K;
-  constexpr int COLS = StreamKey<T>::kCols;
   constexpr int VPL = 16 / (int)sizeof(T);   // columns per thread (16 bytes)
   constexpr int HALF = VPL / 2;              // keys per 16-byte half
   constexpr int P = kStreamStages;
@@ -803,8 +819,8 @@ bt_scan_stream(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
       if (i < M && (kPacked ? ra[q] != 0 : a >= 0 && a < k)) {
         const uint4 x = stage[q * kStreamThreads + tid];
         const uint32_t off = (uint32_t)(rl + RPS * i);
-        // the thread's first HALF keys sit in the row's first 128 bytes, the
-        // others in the second: 8 threads' 16-byte loads cover 32 banks
+        // the thread's first HALF keys sit in the first half of the key row,
+        // the others in the second
         K* lo_p = acc + a * COLS + HALF * cg;
         K* hi_p = lo_p + COLS / 2;
         K key[VPL];
@@ -823,9 +839,9 @@ bt_scan_stream(const T* __restrict__ cm, int64_t ld, int32_t n, int32_t k,
             key[h] = ((K)(uint32_t)((int64_t)w4[h] - o + 2147483648LL) << 32) | off;
         }
         if constexpr (sizeof(T) == 2) {
-          // a key row's halves lie in the two halves of the banks: odd rows
-          // of a warp take theirs in the other order
-          const bool odd = rl & 1;
+          // with 32 columns a key row's halves lie in the two halves of the
+          // banks: odd rows of a warp take theirs in the other order
+          const bool odd = COLS == 32 && (rl & 1);
           const uint32_t la = smem_u32(odd ? hi_p : lo_p), lb = smem_u32(odd ? lo_p : hi_p);
           const uint4 ca = *reinterpret_cast<const uint4*>(odd ? hi_p : lo_p);
           const uint4 cb = *reinterpret_cast<const uint4*>(odd ? lo_p : hi_p);
@@ -923,23 +939,24 @@ __global__ void __launch_bounds__(kThreads) bt_merge_ranges(const K* __restrict_
   }
 }
 
-template <typename T>
+template <typename T, int COLS>
 static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, const int32_t* assign,
-                              int32_t* tc, int32_t* td, const BtWorkspace& W, int nranges,
-                              cudaStream_t st, int num_sms) {
+                              int32_t* tc, int32_t* td, const BtWorkspace& W, cudaStream_t st,
+                              int num_sms) {
   using K = typename StreamKey<T>::K;
+  const int nranges = stream_ranges(n, k, (int)sizeof(T), COLS, num_sms);
   static std::atomic<uint64_t> attr_set{0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!(attr_set.load() & (1ull << dev))) {
-    e = cudaFuncSetAttribute(bt_scan_stream<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)stream_smem_bytes<T>(kStreamMaxK));
+    e = cudaFuncSetAttribute(bt_scan_stream<T, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)stream_smem_bytes<T, COLS>(kStreamMaxK));
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(1ull << dev);
   }
-  const int nslice = (k + StreamKey<T>::kCols - 1) / StreamKey<T>::kCols;
+  const int nslice = (k + COLS - 1) / COLS;
   K* part = reinterpret_cast<K*>(W.part);
   bt_own<T><<<num_sms * 4, kThreads, 0, st>>>(assign, n, k, cm, ld, W.perm);
   // the next two kernels may launch before their predecessor ends; each waits
@@ -953,8 +970,8 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(nslice * nranges);
   cfg.blockDim = dim3(kStreamThreads);
-  cfg.dynamicSmemBytes = stream_smem_bytes<T>(k);
-  e = cudaLaunchKernelEx(&cfg, bt_scan_stream<T>, cm, ld, n, k, assign, (const int32_t*)W.perm,
+  cfg.dynamicSmemBytes = stream_smem_bytes<T, COLS>(k);
+  e = cudaLaunchKernelEx(&cfg, bt_scan_stream<T, COLS>, cm, ld, n, k, assign, (const int32_t*)W.perm,
                          nslice, nranges, part);
   if (e != cudaSuccess) return e;
   cfg.gridDim = dim3(num_sms * 4);
@@ -1459,13 +1476,14 @@ cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_byt
     return elem_bytes == 2
                ? table_call(static_cast<const int16_t*>(cm), ld, n, k, assign, tc, td, base, room, st)
                : table_call(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td, base, room, st);
-  const int nranges = stream_ranges(n, k, elem_bytes, num_sms);
-  if (nranges > 0)
-    return elem_bytes == 2
-               ? stream_run(static_cast<const int16_t*>(cm), ld, n, k, assign, tc, td, W, nranges,
-                            st, num_sms)
-               : stream_run(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td, W, nranges,
-                            st, num_sms);
+  const int cols = stream_cols(n, k, elem_bytes, num_sms);
+  if (stream_ranges(n, k, elem_bytes, cols, num_sms) > 0) {
+    const int16_t* c16 = static_cast<const int16_t*>(cm);
+    const int32_t* c32 = static_cast<const int32_t*>(cm);
+    return elem_bytes == 4 ? stream_run<int32_t, 32>(c32, ld, n, k, assign, tc, td, W, st, num_sms)
+           : cols == 32    ? stream_run<int16_t, 32>(c16, ld, n, k, assign, tc, td, W, st, num_sms)
+                           : stream_run<int16_t, 64>(c16, ld, n, k, assign, tc, td, W, st, num_sms);
+  }
   cudaError_t e = cudaMemsetAsync(W.ctl, 0, 4 * BT_CTL_WORDS + 4ull * (k + 1), st);
   if (e != cudaSuccess) return e;
   bt_count<<<kTiles, kTileThreads, 4 * (size_t)k, st>>>(assign, n, k, W.cnt, W.tile_rel);
