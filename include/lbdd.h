@@ -381,10 +381,9 @@ const char* lbdd_last_cuda_error(void);
  *   workspace  : device scratch of lbdd_best_transfer_workspace(n, k) bytes,
  *                owned by the caller; contents on entry are ignored.  With
  *                fewer than 256 centers and more than 4 MB of int32 costs
- *                this counts 40 packed k x k tables (8k^2 bytes each); a size
- *                with room for fewer of them, down to 4n + n/4 + 8k^2 + 276k
- *                bytes and 2 KB, gives the same table by fewer, larger
- *                clusters.
+ *                this counts 40 or more packed k x k tables (8k^2 bytes each);
+ *                a size with room for fewer of them, down to 4n + n/4 + 8k^2 +
+ *                276k bytes and 2 KB, gives the same table in more time.
  *   stream     : cudaStream_t or NULL.  Asynchronous: results are ready
  *                when the stream reaches this point.
  * Errors: LBDD_ERR_ARG (sizes, alignment, workspace too small),
@@ -405,7 +404,8 @@ int lbdd_best_transfer(int32_t n, int32_t k, const void* cm_dev, int cm_dtype, i
  * loads this library until the process exits.
  *   Arguments as for lbdd_best_transfer (inputs and outputs are still the
  *   caller's device buffers), without the workspace.
- *   Limit: lbdd_best_transfer_workspace(n, k) must not exceed 64 MiB, else
+ *   Limit: lbdd_best_transfer_workspace(n, k) (fewer than 256 centers: the
+ *   least workspace named there) must not exceed 64 MiB, else
  *   LBDD_ERR_BUDGET is returned and nothing is launched (the city-scale
  *   200,000 x 500 case needs 34,988,800 bytes, about 33.4 MiB).
  *   The first call on each device looks up the device address of the array

@@ -100,6 +100,7 @@ static BtWorkspace carve(void* base, int32_t n, int32_t k) {
 }
 
 static size_t table_part_bytes(int32_t n, int32_t k);
+static size_t long_part_bytes(int32_t n, int32_t k);
 
 // The least a call accepts, and what it makes full use of: the packed tables of
 // short rows take the place of everything else, as many as there is room for.
@@ -107,7 +108,9 @@ size_t bt_workspace_min(int32_t n, int32_t k) {
   return n < 1 || k < 1 ? 0 : carve(nullptr, n, k).bytes + 256;
 }
 size_t bt_workspace_bytes(int32_t n, int32_t k) {
-  return n < 1 || k < 1 ? 0 : std::max(bt_workspace_min(n, k), table_part_bytes(n, k) + 256);
+  return n < 1 || k < 1 ? 0
+                        : std::max({bt_workspace_min(n, k), table_part_bytes(n, k) + 256,
+                                    long_part_bytes(n, k) + 256});
 }
 
 // ------------------------------------------------------------- grouping ---
@@ -306,6 +309,7 @@ __global__ void __launch_bounds__(kThreads) bt_sort_items(const int4* __restrict
 // bounded: past kScanWaitLimitNs the waiter sets ctl[BT_ERR] and leaves (the
 // producer first waits, bounded, for its copies in flight), and bt_unpack
 // then marks the whole table.
+constexpr int kBulkMinRowBytes = 512;
 constexpr int kStageBytes = 32768;       // target bytes per stage (the producer's cost is per stage)
 constexpr int kSmemLimit = 232448;       // dynamic shared memory of one CTA (227 KB)
 constexpr int kMaxStages = 16;
@@ -939,12 +943,12 @@ __global__ void __launch_bounds__(kThreads) bt_merge_ranges(const K* __restrict_
   }
 }
 
+// own: n words; part: nranges tables of k x k keys.
 template <typename T, int COLS>
 static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, const int32_t* assign,
-                              int32_t* tc, int32_t* td, const BtWorkspace& W, cudaStream_t st,
-                              int num_sms) {
+                              int32_t* tc, int32_t* td, int32_t* own, void* parts, int nranges,
+                              cudaStream_t st, int num_sms) {
   using K = typename StreamKey<T>::K;
-  const int nranges = stream_ranges(n, k, (int)sizeof(T), COLS, num_sms);
   static std::atomic<uint64_t> attr_set{0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -957,8 +961,8 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
     attr_set.fetch_or(1ull << dev);
   }
   const int nslice = (k + COLS - 1) / COLS;
-  K* part = reinterpret_cast<K*>(W.part);
-  bt_own<T><<<num_sms * 4, kThreads, 0, st>>>(assign, n, k, cm, ld, W.perm);
+  K* part = static_cast<K*>(parts);
+  bt_own<T><<<num_sms * 4, kThreads, 0, st>>>(assign, n, k, cm, ld, own);
   // the next two kernels may launch before their predecessor ends; each waits
   // for it (wait_predecessor) before reading its results
   cudaLaunchAttribute pdl[1];
@@ -971,7 +975,7 @@ static cudaError_t stream_run(const T* cm, int64_t ld, int32_t n, int32_t k, con
   cfg.gridDim = dim3(nslice * nranges);
   cfg.blockDim = dim3(kStreamThreads);
   cfg.dynamicSmemBytes = stream_smem_bytes<T, COLS>(k);
-  e = cudaLaunchKernelEx(&cfg, bt_scan_stream<T, COLS>, cm, ld, n, k, assign, (const int32_t*)W.perm,
+  e = cudaLaunchKernelEx(&cfg, bt_scan_stream<T, COLS>, cm, ld, n, k, assign, (const int32_t*)own,
                          nslice, nranges, part);
   if (e != cudaSuccess) return e;
   cfg.gridDim = dim3(num_sms * 4);
@@ -1091,6 +1095,24 @@ static bool tables_in_workspace(int32_t n, int32_t k) {
 static size_t table_part_bytes(int32_t n, int32_t k) {
   if (!tables_in_workspace(n, k)) return 0;
   return 8ull * k * k * kTableMaxClusters;
+}
+
+// Long tables of int32 costs, from kLongK centers and kLongBytes of costs on: the
+// two-word table scan goes through every batch twice, the row-order scan of 256
+// centers and more (64-bit keys) once, at the price of bt_own and more partial
+// tables, which is why it does not pay below (us per call, table / row order:
+// 200,000 x 64 35.2 / 42.0, 400,000 x 64 64.6 / 54.1, 200,000 x 100 49.8 / 39.9,
+// 400,000 x 40 39.3 / 41.4, 1,000,000 x 255 544 / 211).  The seven launches took
+// 187 us at 1,000,000 x 100 and 337 at 1,000,000 x 255, the table scan 217 and 544.
+// A workspace without room for half the row ranges goes the grouped way, where
+// its rows are long enough for bulk copies.
+constexpr int kLongK = 64;
+constexpr int64_t kLongBytes = 64 << 20;
+static bool long_table(int32_t n, int32_t k) {
+  return k >= kLongK && k < kStreamMinK && (int64_t)n * k * 4 >= kLongBytes;
+}
+static size_t long_part_bytes(int32_t n, int32_t k) {   // (152 SMs)
+  return long_table(n, k) ? al256(4ull * n) + 8ull * k * k * (size_t)(152 / ((k + 31) / 32)) : 0;
 }
 
 // What CTA (slice, range) of a table scan reads.
@@ -1472,17 +1494,33 @@ cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_byt
   void* base = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
   const BtWorkspace W = carve(base, n, k);
   const size_t room = ws_bytes - (size_t)(static_cast<char*>(base) - static_cast<char*>(ws));
-  if (k < kStreamMinK)
+  bool grouped = false;   // the row gathers below 256 centers
+  if (elem_bytes == 4 && long_table(n, k)) {
+    const int nslice = (k + 31) / 32;
+    const size_t own = al256(4ull * n);
+    const int ranges =
+        (int)std::min<size_t>(num_sms / nslice, room > own ? (room - own) / (8ull * k * k) : 0);
+    if (2 * ranges * nslice > num_sms)
+      return stream_run<int32_t, 32>(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td,
+                                     static_cast<int32_t*>(base), static_cast<char*>(base) + own,
+                                     ranges, st, num_sms);
+    grouped = 4 * k >= kBulkMinRowBytes;
+  }
+  if (k < kStreamMinK && !grouped)
     return elem_bytes == 2
                ? table_call(static_cast<const int16_t*>(cm), ld, n, k, assign, tc, td, base, room, st)
                : table_call(static_cast<const int32_t*>(cm), ld, n, k, assign, tc, td, base, room, st);
   const int cols = stream_cols(n, k, elem_bytes, num_sms);
-  if (stream_ranges(n, k, elem_bytes, cols, num_sms) > 0) {
+  const int nranges = stream_ranges(n, k, elem_bytes, cols, num_sms);
+  if (nranges > 0) {
+    auto run = [&](auto* c, auto width) {
+      return stream_run<std::remove_const_t<std::remove_pointer_t<decltype(c)>>, width.value>(
+          c, ld, n, k, assign, tc, td, W.perm, W.part, nranges, st, num_sms);
+    };
     const int16_t* c16 = static_cast<const int16_t*>(cm);
-    const int32_t* c32 = static_cast<const int32_t*>(cm);
-    return elem_bytes == 4 ? stream_run<int32_t, 32>(c32, ld, n, k, assign, tc, td, W, st, num_sms)
-           : cols == 32    ? stream_run<int16_t, 32>(c16, ld, n, k, assign, tc, td, W, st, num_sms)
-                           : stream_run<int16_t, 64>(c16, ld, n, k, assign, tc, td, W, st, num_sms);
+    return elem_bytes == 4 ? run(static_cast<const int32_t*>(cm), std::integral_constant<int, 32>())
+           : cols == 32    ? run(c16, std::integral_constant<int, 32>())
+                           : run(c16, std::integral_constant<int, 64>());
   }
   cudaError_t e = cudaMemsetAsync(W.ctl, 0, 4 * BT_CTL_WORDS + 4ull * (k + 1), st);
   if (e != cudaSuccess) return e;

@@ -15,7 +15,7 @@
 #include "lbdd_device.cuh"
 
 namespace lbdd {
-size_t bt_workspace_bytes(int32_t n, int32_t k);
+size_t bt_workspace_min(int32_t n, int32_t k);
 int bt_max_k(int elem_bytes);
 cudaError_t best_transfer_run(int32_t n, int32_t k, const void* cm, int elem_bytes, int64_t ld,
                               const int32_t* assign, int32_t* tc, int32_t* td, void* ws,
@@ -68,7 +68,7 @@ extern "C" int lbdd_best_transfer_noalloc(int32_t n, int32_t k, const void* cm_d
     return LBDD_ERR_ARG;
   if (k > lbdd::bt_max_k(elem)) return LBDD_ERR_ARG;
   // the scratch the scan needs must fit in the fixed array
-  if (lbdd::bt_workspace_bytes(n, k) > kStaticScratchBytes) return LBDD_ERR_BUDGET;
+  if (lbdd::bt_workspace_min(n, k) > kStaticScratchBytes) return LBDD_ERR_BUDGET;
   int dev = 0;
   const cudaError_t ed = cudaGetDevice(&dev);
   if (ed != cudaSuccess) return lbdd::cuda_fail(ed, "cudaGetDevice");
