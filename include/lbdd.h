@@ -342,7 +342,12 @@ int lbdd_rounds_done(const lbdd_solver* s, int64_t* out);
  * with full Bellman-Fords (asral_cluster_kernel).  Guided rounds need both
  * LBDD_OPT_NCYC_SKIP and LBDD_OPT_NPATH_REUSE on, penalties below 2^30 (strict
  * solvers: costs below 2^30), at most 2,680 centers with int16 and 1,954 with
- * int32 costs, and device memory for one more copy of the best-transfer costs.  Either way the result is the same; only the time differs. */
+ * int32 costs, and device memory for one more copy of the best-transfer costs.
+ * Where rounds scan very long member lists for many entries (one center that
+ * holds tens of thousands of units and loses the best unit of most entries),
+ * the next rounds run on the other kernel, in stretches of 4,096 rounds and
+ * more, inside the same call.  Either way the result is the same; only the
+ * time differs. */
 int lbdd_guided_rounds(const lbdd_solver* s, int64_t* out);
 
 /* Counters of the solve so far (host struct). */

@@ -158,12 +158,38 @@ template <> struct __align__(16) GEnt<int64_t> { int64_t l; uint32_t off, pad; }
 constexpr int32_t kGPenLimit = 1 << 30;
 constexpr int32_t kGNever = kGPenLimit + (1 << 29);   // a price or slot out of every bound
 
+// Rounds that scan long member lists for many entries.  One SM gathers them,
+// where the full Bellman-Ford kernel shares them between the CTAs of a cluster
+// and reads whole rows when most entries of one are affected.  A scan task (32
+// lanes times 16 members) takes about 0.1 us on one CTA; past a number of tasks
+// per round the other kernel is the faster one:
+//  * `wide` tasks, of rows with more than half their entries affected.  Us per
+//    round, guided / full: 20 centers, 660 tasks 73 / 54; 64, 1,270 tasks 129 /
+//    70; 126, 7,900 tasks 837 / 182; 500, 31,700 tasks 3,375 / 187.
+//  * all tasks, from kHeavyK centers on, where the cluster has 16 CTAs: 256,
+//    2,500 tasks 315 / 310; 500, 990 tasks 172 / 177, 2,270 tasks 311 / 249;
+//    1,000, 2,270 tasks 400 / 298; 1,800, 3,940 tasks 1,129 / 1,352, 4,480 tasks
+//    1,897 / 1,639.  (126 centers, 2,040 tasks 242 / 328.)
+// (One center takes half of 20,000 to 60,000 units.  Instances of the city shape
+// have at most 360 tasks per round.)  What rounds scan beyond the limits adds
+// up (a round below them takes the difference off again); past kHeavyRounds
+// limits the rounds end and the host runs the next ones on the other kernel.
+// Counted where a list took more than one task and looked at every kHeavyEvery
+// rounds: in every apply and round it made the smallest solves 3 to 7 % slower.
+constexpr int kHeavyK = 240;
+constexpr int kHeavyRounds = 48, kHeavyEvery = 64;
+__host__ __device__ inline int64_t heavy_wide(int32_t k) { return 500 + k / 2; }
+__host__ __device__ inline int64_t heavy_scans(int32_t k) {
+  return k < kHeavyK ? (int64_t)1 << 40 : k < 320 ? 2500 : 1500 + (k > 1200 ? 9 * (int64_t)(k - 1200) / 2 : 0);
+}
+
 struct GMisc {
   int32_t paid;       // best value of a path to a paid slot in the last search
   uint32_t sink;      // its hop count << kGNodeBits | node, if paid < ql
   uint32_t next[3];   // parents on the way back, by hop count modulo 3
   int32_t cnt[3];     // list lengths, by sweep modulo 3
-  int32_t len, bad, stop;
+  int32_t len, bad, stop, heavy;
+  int32_t scans, wide;   // scan tasks since they were looked at: the other rows', the wide ones'
 };
 
 template <typename T, bool TSM, bool STRICT>
@@ -678,9 +704,13 @@ struct Guided {
       if (split) {
         for (int r = warp; r < i1 - i0; r += kWarps) {
           const int na_r = __shfl_sync(0xffffffffu, na, r);
-          if (__shfl_sync(0xffffffffu, parts, r) > 1)
+          const int parts_r = __shfl_sync(0xffffffffu, parts, r);
+          if (parts_r > 1) {
             for (int e = lane; e < na_r; e += 32)
               put_entry(s_path[i0 + r], s_aff[r * k + e], best_of(r * k + e));
+            // (see heavy_scans)
+            if (lane == 0) atomicAdd(2 * na_r > k ? &M->wide : &M->scans, ((na_r + 31) >> 5) * parts_r);
+          }
         }
       }
       if (split || i1 < m) __syncthreads();
@@ -905,6 +935,16 @@ struct Guided {
     }
   }
 
+  // Thread 0: the levels after the rounds before round q (see heavy_scans).
+  __device__ __forceinline__ void count_scans(int32_t q) {
+    const int64_t rounds = q - B->level_q;
+    B->level = max((int64_t)0, B->level + M->scans + M->wide - rounds * B->scans_limit);
+    B->level_wide = max((int64_t)0, B->level_wide + M->wide - rounds * B->wide_limit);
+    B->level_q = q;
+    M->scans = M->wide = 0;
+    M->heavy = B->level > kHeavyRounds * B->scans_limit || B->level_wide > kHeavyRounds * B->wide_limit;
+  }
+
   // Rows list[0..m) of T against the prices: sets M->bad if an entry breaks
   // P(u) <= T[u][v] + P(v), or a price exceeds q_n.
   __device__ bool broken_rows(const int32_t* list, int m) {
@@ -1037,8 +1077,15 @@ struct Guided {
       B->col_rows = 0;
       B->front_sum = 0;
       for (int h = 0; h < 6; ++h) B->front_hist[h] = 0;
+      M->scans = M->wide = 0;
+      B->level = I.ctl[CTL_LEVEL];
+      B->level_wide = I.ctl[CTL_LEVEL_WIDE];
       M->bad = 0;
       M->stop = 0;
+      B->level_q = 0;
+      B->scans_limit = flags & OPT_NO_EXIT ? (int64_t)1 << 40 : heavy_scans(k);
+      B->wide_limit = flags & OPT_NO_EXIT ? (int64_t)1 << 40 : heavy_wide(k);
+      M->heavy = 0;
     }
     if (TSM || I.ctl[CTL_MIRROR] == 0)
       for (int64_t u = 0; u < k; ++u)
@@ -1054,9 +1101,14 @@ struct Guided {
     int64_t status = ST_OK;
     int32_t q = 0;
     for (int i = 0; i + 1 < nring; ++i) fetch_row(i, count);
+    const int32_t look = (deadline ? kQuantumCheck : kHeavyEvery) - 1;
+    static_assert((kQuantumCheck & (kQuantumCheck - 1)) == 0 && kHeavyEvery % kQuantumCheck == 0, "");
     for (; q < count; ++q) {
-      if (deadline && q > 0 && q % kQuantumCheck == 0) {
-        if (tid == 0) M->stop = gtimer_ns() >= deadline ? 1 : 0;
+      if ((q & look) == 0) {   // (at once inside a stretch of the other kernel)
+        if (tid == 0) {
+          if (q % kHeavyEvery == 0) count_scans(q);
+          M->stop = M->heavy || (deadline && q > 0 && gtimer_ns() >= deadline);
+        }
         __syncthreads();
         if (M->stop) break;
       }
@@ -1186,6 +1238,11 @@ struct Guided {
       if (count > 0) I.ctl[CTL_MIRROR] = TSM ? 0 : 1;
       I.ctl[CTL_ROUNDS] = r_begin + q;
       I.ctl[CTL_GUIDED] += q;
+      const int ended = M->heavy;
+      count_scans(q);
+      I.ctl[CTL_LEVEL] = B->level;
+      I.ctl[CTL_LEVEL_WIDE] = B->level_wide;
+      if (ended && r_begin + q < r_end) I.ctl[CTL_HEAVY] = 1;
       I.ctl[CTL_DELTA] = B->delta;
       I.ctl[CTL_FREE_TOP] = B->free_top;
       I.ctl[CTL_STATUS] = status != ST_OK ? status : B->err0;

@@ -118,6 +118,8 @@ struct Book {
   int64_t t_merge, t_relax, t_sync, t_gather, t_apply, t_rescan, t_rloop, t_rred;
   int64_t npath_reused, col_rows, front_sum, front_hist[6];
   int64_t err0;   // a guard tripped (corrupt state; never expected)
+  // guided rounds: see heavy_scans
+  int64_t scans_limit, wide_limit, level, level_wide, level_q;
   uint64_t deadline;   // globaltimer ns at which the launch yields (0: never)
 };
 

@@ -525,7 +525,7 @@ int lbdd::status_to_rc(int64_t st) {
   return LBDD_ERR_STATE;
 }
 
-static int set_target(lbdd_solver* s, int64_t max_rounds, cudaStream_t st) {
+static int set_target(lbdd_solver* s, int64_t max_rounds, cudaStream_t st, int64_t* to = nullptr) {
   int64_t h[2];
   CK(cudaMemcpyAsync(h, s->ctl + CTL_ROUNDS, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(h + 1, s->ctl + CTL_STATUS, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -534,7 +534,23 @@ static int set_target(lbdd_solver* s, int64_t max_rounds, cudaStream_t st) {
   const int64_t target = max_rounds < 0 ? (int64_t)s->n : std::min<int64_t>(s->n, h[0] + max_rounds);
   CK(cudaMemcpyAsync(s->ctl + CTL_TARGET, &target, sizeof(int64_t), cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));
+  s->round = h[0];
+  if (to) *to = target;
   return LBDD_OK;
+}
+
+void lbdd::note_heavy(lbdd_solver* s, int64_t round) {
+  s->round = round;
+  if (round < s->full_until) return;   // ended at once, inside a stretch
+  s->stretch = std::min<int64_t>(std::max<int64_t>(4096, 2 * s->stretch), (int64_t)1 << 40);
+  s->full_until = round + s->stretch;
+}
+
+cudaError_t lbdd::next_stop(lbdd_solver* s, int64_t target, cudaStream_t st, int64_t* stop) {
+  *stop = s->round < s->full_until ? std::min(target, s->full_until) : target;
+  if (s->full_until == 0 || s->round < s->full_until) return cudaSuccess;
+  s->full_until = 0;
+  return cudaMemsetAsync(s->ctl + CTL_LEVEL, 0, 2 * sizeof(int64_t), st);   // and CTL_LEVEL_WIDE
 }
 
 int lbdd::solver_flags(const lbdd_solver* s) {
@@ -544,6 +560,7 @@ int lbdd::solver_flags(const lbdd_solver* s) {
 }
 
 bool lbdd::solver_guided(const lbdd_solver* s, int C) {
+  if (s->round < s->full_until) return false;
   if (!s->ncyc_skip || !s->npath_reuse || !s->mirror || s->max_pen >= guided_pen_limit() ||
       guided_smem_bytes(s->k, s->elem, kMaxSmem) == 0)
     return false;
@@ -585,21 +602,37 @@ int lbdd::choose_cluster(lbdd_solver* s) {
 
 extern "C" int lbdd_solve(lbdd_solver* s, int64_t max_rounds) {
   if (!s) return LBDD_ERR_ARG;
-  int rc = set_target(s, max_rounds, s->st);
+  int64_t target = 0;
+  int rc = set_target(s, max_rounds, s->st, &target);
   if (rc) return rc;
-  const int C = choose_cluster(s);
-  if (C < 1) return LBDD_ERR_ARG;
-  const size_t smem = launch_smem_of(s, C);
-  CK(cudaMemsetAsync(s->counter, 0, 2 * sizeof(int32_t), s->st));
-  if (s->cluster == 0 && prologue_first(s, C, max_rounds, 0))
-    CK(launch_solver(s->d_inst, 1, s->counter + 1, kPrologueCluster, 1, s->elem, smem,
-                     launch_flags(s, C) | OPT_PROLOGUE, s->st));
-  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, launch_flags(s, C), s->st));
-  int64_t st = 0;
-  CK(cudaMemcpyAsync(&st, s->ctl + CTL_STATUS, sizeof(int64_t), cudaMemcpyDeviceToHost, s->st));
-  CK(cudaStreamSynchronize(s->st));
-  s->fresh = false;
-  return status_to_rc(st);
+  for (;;) {   // one launch, unless guided rounds end early
+    int64_t stop = target;
+    CK(next_stop(s, target, s->st, &stop));
+    if (stop != target)
+      CK(cudaMemcpyAsync(s->ctl + CTL_TARGET, &stop, sizeof(int64_t), cudaMemcpyHostToDevice, s->st));
+    const int C = choose_cluster(s);
+    if (C < 1) return LBDD_ERR_ARG;
+    const size_t smem = launch_smem_of(s, C);
+    CK(cudaMemsetAsync(s->counter, 0, 2 * sizeof(int32_t), s->st));
+    if (s->cluster == 0 && prologue_first(s, C, max_rounds, 0))
+      CK(launch_solver(s->d_inst, 1, s->counter + 1, kPrologueCluster, 1, s->elem, smem,
+                       launch_flags(s, C) | OPT_PROLOGUE, s->st));
+    CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, launch_flags(s, C), s->st));
+    int64_t c[CTL_COUNT];
+    CK(cudaMemcpyAsync(c, s->ctl, sizeof(c), cudaMemcpyDeviceToHost, s->st));
+    CK(cudaStreamSynchronize(s->st));
+    s->fresh = false;
+    const int64_t from = s->round;
+    s->round = c[CTL_ROUNDS];
+    if (c[CTL_STATUS] != 0 || s->round >= target) return status_to_rc(c[CTL_STATUS]);
+    if (c[CTL_HEAVY]) {
+      note_heavy(s, c[CTL_ROUNDS]);
+      CK(cudaMemsetAsync(s->ctl + CTL_HEAVY, 0, sizeof(int64_t), s->st));
+    } else if (s->round == from) {
+      return LBDD_ERR_STATE;   // (no launch ends without a round otherwise)
+    }
+    CK(cudaMemcpyAsync(s->ctl + CTL_TARGET, &target, sizeof(int64_t), cudaMemcpyHostToDevice, s->st));
+  }
 }
 
 int lbdd::solve_timed(lbdd_solver* s, int64_t max_rounds, int C, float* ms) {
@@ -617,10 +650,10 @@ int lbdd::solve_timed(lbdd_solver* s, int64_t max_rounds, int C, float* ms) {
   CK(cudaEventCreate(&ev.a));
   CK(cudaEventCreate(&ev.b));
   CK(cudaMemsetAsync(s->counter, 0, sizeof(int32_t), s->st));
-  CK(prepare_solver(C, s->elem, smem, launch_flags(s, C)));
+  const int flags = launch_flags(s, C) | OPT_NO_EXIT;
+  CK(prepare_solver(C, s->elem, smem, flags));
   CK(cudaEventRecord(ev.a, s->st));
-  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, launch_flags(s, C), s->st, 0,
-                   false));
+  CK(launch_solver(s->d_inst, 1, s->counter, C, 1, s->elem, smem, flags, s->st, 0, false));
   CK(cudaEventRecord(ev.b, s->st));
   int64_t st = 0;
   CK(cudaMemcpyAsync(&st, s->ctl + CTL_STATUS, sizeof(int64_t), cudaMemcpyDeviceToHost, s->st));
@@ -774,6 +807,7 @@ extern "C" int lbdd_insert(lbdd_solver* s, const void* row, int cm_dtype, int32_
 extern "C" int lbdd_reset(lbdd_solver* s) {
   if (!s) return LBDD_ERR_ARG;
   s->fresh = true;
+  s->round = s->full_until = s->stretch = 0;
   CK(cudaMemsetAsync(s->ctl, 0, sizeof(int64_t) * CTL_COUNT, s->st));
   CK(cudaMemsetAsync(s->assign, 0xff, 4ull * s->n, s->st));
   CK(cudaMemsetAsync(s->load, 0, 4ull * s->k, s->st));

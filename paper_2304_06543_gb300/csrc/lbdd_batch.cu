@@ -52,13 +52,18 @@ __global__ void batch_set_targets(const DevInst* __restrict__ insts, int m,
   c[CTL_TARGET] = mr < 0 ? n : min(n, c[CTL_ROUNDS] + mr);
 }
 
-// out[2i] = status, out[2i+1] = rounds done of instance i.
+// out[kOut i ...] = status, rounds done, whether guided rounds ended early, and
+// round target of instance i.
+constexpr int kOut = 4;
 __global__ void batch_gather(const DevInst* __restrict__ insts, int m, int64_t* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
-  const int64_t* c = insts[i].ctl;
-  out[2 * i] = c[CTL_STATUS];
-  out[2 * i + 1] = c[CTL_ROUNDS];
+  int64_t* c = insts[i].ctl;
+  out[kOut * i] = c[CTL_STATUS];
+  out[kOut * i + 1] = c[CTL_ROUNDS];
+  out[kOut * i + 2] = c[CTL_HEAVY];
+  out[kOut * i + 3] = c[CTL_TARGET];
+  c[CTL_HEAVY] = 0;
 }
 
 // --------------------------------------------------------- tuning table ---
@@ -321,6 +326,7 @@ struct lbdd_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   uint64_t quantum_ns = 0;
+  int forced = 0, max_clusters = 0; // as batch_set got them
   int launches = 0;                 // kernels of the last pass
   int dev = 0, sms = 0;
 };
@@ -345,12 +351,15 @@ static void batch_free(lbdd_batch* b) {
   delete b;
 }
 
-// Issues one pass of the batch on b->st (asynchronous).
-static int batch_enqueue(lbdd_batch* b) {
+// Issues one pass of the batch on b->st (asynchronous).  targets: set them from
+// h_params (otherwise they stand).
+static int batch_enqueue(lbdd_batch* b, bool targets = true) {
   const int m = (int)b->solvers.size();
-  CK(cudaMemcpyAsync(b->d_params, b->h_params, sizeof(int64_t), cudaMemcpyHostToDevice, b->st));
-  batch_set_targets<<<(m + 255) / 256, 256, 0, b->st>>>(b->d_insts, m, b->d_params);
-  CK(cudaGetLastError());
+  if (targets) {
+    CK(cudaMemcpyAsync(b->d_params, b->h_params, sizeof(int64_t), cudaMemcpyHostToDevice, b->st));
+    batch_set_targets<<<(m + 255) / 256, 256, 0, b->st>>>(b->d_insts, m, b->d_params);
+    CK(cudaGetLastError());
+  }
   CK(cudaMemsetAsync(b->d_counters, 0, sizeof(int) * b->groups.size(), b->st));
   CK(cudaEventRecord(b->fork, b->st));
   for (size_t g = 0; g < b->groups.size(); ++g) {
@@ -366,7 +375,7 @@ static int batch_enqueue(lbdd_batch* b) {
   }
   batch_gather<<<(m + 255) / 256, 256, 0, b->st>>>(b->d_insts, m, b->d_out);
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(b->h_out, b->d_out, sizeof(int64_t) * 2 * m, cudaMemcpyDeviceToHost, b->st));
+  CK(cudaMemcpyAsync(b->h_out, b->d_out, sizeof(int64_t) * kOut * m, cudaMemcpyDeviceToHost, b->st));
   return LBDD_OK;
 }
 
@@ -392,10 +401,10 @@ int batch_alloc(lbdd_batch** out, int capacity, uint64_t quantum_ns, void* strea
   if ((e = cudaMalloc(&b->d_insts, sizeof(DevInst) * capacity))) return cf(e, "batch insts");
   if ((e = cudaMalloc(&b->d_counters, sizeof(int) * 2 * kMaxGroups))) return cf(e, "batch counters");
   if ((e = cudaMalloc(&b->d_params, sizeof(int64_t) * 2))) return cf(e, "batch params");
-  if ((e = cudaMalloc(&b->d_out, sizeof(int64_t) * 2 * capacity))) return cf(e, "batch out");
+  if ((e = cudaMalloc(&b->d_out, sizeof(int64_t) * kOut * capacity))) return cf(e, "batch out");
   if ((e = cudaMallocHost(&b->h_insts, sizeof(DevInst) * capacity))) return cf(e, "batch insts (host)");
   if ((e = cudaMallocHost(&b->h_params, sizeof(int64_t) * 2))) return cf(e, "batch params (host)");
-  if ((e = cudaMallocHost(&b->h_out, sizeof(int64_t) * 2 * capacity))) return cf(e, "batch out (host)");
+  if ((e = cudaMallocHost(&b->h_out, sizeof(int64_t) * kOut * capacity))) return cf(e, "batch out (host)");
   if ((e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming))) return cf(e, "event");
   for (int g = 0; g < kMaxGroups - 1; ++g) {
     if ((e = cudaStreamCreateWithFlags(&b->side[g], cudaStreamNonBlocking))) return cf(e, "stream");
@@ -418,6 +427,8 @@ int batch_set(lbdd_batch* b, lbdd_solver* const* solvers, const int64_t* rem, in
     if (!solvers[i] || solvers[i]->device != b->dev) return LBDD_ERR_ARG;
     r[i] = rem ? std::max<int64_t>(rem[i], 1) : solvers[i]->n;
   }
+  b->forced = cluster_size;
+  b->max_clusters = max_clusters;
   for (lbdd_solver* old : b->solvers) old->in_batches--;
   b->solvers.assign(solvers, solvers + m);
   for (lbdd_solver* x : b->solvers) x->in_batches++;
@@ -490,6 +501,10 @@ int batch_launch(lbdd_batch* b, int64_t max_rounds) {
   b->h_params[0] = max_rounds;
   for (auto& g : b->groups) CK(prepare_solver(g.C, g.elem, g.smem, g.flags));
   b->launches = 2 + (int)b->groups.size();
+  for (lbdd_solver* s : b->solvers) {   // (stretches that are over are forgotten)
+    int64_t stop = 0;
+    CK(next_stop(s, s->n, b->st, &stop));
+  }
   const int rc = batch_prologues(b, max_rounds);
   if (rc) return rc;
   if (b->exec) {
@@ -504,8 +519,12 @@ int batch_wait(lbdd_batch* b, int* first_rc) {
   CK(cudaStreamSynchronize(b->st));
   int first = LBDD_OK;
   for (size_t i = 0; i < b->solvers.size(); ++i) {
-    if (b->h_out[2 * b->slot_of[i] + 1] > 0) b->solvers[i]->fresh = false;
-    const int r = status_to_rc(b->h_out[2 * b->slot_of[i]]);
+    const int64_t* out = b->h_out + kOut * b->slot_of[i];
+    lbdd_solver* s = b->solvers[i];
+    if (out[1] > 0) s->fresh = false;
+    s->round = out[1];
+    if (out[2]) note_heavy(s, out[1]);
+    const int r = status_to_rc(out[0]);
     if (r && first == LBDD_OK) first = r;
   }
   if (first_rc) *first_rc = first;
@@ -520,10 +539,63 @@ void batch_detach(lbdd_batch* b) {
 }
 
 int batch_launches(const lbdd_batch* b) { return b->launches; }
-int64_t batch_rounds(const lbdd_batch* b, int i) { return b->h_out[2 * b->slot_of[i] + 1]; }
-int64_t batch_status(const lbdd_batch* b, int i) { return b->h_out[2 * b->slot_of[i]]; }
+int64_t batch_rounds(const lbdd_batch* b, int i) { return b->h_out[kOut * b->slot_of[i] + 1]; }
+int64_t batch_status(const lbdd_batch* b, int i) { return b->h_out[kOut * b->slot_of[i]]; }
 void batch_destroy(lbdd_batch* b) {
   if (b) batch_free(b);
+}
+
+// Runs the instances whose guided rounds ended early to their targets: passes
+// of the others' kind, stretch by stretch, planned afresh.
+static int batch_finish(lbdd_batch* b, int* first_rc) {
+  std::vector<lbdd_solver*> v;
+  std::vector<int64_t> target;
+  for (size_t i = 0; i < b->solvers.size(); ++i) {
+    const int64_t* out = b->h_out + kOut * b->slot_of[i];
+    if (out[0] == 0 && out[1] < out[3]) {
+      v.push_back(b->solvers[i]);
+      target.push_back(out[3]);
+    }
+  }
+  while (!v.empty()) {
+    const int m = (int)v.size();
+    lbdd_batch* p = nullptr;
+    int rc = batch_alloc(&p, m, 0, b->st);
+    if (rc) return rc;
+    std::vector<int64_t> stop(m), rem(m), from(m);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < m && !e; ++i) {
+      from[i] = v[i]->round;
+      e = next_stop(v[i], target[i], b->st, &stop[i]);
+      rem[i] = stop[i] - from[i];
+      if (!e)
+        e = cudaMemcpyAsync(v[i]->ctl + CTL_TARGET, &stop[i], sizeof(int64_t),
+                            cudaMemcpyHostToDevice, b->st);
+    }
+    rc = e ? cuda_fail(e, "batch stretch")
+           : batch_set(p, v.data(), rem.data(), m, b->forced, b->max_clusters, false, nullptr);
+    if (!rc) rc = batch_enqueue(p, false);
+    int first = LBDD_OK;
+    if (!rc) rc = batch_wait(p, &first);
+    std::vector<lbdd_solver*> v2;
+    std::vector<int64_t> target2;
+    bool moved = false;
+    for (int i = 0; i < m && !rc; ++i) {
+      const int64_t* out = p->h_out + kOut * p->slot_of[i];
+      moved |= out[0] != 0 || out[1] > from[i] || out[2] != 0;
+      if (out[0] == 0 && out[1] < target[i]) {
+        v2.push_back(v[i]);
+        target2.push_back(target[i]);
+      }
+    }
+    batch_free(p);
+    if (rc) return rc;
+    if (first && first_rc && *first_rc == LBDD_OK) *first_rc = first;
+    if (!moved) return LBDD_ERR_STATE;   // (cannot happen: a pass runs rounds or ends a stretch)
+    v.swap(v2);
+    target.swap(target2);
+  }
+  return LBDD_OK;
 }
 
 }  // namespace lbdd
@@ -550,6 +622,7 @@ extern "C" int lbdd_batch_run(lbdd_batch* b, int64_t max_rounds) {
   int first = LBDD_OK;
   int rc = batch_launch(b, max_rounds);
   if (!rc) rc = batch_wait(b, &first);
+  if (!rc) rc = batch_finish(b, &first);
   return rc ? rc : first;
 }
 
@@ -580,6 +653,7 @@ extern "C" int lbdd_solve_batch(lbdd_solver* const* solvers, int m, int64_t max_
   int first = LBDD_OK;
   if (!rc) rc = batch_launch(b, max_rounds);
   if (!rc) rc = batch_wait(b, &first);
+  if (!rc) rc = batch_finish(b, &first);
   batch_free(b);
   return rc ? rc : first;
 }

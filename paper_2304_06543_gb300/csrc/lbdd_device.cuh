@@ -56,6 +56,9 @@ enum CtlIndex {
   CTL_POT = CTL_FRONT_HIST + 6,  // 1: the prices hold for the current table (guided rounds)
   CTL_MIRROR,          // 1: the global mirror of T's costs is current (guided rounds)
   CTL_GUIDED,          // rounds that ran guided
+  CTL_LEVEL,           // member scans of guided rounds beyond their limits (heavy_scans),
+  CTL_LEVEL_WIDE,      // of all rows and of rows with most entries affected
+  CTL_HEAVY,           // 1: guided rounds ended early because that level is past its limit
   CTL_COUNT
 };
 
@@ -75,6 +78,7 @@ enum : int {
   OPT_STRICT = 32,        // strict-LBDD (Alg. 5): vacancies as zero-cost dummy units
   OPT_GUIDED = 64,        // the price-guided rounds: CTA 0 runs them (set by the host)
   OPT_PROLOGUE = 128,     // guided launch that runs no rounds, only due prologues (host)
+  OPT_NO_EXIT = 256,      // guided rounds do not end early, however many members they scan
 };
 
 // Whether a prologue is worth a launch of its own on a larger cluster (about

@@ -63,6 +63,10 @@ struct lbdd_solver {
   int32_t max_cost = 0;    // largest cost at creation
   int32_t max_pen = 0;     // largest penalty (guided rounds need it below guided_pen_limit())
   bool fresh = true;       // no round has run: the next ones begin with the prologue
+  // Rounds that scan too many members for one SM (heavy_scans) run on the full
+  // Bellman-Ford kernel: until this round, in stretches that double each time.
+  int64_t round = 0;       // rounds done, as the host last saw it
+  int64_t full_until = 0, stretch = 0;
   int in_batches = 0;      // batches that hold a copy of this solver's device view
   int32_t* ins_row = nullptr;  // k costs of a unit being inserted (device staging)
   size_t bytes = 0;        // device bytes held now
@@ -85,6 +89,11 @@ int solver_flags(const lbdd_solver* s);
 // Whether s's next rounds on C-CTA clusters run guided (both shortcuts on,
 // penalties and the layout within the guided limits).
 bool solver_guided(const lbdd_solver* s, int C);
+// After guided rounds ended early at round `round`: the next stretch.
+void note_heavy(lbdd_solver* s, int64_t round);
+// Where the next launch of s has to stop on its way to round `target`; a
+// stretch that is over is forgotten (its level cleared on `st`).
+cudaError_t next_stop(lbdd_solver* s, int64_t target, cudaStream_t st, int64_t* stop);
 // Whether s runs on C-CTA clusters, guided or not.
 bool solver_fits(const lbdd_solver* s, int C);
 // A prologue ahead of rounds on smaller clusters: its cluster size, and whether
