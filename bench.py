@@ -1120,9 +1120,9 @@ def run_scan(args):
                                f"instance, {inst.n} x {inst.k}", "n": inst.n, "k": inst.k},
         "roofline": res["i16"], "scan": res,
         "tables_equal_i16_i32": res["i16"]["table_sha256"] == res["i32"]["table_sha256"],
-        # per call: bt_own, bt_scan_stream16, bt_merge_ranges on the int16 row-order path,
+        # per call: bt_own, bt_scan_stream, bt_merge_ranges on the row-order path,
         # else bt_count, bt_plan, bt_place, bt_sort_items, the scan and bt_unpack
-        "gpu_launches": args.steps * ((3 if 256 <= inst.k <= 512 and inst.n <= 32 * 65536 else 6) + 6),
+        "gpu_launches": args.steps * 2 * (3 if 256 <= inst.k <= 512 and inst.n <= 32 * 65536 else 6),
         "clocks": clk,
     }
     print(json.dumps(line), flush=True)
